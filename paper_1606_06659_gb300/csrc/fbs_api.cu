@@ -962,17 +962,14 @@ int fbs_beta_ess(fbs_handle* h, double* ess) {
   if (hy.trace_rows < 4) return fail(FBS_E_ARG, "the beta trace holds fewer than 4 rows");
   const int L = h->mc.L, G = h->mc.G;
   const long long S = (long long)L * G;
-  double* d_ess = nullptr;
-  FBS_CUDA(cudaMallocAsync((void**)&d_ess, (size_t)S * 8, h->s));
-  cudaError_t e = launch_ess(h->p.trace_beta, hy.trace_rows, S, d_ess, h->s);
-  std::vector<double> tmp((size_t)S);
+  double* d_ess = nullptr;  // the results, then the launch's scratch
+  FBS_CUDA(cudaMallocAsync((void**)&d_ess, 2 * (size_t)S * 8, h->s));
+  cudaError_t e = launch_ess(h->p.trace_beta, hy.trace_rows, L, G, d_ess + S, d_ess, h->s);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(tmp.data(), d_ess, (size_t)S * 8, cudaMemcpyDeviceToHost, h->s);
+    e = cudaMemcpyAsync(ess, d_ess, (size_t)S * 8, cudaMemcpyDeviceToHost, h->s);
   cudaFreeAsync(d_ess, h->s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->s);
   FBS_CUDA(e);
-  for (int l = 0; l < L; ++l)
-    for (int g = 0; g < G; ++g) ess[(size_t)g * L + l] = tmp[(size_t)l * G + g];
   return leave(h);
 }
 

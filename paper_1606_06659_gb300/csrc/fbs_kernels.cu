@@ -1,6 +1,5 @@
 // fbs_kernels.cu -- CUDA kernels of one Gibbs sweep (Algorithm 1 of Landau &
-// Niemi, arXiv 1606.06659) for sm_103a, plus initialisation, trace and ESS
-// kernels.
+// Niemi, arXiv 1606.06659) for sm_103a, plus initialisation and trace kernels.
 //
 // A sweep is two launches:
 //   gene kernel   one thread per gene g: slice updates of eps_g1..eps_gN
@@ -931,7 +930,7 @@ __global__ void k_init_hyper(ModelConst mc, Hyper* hy, const double* beta_d,
   }
 }
 
-// ---------------------------------------------------------------- uniforms, ESS
+// ---------------------------------------------------------------- uniforms
 
 __global__ void k_uniforms(uint32_t seed_lo, uint32_t seed_hi, uint32_t chain, uint32_t stream,
                            uint32_t index0, int n_index, uint32_t iter, uint32_t k0, int n_k,
@@ -940,44 +939,6 @@ __global__ void k_uniforms(uint32_t seed_lo, uint32_t seed_hi, uint32_t chain, u
   if (i >= n_index) return;
   Rng r(seed_lo, seed_hi, chain, stream, index0 + (uint32_t)i, iter);
   for (int k = 0; k < n_k; ++k) out[(size_t)i * n_k + k] = r.u(k0 + (uint32_t)k);
-}
-
-// Geyer initial-monotone-sequence ESS of every column of a [rows][S] trace:
-// one thread per series, reading row by row (consecutive series are adjacent).
-__global__ void k_ess(const double* __restrict__ tr, long long rows, long long S, double* ess) {
-  const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= S) return;
-  const long long n = rows;
-  double mean = 0.0;
-  for (long long t = 0; t < n; ++t) mean += tr[t * S + s];
-  mean /= (double)n;
-  double c0 = 0.0;
-  for (long long t = 0; t < n; ++t) {
-    const double dv = tr[t * S + s] - mean;
-    c0 += dv * dv;
-  }
-  c0 /= (double)n;
-  if (!(c0 > 0.0)) {
-    ess[s] = (double)n;
-    return;
-  }
-  double sum = 0.0, prev = INFINITY;
-  for (long long j = 0; 2 * j + 1 < n; ++j) {
-    double pair = 0.0;
-    for (long long k = 2 * j; k <= 2 * j + 1; ++k) {
-      double ck = 0.0;
-      for (long long t = 0; t + k < n; ++t)
-        ck += (tr[t * S + s] - mean) * (tr[(t + k) * S + s] - mean);
-      pair += ck / (double)n / c0;
-    }
-    if (!(pair > 0.0)) break;
-    if (pair > prev) pair = prev;
-    sum += pair;
-    prev = pair;
-  }
-  double tau = -1.0 + 2.0 * sum;
-  if (tau < 1.0 / (double)n) tau = 1.0 / (double)n;
-  ess[s] = (double)n / tau;
 }
 
 // ---------------------------------------------------------------- launchers
@@ -1080,13 +1041,6 @@ cudaError_t launch_uniforms(uint64_t seed, uint32_t chain, uint32_t stream, uint
   k_uniforms<<<(n_index + blk - 1) / blk, blk, 0, s>>>((uint32_t)seed, (uint32_t)(seed >> 32),
                                                         chain, stream, index0, n_index, iter, k0,
                                                         n_k, out);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_ess(const double* tr, long long rows, long long S, double* ess,
-                       cudaStream_t s) {
-  const int blk = 128;
-  k_ess<<<(unsigned)((S + blk - 1) / blk), blk, 0, s>>>(tr, rows, S, ess);
   return cudaGetLastError();
 }
 

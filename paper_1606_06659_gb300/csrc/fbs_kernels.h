@@ -1,5 +1,4 @@
-// fbs_kernels.h -- host-side launchers of the sweep, set-up, uniform and ESS
-// kernels (fbs_kernels.cu).
+// fbs_kernels.h -- host-side launchers of the kernels.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -129,7 +128,9 @@ cudaError_t launch_uniforms(uint64_t seed, uint32_t chain, uint32_t stream, uint
 // Sets the message fbs_last_error_string() returns on the calling thread.
 void set_last_error(const std::string& msg);
 
-cudaError_t launch_ess(const double* tr, long long rows, long long S, double* ess,
+// Effective sample sizes of the series of a [rows][L][G] trace (fbs_ess.cu):
+// ess [G][L]; mean: L * G doubles of scratch.
+cudaError_t launch_ess(const double* tr, long long rows, int L, int G, double* mean, double* ess,
                        cudaStream_t s);
 
 }  // namespace fbs
