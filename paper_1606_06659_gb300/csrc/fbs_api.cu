@@ -38,6 +38,10 @@ int fail(int code, const std::string& msg) {
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
+// Results of up to kPackMost bytes are read back in one copy if the staging area
+// holds them (see read_arrays); it has kPackBytes at least.
+constexpr size_t kPackBytes = 256 << 10, kPackMost = 1 << 20;
+
 // Byte offsets of every device buffer inside one workspace.
 struct Layout {
   size_t y, T, eps, w_eps, waux_eps, m_eps, q_eps, mu, beta, w_beta, waux_beta, m_beta, q_beta;
@@ -61,7 +65,7 @@ Layout make_layout(int N, int G, int L, int nblk, long long trace_cap, int trace
   o.waux_eps = take(NG * 8);
   o.m_eps = take(NG * 8);
   o.q_eps = take(NG * 8);
-  o.mu = take(NG * 8);
+  o.mu = take(std::max(NG * 8, kPackBytes));  // also the staging area of read_arrays
   o.beta = take(LG * 8);
   o.w_beta = take(LG * 8);
   o.waux_beta = take(LG * 8);
@@ -74,9 +78,10 @@ Layout make_layout(int N, int G, int L, int nblk, long long trace_cap, int trace
   o.q_gam = take((size_t)G * 8);
   o.partial = take((size_t)nblk * kNumPart * 8);
   o.hyp = take(sizeof(Hyper));
+  // right behind the Hyper block, so that one copy reads both (read_status)
+  o.counters = take(kCounterCopies * FBS_NUM_COUNTERS * sizeof(unsigned long long));
   o.trace_phi = take((size_t)(trace_cap > 0 ? trace_cap : 1) * P * 8);
   o.trace_beta = trace_beta && trace_cap > 0 ? take((size_t)trace_cap * LG * 8) : 0;
-  o.counters = take(kCounterCopies * FBS_NUM_COUNTERS * sizeof(unsigned long long));
   o.pinv = take((size_t)kMaxL * kMaxN * 8);
   o.total = at + 256;  // slack for aligning an unaligned base
   return o;
@@ -103,7 +108,7 @@ LayoutF32 make_layout_f32(int N, int G, int L, int nblk, long long trace_cap, in
   o.w_eps = take(NG * 4);
   o.waux_eps = take(NG * 4);
   o.mom_eps = take(4 * NG * 4);
-  o.mu = take(NG * 4);
+  o.mu = take(std::max(NG * 4, kPackBytes));  // also the staging area of read_arrays
   o.beta = take(LG * 4);
   o.w_beta = take(LG * 4);
   o.waux_beta = take(LG * 4);
@@ -112,9 +117,9 @@ LayoutF32 make_layout_f32(int N, int G, int L, int nblk, long long trace_cap, in
   o.mom_gam = take(4 * (size_t)G * 4);
   o.partial = take((size_t)nblk * kNumPart * 8);
   o.hyp = take(sizeof(Hyper));
+  o.counters = take(kCounterCopies * FBS_NUM_COUNTERS * sizeof(unsigned long long));  // (read_status)
   o.trace_phi = take((size_t)(trace_cap > 0 ? trace_cap : 1) * P * 8);
   o.trace_beta = trace_beta && trace_cap > 0 ? take((size_t)trace_cap * LG * 8) : 0;
-  o.counters = take(kEpsCounterCopiesHost * FBS_NUM_COUNTERS * sizeof(unsigned long long));
   o.pinv = take((size_t)kMaxL * kMaxN * 8);
   o.gsync = take(kPersistentSyncBytes);
   o.total = at + 256;
@@ -179,6 +184,9 @@ struct fbs_handle {
   unsigned* con_count = nullptr;   // device counts [FBS_MAX_CONTRASTS][G]
   int ncon = 0;
   long long con_nmom0 = 0;         // moment count when the propositions were set
+  char* stage = nullptr;           // device staging of what is read back: the rates' plane,
+  size_t stage_cap = 0;            // which holds nothing between sweeps
+  std::vector<char> stage_host;    // up to kPackMost
 };
 
 namespace {
@@ -330,15 +338,95 @@ void carve_f32(char* base, const LayoutF32& o32, int trace_beta, DevPtrsF32& f, 
   p.counters = f.counters;
 }
 
-// Copy a device [R][G] plane set (double or float) to a host [G][R] double array.
-template <class T>
-int to_host_gene_major(fbs_handle* h, const T* dev, int R, double* host) {
-  const int G = h->mc.G;
-  std::vector<T> tmp((size_t)R * G);
-  FBS_CUDA(cudaMemcpyAsync(tmp.data(), dev, tmp.size() * sizeof(T), cudaMemcpyDeviceToHost, h->s));
+int read_hyper(fbs_handle* h, Hyper* out) {
+  FBS_CUDA(cudaMemcpyAsync(out, h->p.hyp, sizeof(Hyper), cudaMemcpyDeviceToHost, h->s));
   FBS_CUDA(cudaStreamSynchronize(h->s));
-  for (int r = 0; r < R; ++r)
-    for (int g = 0; g < G; ++g) host[(size_t)g * R + r] = (double)tmp[(size_t)r * G + g];
+  return FBS_OK;
+}
+
+// What is read back goes through a staging area on the device, where kernels
+// convert it to FP64 and transpose it to the gene-major order of the caller's
+// arrays.  The area is the plane of the rates mu, which the eps kernel hands to
+// the gamma/beta kernel of the same sweep and which holds nothing between
+// sweeps, so reading allocates nothing.  Up to kPackMost a call's arrays come
+// back in one copy and are handed out on the host (a copy to pageable memory
+// costs about 20 us of latency); larger ones are copied straight to the caller's
+// arrays, the genes in as many pieces as the area needs.
+
+// Hands out the host copy of a packed stage.
+struct StageOut {
+  double* host;
+  size_t off, bytes;
+};
+
+int stage_fetch(fbs_handle* h, size_t bytes, const std::vector<StageOut>& outs) {
+  h->stage_host.resize(bytes);
+  FBS_CUDA(cudaMemcpyAsync(h->stage_host.data(), h->stage, bytes, cudaMemcpyDeviceToHost, h->s));
+  FBS_CUDA(cudaStreamSynchronize(h->s));
+  for (const StageOut& o : outs) memcpy(o.host, h->stage_host.data() + o.off, o.bytes);
+  return FBS_OK;
+}
+
+// Device planes [R][G] to a host array [G][R] of doubles (host null: skipped).
+struct ReadJob {
+  const void* src;
+  GatherKind kind;
+  int R;
+  double* host;
+};
+
+template <class T>
+ReadJob planes(const T* src, int R, double* host) {
+  return ReadJob{src, sizeof(T) == 8 ? GatherKind::f64 : GatherKind::f32, R, host};
+}
+// A Kahan-compensated FP32 moment: the planes of the value m, then those of the
+// compensation c; the moment is m - c.
+ReadJob kahan(const float* src, int R, double* host) {
+  return ReadJob{src, GatherKind::kahan, R, host};
+}
+
+// Reads the jobs' arrays and the Hyper block (synchronous).
+int read_arrays(fbs_handle* h, const std::vector<ReadJob>& all, Hyper* hy) {
+  const size_t G = (size_t)h->mc.G;
+  GatherArgs a;
+  a.n = 0;
+  a.G = h->mc.G;
+  size_t total = sizeof(Hyper);
+  for (const ReadJob& j : all)
+    if (j.host) total += (size_t)j.R * G * 8;
+  static_assert(sizeof(Hyper) % 8 == 0, "the Hyper block is gathered as 8-byte words");
+  auto put = [&](const ReadJob& j, size_t g0, size_t ng, size_t off) {
+    a.job[a.n++] = GatherJob{j.src, j.kind, j.R, (long long)g0, (long long)ng, (long long)(off / 8)};
+  };
+  if (total == sizeof(Hyper)) return read_hyper(h, hy);  // no array is wanted
+  if (total <= std::min(kPackMost, h->stage_cap)) {
+    std::vector<StageOut> outs;
+    size_t off = 0;
+    for (const ReadJob& j : all) {
+      if (!j.host) continue;
+      put(j, 0, G, off);
+      outs.push_back(StageOut{j.host, off, (size_t)j.R * G * 8});
+      off += (size_t)j.R * G * 8;
+    }
+    a.job[a.n++] = GatherJob{h->p.hyp, GatherKind::f64, 1, 0, (long long)(sizeof(Hyper) / 8),
+                             (long long)(off / 8)};
+    outs.push_back(StageOut{reinterpret_cast<double*>(hy), off, sizeof(Hyper)});
+    FBS_CUDA(launch_gather(a, (double*)h->stage, h->s));
+    return stage_fetch(h, total, outs);
+  }
+  for (const ReadJob& j : all) {
+    if (!j.host) continue;
+    const size_t row = (size_t)j.R * 8, chunk = h->stage_cap / row;
+    for (size_t g0 = 0; g0 < G; g0 += chunk) {
+      const size_t ng = std::min(chunk, G - g0);
+      a.n = 0;
+      put(j, g0, ng, 0);
+      FBS_CUDA(launch_gather(a, (double*)h->stage, h->s));
+      FBS_CUDA(cudaMemcpyAsync(j.host + g0 * j.R, h->stage, ng * row, cudaMemcpyDeviceToHost, h->s));
+    }
+  }
+  FBS_CUDA(cudaMemcpyAsync(hy, h->p.hyp, sizeof(Hyper), cudaMemcpyDeviceToHost, h->s));
+  FBS_CUDA(cudaStreamSynchronize(h->s));
   return FBS_OK;
 }
 
@@ -353,24 +441,24 @@ int from_host_gene_major(fbs_handle* h, T* dev, int R, const double* host) {
   return FBS_OK;
 }
 
-// A Kahan-compensated FP32 moment: planes value m and compensation c of
-// [R][G] each, starting at `base + plane_offset`; the moment is m - c.
-int kahan_to_host(fbs_handle* h, const float* base, int R, double* host) {
-  const int G = h->mc.G;
-  const size_t n = (size_t)R * G;
-  std::vector<float> tmp(2 * n);
-  FBS_CUDA(cudaMemcpyAsync(tmp.data(), base, 2 * n * 4, cudaMemcpyDeviceToHost, h->s));
+// The Hyper block and the counters summed over their copies, in one copy
+// (synchronous).
+int read_status(fbs_handle* h, Hyper* hy, int64_t* out) {
+  const size_t at = (const char*)h->p.counters - (const char*)h->p.hyp;
+  char buf[2048 + kCounterCopies * FBS_NUM_COUNTERS * 8];
+  const size_t bytes = at + kCounterCopies * FBS_NUM_COUNTERS * sizeof(unsigned long long);
+  static_assert(sizeof(Hyper) <= 2048 - 256, "the counters follow at the next 256 bytes");
+  FBS_CUDA(cudaMemcpyAsync(buf, h->p.hyp, bytes, cudaMemcpyDeviceToHost, h->s));
   FBS_CUDA(cudaStreamSynchronize(h->s));
-  for (int r = 0; r < R; ++r)
-    for (int g = 0; g < G; ++g)
-      host[(size_t)g * R + r] =
-          (double)tmp[(size_t)r * G + g] - (double)tmp[n + (size_t)r * G + g];
-  return FBS_OK;
-}
-
-int read_hyper(fbs_handle* h, Hyper* out) {
-  FBS_CUDA(cudaMemcpyAsync(out, h->p.hyp, sizeof(Hyper), cudaMemcpyDeviceToHost, h->s));
-  FBS_CUDA(cudaStreamSynchronize(h->s));
+  memcpy(hy, buf, sizeof(Hyper));
+  for (int i = 0; i < FBS_NUM_COUNTERS; ++i) {
+    unsigned long long t = 0, v;
+    for (int k = 0; k < kCounterCopies; ++k) {
+      memcpy(&v, buf + at + ((size_t)k * FBS_NUM_COUNTERS + i) * sizeof(v), sizeof(v));
+      t += v;
+    }
+    out[i] = (int64_t)t;
+  }
   return FBS_OK;
 }
 
@@ -657,10 +745,14 @@ int fbs_init(fbs_handle** out, const int32_t* y, int N, int G, int gene_major, c
     const LayoutF32& o32 = h->lay32;
     y_raw = (int32_t*)f.mom_eps;
     d_pinv = (double*)(base + o32.pinv);
+    h->stage = (char*)f.mu;
+    h->stage_cap = std::max((size_t)N * G * 4, kPackBytes);
     if ((e = prepare_gene_kernel_f32(N, h->block)) != cudaSuccess)
       return bail(FBS_E_CUDA, std::string("kernel attribute: ") + cudaGetErrorString(e));
   } else {
     h->p = carve(base, h->lay, mc.trace_beta);
+    h->stage = (char*)h->p.mu;
+    h->stage_cap = std::max((size_t)N * G * 8, kPackBytes);
     y_raw = (int32_t*)h->p.q_eps;
     d_pinv = (double*)(base + h->lay.pinv);
     if ((e = prepare_gene_kernel(N, h->block)) != cudaSuccess)
@@ -699,27 +791,9 @@ int fbs_init(fbs_handle** out, const int32_t* y, int N, int G, int gene_major, c
 
 namespace {
 
-// The handle's counters summed over their copies (synchronous).
-int sum_counters(fbs_handle* h, int64_t* out) {
-  const int copies = kCounterCopies;
-  std::vector<unsigned long long> c((size_t)copies * FBS_NUM_COUNTERS);
-  FBS_CUDA(cudaMemcpyAsync(c.data(), h->p.counters, c.size() * sizeof(unsigned long long),
-                           cudaMemcpyDeviceToHost, h->s));
-  FBS_CUDA(cudaStreamSynchronize(h->s));
-  for (int i = 0; i < FBS_NUM_COUNTERS; ++i) {
-    unsigned long long t = 0;
-    for (int k = 0; k < copies; ++k) t += c[(size_t)k * FBS_NUM_COUNTERS + i];
-    out[i] = (int64_t)t;
-  }
-  return FBS_OK;
-}
-
 // FBS_E_SLICE_CAP once any slice update of the handle has used up its shrinkage
 // proposals (Algorithm 2 has no bound; the update kept its value).
-int slice_cap_status(fbs_handle* h) {
-  int64_t c[FBS_NUM_COUNTERS];
-  int rc = sum_counters(h, c);
-  if (rc) return rc;
+int slice_cap_status(const int64_t* c) {
   if (c[FBS_CNT_SLICE_CAPS] > 0)
     return fail(FBS_E_SLICE_CAP, std::to_string(c[FBS_CNT_SLICE_CAPS]) +
                                      " slice update(s) ran out of shrinkage proposals and kept "
@@ -770,14 +844,15 @@ int fbs_sync(fbs_handle* h) {
   FBS_CUDA(cudaStreamSynchronize(h->s));
   FBS_CUDA(cudaGetLastError());
   Hyper hy;
-  int rc = read_hyper(h, &hy);
+  int64_t cnt[FBS_NUM_COUNTERS];
+  int rc = read_status(h, &hy, cnt);
   if (rc) return rc;
   if (hy.flags & kFlagTimeout)
     return fail(FBS_E_CUDA, "a bounded wait gave up (a tensor-core wait of the proposal network "
                             "or a grid barrier of the persistent sweep)");
   if (hy.flags & kFlagNonfinite)
     return fail(FBS_E_NONFINITE, "a slice update started from a non-finite log density");
-  return slice_cap_status(h);
+  return slice_cap_status(cnt);
 }
 
 int fbs_moments(fbs_handle* h, double* mean_eps, double* msq_eps, double* mean_beta,
@@ -787,25 +862,24 @@ int fbs_moments(fbs_handle* h, double* mean_eps, double* msq_eps, double* mean_b
   int rc = enter(h);
   if (rc) return rc;
   const int N = h->mc.N, L = h->mc.L, G = h->mc.G, P = h->mc.P;
+  Hyper hy;
   if (h->prec == FBS_F32) {
     const size_t NG = (size_t)N * G, LG = (size_t)L * G;
     const DevPtrsF32& f = h->pf;
-    if (mean_eps && (rc = kahan_to_host(h, f.mom_eps, N, mean_eps))) return rc;
-    if (msq_eps && (rc = kahan_to_host(h, f.mom_eps + 2 * NG, N, msq_eps))) return rc;
-    if (mean_beta && (rc = kahan_to_host(h, f.mom_beta, L, mean_beta))) return rc;
-    if (msq_beta && (rc = kahan_to_host(h, f.mom_beta + 2 * LG, L, msq_beta))) return rc;
-    if (mean_gam && (rc = kahan_to_host(h, f.mom_gam, 1, mean_gam))) return rc;
-    if (msq_gam && (rc = kahan_to_host(h, f.mom_gam + 2 * (size_t)G, 1, msq_gam))) return rc;
+    rc = read_arrays(h,
+                     {kahan(f.mom_eps, N, mean_eps), kahan(f.mom_eps + 2 * NG, N, msq_eps),
+                      kahan(f.mom_beta, L, mean_beta), kahan(f.mom_beta + 2 * LG, L, msq_beta),
+                      kahan(f.mom_gam, 1, mean_gam), kahan(f.mom_gam + 2 * (size_t)G, 1, msq_gam)},
+                     &hy);
   } else {
-    if (mean_eps && (rc = to_host_gene_major(h, h->p.m_eps, N, mean_eps))) return rc;
-    if (msq_eps && (rc = to_host_gene_major(h, h->p.q_eps, N, msq_eps))) return rc;
-    if (mean_beta && (rc = to_host_gene_major(h, h->p.m_beta, L, mean_beta))) return rc;
-    if (msq_beta && (rc = to_host_gene_major(h, h->p.q_beta, L, msq_beta))) return rc;
-    if (mean_gam) FBS_CUDA(cudaMemcpyAsync(mean_gam, h->p.m_gam, (size_t)G * 8, cudaMemcpyDeviceToHost, h->s));
-    if (msq_gam) FBS_CUDA(cudaMemcpyAsync(msq_gam, h->p.q_gam, (size_t)G * 8, cudaMemcpyDeviceToHost, h->s));
+    const DevPtrs& p = h->p;
+    rc = read_arrays(h,
+                     {planes(p.m_eps, N, mean_eps), planes(p.q_eps, N, msq_eps),
+                      planes(p.m_beta, L, mean_beta), planes(p.q_beta, L, msq_beta),
+                      planes(p.m_gam, 1, mean_gam), planes(p.q_gam, 1, msq_gam)},
+                     &hy);
   }
-  Hyper hy;
-  if ((rc = read_hyper(h, &hy))) return rc;
+  if (rc) return rc;
   if (mean_phi) memcpy(mean_phi, hy.m_phi, (size_t)P * 8);
   if (msq_phi) memcpy(msq_phi, hy.q_phi, (size_t)P * 8);
   if (count) *count = hy.n_mom;
@@ -818,27 +892,18 @@ int fbs_get_state(fbs_handle* h, double* eps, double* beta, double* gam, double*
   if (!h) return fail(FBS_E_ARG, "handle is NULL");
   int rc = enter(h);
   if (rc) return rc;
-  const int N = h->mc.N, L = h->mc.L, G = h->mc.G, P = h->mc.P;
-  if (h->prec == FBS_F32) {
-    const DevPtrsF32& f = h->pf;
-    if (eps && (rc = to_host_gene_major(h, (const float*)f.eps, N, eps))) return rc;
-    if (w_eps && (rc = to_host_gene_major(h, (const float*)f.w_eps, N, w_eps))) return rc;
-    if (waux_eps && (rc = to_host_gene_major(h, (const float*)f.waux_eps, N, waux_eps))) return rc;
-    if (beta && (rc = to_host_gene_major(h, (const float*)f.beta, L, beta))) return rc;
-    if (w_beta && (rc = to_host_gene_major(h, (const float*)f.w_beta, L, w_beta))) return rc;
-    if (waux_beta && (rc = to_host_gene_major(h, (const float*)f.waux_beta, L, waux_beta))) return rc;
-    if (gam && (rc = to_host_gene_major(h, (const float*)f.gam, 1, gam))) return rc;
-  } else {
-    if (eps && (rc = to_host_gene_major(h, (const double*)h->p.eps, N, eps))) return rc;
-    if (w_eps && (rc = to_host_gene_major(h, (const double*)h->p.w_eps, N, w_eps))) return rc;
-    if (waux_eps && (rc = to_host_gene_major(h, (const double*)h->p.waux_eps, N, waux_eps))) return rc;
-    if (beta && (rc = to_host_gene_major(h, (const double*)h->p.beta, L, beta))) return rc;
-    if (w_beta && (rc = to_host_gene_major(h, (const double*)h->p.w_beta, L, w_beta))) return rc;
-    if (waux_beta && (rc = to_host_gene_major(h, (const double*)h->p.waux_beta, L, waux_beta))) return rc;
-    if (gam) FBS_CUDA(cudaMemcpyAsync(gam, h->p.gam, (size_t)G * 8, cudaMemcpyDeviceToHost, h->s));
-  }
+  const int N = h->mc.N, L = h->mc.L, P = h->mc.P;
   Hyper hy;
-  if ((rc = read_hyper(h, &hy))) return rc;
+  auto read = [&](const auto& p) {
+    return read_arrays(h,
+                       {planes(p.eps, N, eps), planes(p.w_eps, N, w_eps),
+                        planes(p.waux_eps, N, waux_eps), planes(p.beta, L, beta),
+                        planes(p.w_beta, L, w_beta), planes(p.waux_beta, L, waux_beta),
+                        planes(p.gam, 1, gam)},
+                       &hy);
+  };
+  rc = h->prec == FBS_F32 ? read(h->pf) : read(h->p);
+  if (rc) return rc;
   if (phi) memcpy(phi, hy.phi, (size_t)P * 8);
   if (w_nu) *w_nu = hy.w_nu;
   if (waux_nu) *waux_nu = hy.waux_nu;
@@ -991,7 +1056,8 @@ int fbs_counters(fbs_handle* h, int64_t* out) {
   if (!h || !out) return fail(FBS_E_ARG, "handle or out is NULL");
   int rc = enter(h);
   if (rc) return rc;
-  if ((rc = sum_counters(h, out))) return rc;
+  Hyper hy;
+  if ((rc = read_status(h, &hy, out))) return rc;
   return leave(h);
 }
 
@@ -1479,30 +1545,103 @@ int fbs_proposal_stats(fbs_handle* h, int64_t* accepted, int64_t* tried, int* n_
                        int* n_prior_genes) {
   if (!h || !h->learned) return fail(FBS_E_ARG, "the handle has no learned proposal");
   LearnedState* ls = h->learned;
-  const int G = h->mc.G;
-  const size_t n2 = 2 * (size_t)G;
-  std::vector<unsigned> acc(n2), tr(n2);
-  std::vector<uint8_t> use(G);
+  unsigned long long c[4];
+  FBS_CUDA(launch_mh_stats(ls->mh_acc, ls->mh_try, ls->use_mh, h->mc.G,
+                           (unsigned long long*)h->stage, h->s));
+  FBS_CUDA(cudaMemcpyAsync(c, h->stage, sizeof(c), cudaMemcpyDeviceToHost, h->s));
   FBS_CUDA(cudaStreamSynchronize(h->s));
-  FBS_CUDA(cudaMemcpy(acc.data(), ls->mh_acc, sizeof(unsigned) * n2, cudaMemcpyDeviceToHost));
-  FBS_CUDA(cudaMemcpy(tr.data(), ls->mh_try, sizeof(unsigned) * n2, cudaMemcpyDeviceToHost));
-  FBS_CUDA(cudaMemcpy(use.data(), ls->use_mh, (size_t)G, cudaMemcpyDeviceToHost));
-  int64_t a = 0, t = 0;
-  int u = 0, up = 0;
-  for (size_t i = 0; i < n2; ++i) {
-    a += acc[i];
-    t += tr[i];
-  }
-  for (int g = 0; g < G; ++g) {
-    u += use[g] != 0;
-    up += use[g] == kMovePrior;
-  }
-  if (accepted) *accepted = a;
-  if (tried) *tried = t;
-  if (n_mh_genes) *n_mh_genes = u;
-  if (n_prior_genes) *n_prior_genes = up;
+  if (accepted) *accepted = (int64_t)c[0];
+  if (tried) *tried = (int64_t)c[1];
+  if (n_mh_genes) *n_mh_genes = (int)c[2];
+  if (n_prior_genes) *n_prior_genes = (int)c[3];
   return FBS_OK;
 }
+
+}  // extern "C"
+
+namespace {
+
+// Statistics of the pooled running moments of C chains (checked by the caller: the
+// same N, G, L and precision, M draws each) to host arrays in gene-major order:
+// launch(in, out, stream) writes dst.size() arrays of in.n values, one after the
+// other; a quantity whose destinations are all null is skipped.  Small results
+// come back in one copy, larger ones straight to the caller's arrays.
+template <class Launch>
+int pooled_read(int C, fbs_handle* const* chains, long long M, const std::vector<double*>& beta,
+                const std::vector<double*>& gam, const std::vector<double*>& eps,
+                const std::vector<double*>& phi, Launch launch) {
+  fbs_handle* h0 = chains[0];
+  const bool f32 = h0->prec == FBS_F32;
+  const size_t G = (size_t)h0->mc.G, k = phi.size();
+  struct Part {
+    int which, R;
+    size_t n;  // genes (values of phi)
+    const std::vector<double*>* dst;
+  };
+  std::vector<Part> parts;
+  size_t total = 0;
+  auto add = [&](int which, int R, size_t n, const std::vector<double*>& dst) {
+    for (double* d : dst)
+      if (d) {
+        parts.push_back(Part{which, R, n, &dst});
+        total += (size_t)R * n * k * 8;
+        return;
+      }
+  };
+  add(0, h0->mc.L, G, beta);
+  add(1, 1, G, gam);
+  add(2, h0->mc.N, G, eps);
+  add(3, 1, (size_t)h0->mc.P, phi);
+  const bool pack = total <= std::min(kPackMost, h0->stage_cap);
+  std::vector<StageOut> outs;
+  size_t off = 0;
+  for (const Part& q : parts) {
+    RhatInput in;
+    memset(&in, 0, sizeof(in));
+    in.C = C;
+    in.M = M;
+    in.R = q.R;
+    in.G = (long long)q.n;
+    in.f32 = f32 && q.which != 3;
+    for (int c = 0; c < C; ++c) {
+      const fbs_handle* h = chains[c];
+      if (q.which == 3) {  // phi: FP64 moments in the Hyper block of either form
+        in.m[c] = (const double*)((const char*)h->p.hyp + offsetof(Hyper, m_phi));
+        in.q[c] = (const double*)((const char*)h->p.hyp + offsetof(Hyper, q_phi));
+      } else if (f32) {
+        in.mf[c] = q.which == 0 ? h->pf.mom_beta : (q.which == 1 ? h->pf.mom_gam : h->pf.mom_eps);
+      } else {
+        in.m[c] = q.which == 0 ? h->p.m_beta : (q.which == 1 ? h->p.m_gam : h->p.m_eps);
+        in.q[c] = q.which == 0 ? h->p.q_beta : (q.which == 1 ? h->p.q_gam : h->p.q_eps);
+      }
+    }
+    const size_t row = (size_t)q.R * k * 8;
+    const size_t chunk = pack ? q.n : h0->stage_cap / row;
+    for (size_t g0 = 0; g0 < q.n; g0 += chunk) {
+      const size_t ng = std::min(chunk, q.n - g0), bytes = ng * q.R * 8;
+      in.g0 = (long long)g0;
+      in.n = (long long)(ng * q.R);
+      FBS_CUDA(launch(in, (double*)(h0->stage + off), h0->s));
+      for (size_t i = 0; i < k; ++i) {
+        double* host = (*q.dst)[i];
+        if (!host) continue;
+        if (pack)
+          outs.push_back(StageOut{host, off + i * bytes, bytes});
+        else
+          FBS_CUDA(cudaMemcpyAsync(host + g0 * q.R, h0->stage + i * bytes, bytes,
+                                   cudaMemcpyDeviceToHost, h0->s));
+      }
+      if (pack) off += bytes * k;
+    }
+  }
+  if (pack) return total ? stage_fetch(h0, total, outs) : FBS_OK;
+  FBS_CUDA(cudaStreamSynchronize(h0->s));
+  return FBS_OK;
+}
+
+}  // namespace
+
+extern "C" {
 
 int fbs_rhat(int C, fbs_handle* const* chains, double* rhat_phi, double* rhat_beta,
              double* rhat_gam, double* rhat_eps) {
@@ -1511,7 +1650,7 @@ int fbs_rhat(int C, fbs_handle* const* chains, double* rhat_phi, double* rhat_be
   for (int c = 0; c < C; ++c)
     if (!chains[c]) return fail(FBS_E_ARG, "a chain handle is NULL");
   const fbs_handle* h0 = chains[0];
-  const int N = h0->mc.N, G = h0->mc.G, L = h0->mc.L, P = h0->mc.P;
+  const int N = h0->mc.N, G = h0->mc.G, L = h0->mc.L;
   long long M = -1;
   for (int c = 0; c < C; ++c) {
     fbs_handle* h = chains[c];
@@ -1526,51 +1665,10 @@ int fbs_rhat(int C, fbs_handle* const* chains, double* rhat_phi, double* rhat_be
     if (hy.n_mom != M) return fail(FBS_E_ARG, "chains hold different numbers of draws");
   }
   if (M < 2) return fail(FBS_E_ARG, "need at least 2 post-burn-in draws per chain");
-  const bool f32 = h0->prec == FBS_F32;
-  const size_t NG = (size_t)N * G, LG = (size_t)L * G;
-  double* d_out = nullptr;
-  FBS_CUDA(cudaMalloc((void**)&d_out, sizeof(double) * std::max(NG, std::max(LG, (size_t)P))));
-  cudaStream_t s = h0->s;
-  auto run = [&](int which, long long n, double* host, int R) -> int {
-    RhatInput in;
-    memset(&in, 0, sizeof(in));
-    in.C = C;
-    in.M = M;
-    in.n = n;
-    in.f32 = f32 && which != 3;
-    for (int c = 0; c < C; ++c) {
-      const fbs_handle* h = chains[c];
-      if (which == 3) {  // phi: FP64 moments in the Hyper block of either form
-        in.m[c] = (const double*)((const char*)h->p.hyp + offsetof(Hyper, m_phi));
-        in.q[c] = (const double*)((const char*)h->p.hyp + offsetof(Hyper, q_phi));
-      } else if (f32) {
-        in.mf[c] = which == 0 ? h->pf.mom_beta : (which == 1 ? h->pf.mom_gam : h->pf.mom_eps);
-      } else {
-        in.m[c] = which == 0 ? h->p.m_beta : (which == 1 ? h->p.m_gam : h->p.m_eps);
-        in.q[c] = which == 0 ? h->p.q_beta : (which == 1 ? h->p.q_gam : h->p.q_eps);
-      }
-    }
-    cudaError_t e = launch_rhat(in, d_out, s);
-    std::vector<double> tmp((size_t)n);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(tmp.data(), d_out, sizeof(double) * n, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return fail(FBS_E_CUDA, std::string("rhat: ") + cudaGetErrorString(e));
-    if (which == 3) {
-      for (int k = 0; k < P; ++k) host[k] = tmp[k];
-    } else {
-      for (int r = 0; r < R; ++r)
-        for (int g = 0; g < G; ++g) host[(size_t)g * R + r] = tmp[(size_t)r * G + g];
-    }
-    return FBS_OK;
-  };
-  int rc = FBS_OK;
-  if (!rc && rhat_beta) rc = run(0, (long long)LG, rhat_beta, L);
-  if (!rc && rhat_gam) rc = run(1, (long long)G, rhat_gam, 1);
-  if (!rc && rhat_eps) rc = run(2, (long long)NG, rhat_eps, N);
-  if (!rc && rhat_phi) rc = run(3, (long long)P, rhat_phi, 1);
-  cudaFree(d_out);
-  return rc;
+  return pooled_read(C, chains, M, {rhat_beta}, {rhat_gam}, {rhat_eps}, {rhat_phi},
+                     [&](const RhatInput& in, double* out, cudaStream_t s) {
+                       return launch_rhat(in, out, s);
+                     });
 }
 
 int fbs_estimates_pooled(int C, fbs_handle* const* chains, fbs_estimates_out* out) {
@@ -1582,7 +1680,7 @@ int fbs_estimates_pooled(int C, fbs_handle* const* chains, fbs_estimates_out* ou
   for (int c = 0; c < C; ++c)
     if (!chains[c]) return fail(FBS_E_ARG, "a chain handle is NULL");
   fbs_handle* h0 = chains[0];
-  const int N = h0->mc.N, G = h0->mc.G, L = h0->mc.L, P = h0->mc.P;
+  const int N = h0->mc.N, G = h0->mc.G, L = h0->mc.L;
   const bool want_eps = out->mean_eps || out->sd_eps || out->lo_eps || out->hi_eps;
   long long M = -1;
   for (int k = 0; k < FBS_NUM_COUNTERS; ++k) out->counters[k] = 0;
@@ -1594,12 +1692,11 @@ int fbs_estimates_pooled(int C, fbs_handle* const* chains, fbs_estimates_out* ou
     if (want_eps && !h->mc.moments_eps) return fail(FBS_E_ARG, "a chain has no eps moments");
     FBS_CUDA(cudaStreamSynchronize(h->s));
     Hyper hy;
-    int rc = read_hyper(h, &hy);
+    int64_t cnt[FBS_NUM_COUNTERS];
+    int rc = read_status(h, &hy, cnt);
     if (rc) return rc;
     if (M < 0) M = hy.n_mom;
     if (hy.n_mom != M) return fail(FBS_E_ARG, "chains hold different numbers of draws");
-    int64_t cnt[FBS_NUM_COUNTERS];
-    if ((rc = sum_counters(h, cnt))) return rc;
     for (int k = 0; k < FBS_NUM_COUNTERS; ++k) out->counters[k] += cnt[k];
     if (h->learned) {
       int64_t a = 0, t = 0;
@@ -1610,57 +1707,14 @@ int fbs_estimates_pooled(int C, fbs_handle* const* chains, fbs_estimates_out* ou
   }
   if (M < 1) return fail(FBS_E_ARG, "the chains hold no post-burn-in draws");
   out->count = M;
-  const bool f32 = h0->prec == FBS_F32;
-  const size_t NG = (size_t)N * G, LG = (size_t)L * G;
-  const size_t nmax = std::max(NG, std::max(LG, (size_t)P));
-  double* d_out = nullptr;
-  FBS_CUDA(cudaMalloc((void**)&d_out, sizeof(double) * 4 * nmax));
-  cudaStream_t s = h0->s;
-  // which: 0 beta, 1 gamma, 2 eps, 3 phi; dst = mean, sd, lo, hi (each may be NULL)
-  auto run = [&](int which, long long n, int R, double* const* dst) -> int {
-    if (!dst[0] && !dst[1] && !dst[2] && !dst[3]) return FBS_OK;
-    RhatInput in;
-    memset(&in, 0, sizeof(in));
-    in.C = C;
-    in.M = M;
-    in.n = n;
-    in.f32 = f32 && which != 3;
-    for (int c = 0; c < C; ++c) {
-      const fbs_handle* h = chains[c];
-      if (which == 3) {  // phi: FP64 moments in the Hyper block of either form
-        in.m[c] = (const double*)((const char*)h->p.hyp + offsetof(Hyper, m_phi));
-        in.q[c] = (const double*)((const char*)h->p.hyp + offsetof(Hyper, q_phi));
-      } else if (f32) {
-        in.mf[c] = which == 0 ? h->pf.mom_beta : (which == 1 ? h->pf.mom_gam : h->pf.mom_eps);
-      } else {
-        in.m[c] = which == 0 ? h->p.m_beta : (which == 1 ? h->p.m_gam : h->p.m_eps);
-        in.q[c] = which == 0 ? h->p.q_beta : (which == 1 ? h->p.q_gam : h->p.q_eps);
-      }
-    }
-    cudaError_t e = launch_estimates(in, out->z, d_out, s);
-    std::vector<double> tmp(4 * (size_t)n);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(tmp.data(), d_out, sizeof(double) * 4 * n, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return fail(FBS_E_CUDA, std::string("estimates: ") + cudaGetErrorString(e));
-    for (int k = 0; k < 4; ++k) {
-      double* host = dst[k];
-      if (!host) continue;
-      const double* src = tmp.data() + (size_t)k * n;
-      for (int r = 0; r < R; ++r)
-        for (long long g = 0; g < n / R; ++g) host[(size_t)g * R + r] = src[(size_t)r * (n / R) + g];
-    }
-    return FBS_OK;
-  };
-  double* const beta_d[4] = {out->mean_beta, out->sd_beta, out->lo_beta, out->hi_beta};
-  double* const gam_d[4] = {out->mean_gam, out->sd_gam, out->lo_gam, out->hi_gam};
-  double* const eps_d[4] = {out->mean_eps, out->sd_eps, out->lo_eps, out->hi_eps};
-  double* const phi_d[4] = {out->mean_phi, out->sd_phi, out->lo_phi, out->hi_phi};
-  int rc = run(0, (long long)LG, L, beta_d);
-  if (!rc) rc = run(1, (long long)G, 1, gam_d);
-  if (!rc) rc = run(2, (long long)NG, N, eps_d);
-  if (!rc) rc = run(3, (long long)P, 1, phi_d);
-  cudaFree(d_out);
+  const double z = out->z;
+  int rc = pooled_read(C, chains, M, {out->mean_beta, out->sd_beta, out->lo_beta, out->hi_beta},
+                       {out->mean_gam, out->sd_gam, out->lo_gam, out->hi_gam},
+                       {out->mean_eps, out->sd_eps, out->lo_eps, out->hi_eps},
+                       {out->mean_phi, out->sd_phi, out->lo_phi, out->hi_phi},
+                       [&](const RhatInput& in, double* o, cudaStream_t s) {
+                         return launch_estimates(in, z, o, s);
+                       });
   if (rc) return rc;
   out->trace_rows = 0;
   if (out->trace_phi && out->trace_rows_max > 0)
@@ -2047,6 +2101,8 @@ int fbs_batch_init(fbs_batch** out, int C, const fbs_dataset* sets, const fbs_op
     v->s = b->s;
     carve_f32(base, lay[c], b->mcs[c].trace_beta, v->pf, v->p);
     b->pfs[c] = v->pf;
+    v->stage = (char*)v->pf.mu;
+    v->stage_cap = std::max((size_t)ds.N * ds.G * 4, kPackBytes);
     if ((e = cudaEventCreateWithFlags(&v->ev_in, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&v->ev_out, cudaEventDisableTiming)) != cudaSuccess)
       return bail(FBS_E_CUDA, cudaGetErrorString(e));
@@ -2124,15 +2180,16 @@ int fbs_batch_run(fbs_batch* b, int64_t n_iter, int64_t burnin, int64_t thin) {
 int fbs_batch_sync(fbs_batch* b) {
   if (!b) return fail(FBS_E_ARG, "batch is NULL");
   FBS_CUDA(cudaStreamSynchronize(b->s));
-  for (fbs_handle* v : b->views) {
+  std::vector<int64_t> cnt((size_t)b->C * FBS_NUM_COUNTERS);
+  for (int c = 0; c < b->C; ++c) {
     Hyper hy;
-    int rc = read_hyper(v, &hy);
+    int rc = read_status(b->views[c], &hy, cnt.data() + (size_t)c * FBS_NUM_COUNTERS);
     if (rc) return rc;
     if (hy.flags & kFlagNonfinite)
       return fail(FBS_E_NONFINITE, "a slice update started from a non-finite log density");
   }
-  for (fbs_handle* v : b->views) {
-    int rc = slice_cap_status(v);
+  for (int c = 0; c < b->C; ++c) {
+    int rc = slice_cap_status(cnt.data() + (size_t)c * FBS_NUM_COUNTERS);
     if (rc) return rc;
   }
   return FBS_OK;

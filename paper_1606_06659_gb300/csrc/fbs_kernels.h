@@ -48,18 +48,39 @@ cudaError_t launch_sweeps_f32(const ModelConst& mc, const DevPtrsF32& p, const D
 cudaError_t launch_mh_step_f32(const ModelConst& mc, const DevPtrsF32& p, long long it,
                               cudaStream_t s);
 
-// Gelman-Rubin factors of n parameters from C chains' moments (FP64 arrays, or
-// FP32 Kahan planes [4][n] when f32)
+// Device planes [R][G] converted to FP64 and transposed to [G][R] (the genes g0
+// .. g0 + ng - 1 of them), at doubles off.. of a staging buffer.
+enum class GatherKind : int { f64, f32, kahan };  // kahan: value planes, then compensation planes
+struct GatherJob {
+  const void* src;
+  GatherKind kind;
+  int R;
+  long long g0, ng, off;
+};
+constexpr int kMaxGather = 8;
+struct GatherArgs {
+  int n, G;
+  GatherJob job[kMaxGather];
+};
+cudaError_t launch_gather(const GatherArgs& a, double* out, cudaStream_t s);
+// Sums of the learned move's counts acc, tried [2][G] and numbers of genes with a
+// proposal and with the prior-centred one (use [G]): out [4].
+cudaError_t launch_mh_stats(const unsigned* acc, const unsigned* tried, const uint8_t* use, int G,
+                            unsigned long long* out, cudaStream_t s);
+
+// Statistics of parameters from C chains' moments (FP64 arrays [R][G], or FP32
+// Kahan planes [4][R][G] when f32): n of them, from gene g0 on in gene-major order.
 struct RhatInput {
-  int C, f32;
-  long long M, n;
+  int C, f32, R;
+  long long M, G, g0, n;
   const double* m[FBS_MAX_RHAT_CHAINS];
   const double* q[FBS_MAX_RHAT_CHAINS];
   const float* mf[FBS_MAX_RHAT_CHAINS];
 };
+// Gelman-Rubin factors: out [n].
 cudaError_t launch_rhat(const RhatInput& in, double* out, cudaStream_t s);
-// Pooled posterior mean, sd and the interval mean -/+ z sd of n parameters from
-// the same inputs as launch_rhat (C >= 1): out [4][n] = mean, sd, lo, hi.
+// Pooled posterior mean, sd and the interval mean -/+ z sd (C >= 1): out [4][n] =
+// mean, sd, lo, hi.
 cudaError_t launch_estimates(const RhatInput& in, double z, double* out, cudaStream_t s);
 
 // learned proposal (fbs_learned.cu)
@@ -117,7 +138,6 @@ cudaError_t launch_top_level(const ModelConst* mcs, const DevPtrsF32* ps, int C,
                              double* trace, cudaStream_t s);
 cudaError_t launch_set_run_batch(const DevPtrsF32* ps, int C, long long burnin,
                                  long long tune_start, long long thin, cudaStream_t s);
-constexpr int kEpsCounterCopiesHost = kCounterCopies;
 cudaError_t launch_init_f32(const ModelConst& mc, const DevPtrsF32& p, const int32_t* y_in,
                             int gene_major, const double* pinv, double w0, int set_state,
                             cudaStream_t s);
