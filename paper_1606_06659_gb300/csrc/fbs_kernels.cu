@@ -1,22 +1,24 @@
 // fbs_kernels.cu -- CUDA kernels of one Gibbs sweep (Algorithm 1 of Landau &
 // Niemi, arXiv 1606.06659) for sm_103a, plus initialisation and trace kernels.
 //
-// A sweep is two launches:
-//   gene kernel   one thread per gene g: slice updates of eps_g1..eps_gN
-//                 (Algorithm 1 step 1), the conjugate gamma_g draw (step 2), slice
-//                 updates of beta_g1..beta_gL in order (step 5), width tuning
-//                 (Algorithm 2 step 7), Welford moments (Section 3.1) and the
-//                 per-block FP64 partial sums that feed steps 3, 4, 6, 7;
+// A sweep is three launches:
+//   eps kernel    one thread per eps_gn: its slice update (Algorithm 1 step 1);
+//   gb kernel     one thread per gene g: the conjugate gamma_g draw (step 2), slice
+//                 updates of beta_g1..beta_gL in order (step 5), and the per-block
+//                 FP64 partial sums that feed steps 3, 4, 6, 7;
+//                 both with width tuning (Algorithm 2 step 7) and Welford moments
+//                 (Section 3.1);
 //   hyper kernel  one block: fixed-order reduction of the partials, then nu (slice,
 //                 step 3) and tau (step 4) on lane 0 while lanes 1..L draw
 //                 theta_l (step 6) and sigma_l^2 (step 7).
 // Drawing beta before nu and tau is exact: the beta_gl conditional involves
 // neither, and theirs involve no beta (Figure 3); the counter-based generator
 // gives every variable the same uniforms in either order.
-// With ModelConst::all_slice the gamma_g draw (gene kernel), tau (warp 0 of the
+// With ModelConst::all_slice the gamma_g draw (gb kernel), tau (warp 0 of the
 // hyper kernel, after nu) and sigma_l (lane 32+l) are slice updates of the same
 // full conditionals instead, each variable with its own tuned width, as
 // Section 4.2 slice-samples every non-normal conditional.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -28,51 +30,28 @@
 
 namespace fbs {
 
+namespace cg = cooperative_groups;
+
 // ---------------------------------------------------------------- densities
 
 // log f(eps_gn = x | ...) = y x - exp(A + x) - x^2 hg, with A = h_n + X_n beta_g and
 // hg = 1/(2 gamma_g).  aux = exp(A + x), the Poisson mean at x.
 struct EpsDensity {
-  double y, A, hg;
+  int32_t y;
+  double A, hg;
   __device__ __forceinline__ double operator()(double x, double* aux) const {
     const double e = exp(A + x);
     *aux = e;
-    return y * x - e - x * x * hg;
+    return (double)y * x - e - x * x * hg;
   }
 };
 
 // log f(beta_gl = b | ...) = b T_gl - sum_j Q_j exp(v_j (b - b0)) - (b - theta_l)^2 hs,
 // where Q_j sums exp(h_n + eps_gn + X_n beta_g) (current beta, beta_gl = b0) over
 // the samples n whose X_nl equals the j-th distinct non-zero value v_j of
-// column l.  Samples with X_nl = 0 only add a constant.  hs = 1/(2 sigma_l^2).
-struct BetaDensity {
-  double T, b0, theta, hs;
-  int ncls;
-  double Q[kMaxCls];
-  double v[kMaxCls];
-  int8_t kind[kMaxCls];
-  __device__ __forceinline__ double operator()(double b, double* aux) const {
-    const double dlt = b - b0;
-    const double z = exp(dlt);
-    double s = 0.0;
-#pragma unroll
-    for (int j = 0; j < kMaxCls; ++j) {
-      if (j < ncls) {
-        double e;
-        if (kind[j] == kClsPlus) e = z;
-        else if (kind[j] == kClsMinus) e = 1.0 / z;
-        else e = exp(v[j] * dlt);
-        s += Q[j] * e;
-      }
-    }
-    *aux = z;
-    const double dv = b - theta;
-    return b * T - s - dv * dv * hs;
-  }
-};
-
-// BetaDensity with the class count NC fixed at compile time (NC = kMaxCls keeps
-// the runtime bound `ncls`); the same arithmetic over the classes a column has.
+// column l.  Samples with X_nl = 0 only add a constant.  hs = 1/(2 sigma_l^2).  The
+// class count NC is fixed at compile time (NC = kMaxCls keeps the runtime bound
+// `ncls`).
 template <int NC>
 struct BetaDensityT {
   double T, b0, theta, hs;
@@ -101,68 +80,83 @@ struct BetaDensityT {
 };
 
 // FP32 filters of the FP64 slice updates (slice_update_filtered).  Each returns
-// Delta(p) = log f(p) - log f(x0) in the relative form of the FP32 sweep, which
+// Delta = log f(x0 + d) - log f(x0) in the relative form of the FP32 sweep, which
 // needs no evaluation at x0, and a bound on |Delta32 - Delta| + |the FP64
-// evaluation's error|.  FP32 part: 2^-20 (16 times the unit roundoff) times the
-// sum of the terms' magnitudes and of the sensitivities of Delta to the FP32
-// roundings of its inputs (x - x0, y or T, the rate mu0 from expf of the rounded
-// log-rate, Q_j, 1/(2 gamma) or 1/(2 sigma^2)) and to the series or expf of
-// e^z - 1 - z; FP64 part: 2^-46 (64 times the FP64 unit roundoff) times the
-// magnitudes of the terms of log f(p), log f(x0) and the level.
+// evaluation's error|, with e = 2^-24 the FP32 unit roundoff:
+//   - 2^-20 (16 e) times the magnitudes of the terms.  A term is a product of at
+//     most six rounded factors, the series for e^z - 1 - z below |z| = 1/2 is within
+//     8 e of itself, and the terms are added with two more roundings;
+//   - the FP32 inputs' roundings times the sensitivities of Delta to them, where
+//     these are not multiples of a term, with twice to four times the roundoff;
+//   - for |z| >= 1/2, where e^z - 1 - z is a difference of rounded numbers (expf is
+//     within 4 e of itself), 2^-21 (8 e) times their magnitudes;
+//   - derr, the error of d, times 5/4 of a bound on |Delta'| there (a derr that
+//     could change the exponential by more than a tenth is refused: infinite
+//     bound, the comparison is made in FP64);
+//   - 2^-46 (64 times the FP64 unit roundoff) times the magnitudes of the terms of
+//     log f(p), log f(x0) and the level.
+// What matters is that no part grows with the counts alone: near the decision the
+// terms are of order one whatever the count, while a bound of a fixed fraction of
+// the rate sent every evaluation of a gene with 10^5 counts to FP64 (0.35% of all
+// at N=16 G=40000, most warps had some).
 
-// eps: Delta(x) = d (y - mu0) - mu0 (e^d - 1 - d) - d (d + 2 x0) hg, d = x - x0.
+// eps: Delta = d (y - mu0) - mu0 (e^d - 1 - d) - d (d + 2 x0) hg.  mu0 carries the
+// rounding of the log-rate at x0 (|log-rate| e) and of expf: amag = |log-rate| + 8.
 struct EpsFilter {
-  double x0;
-  float y, mu0, x0f, hg, amag, c64;  // amag = |log-rate at x0| + 8; c64: log f(x0) magnitude
-  __device__ __forceinline__ float operator()(double pt, float* eb) const {
-    const float d = (float)(pt - x0);
-    const float ad = fabsf(d);
+  float y, mu0, x0f, hg, amag, c64;  // c64: log f(x0) magnitude
+  __device__ __forceinline__ float operator()(float d, float derr, float* eb) const {
+    const float ad = fabsf(d), ax = fabsf(x0f);
     const float e = em1mx(d);
     const float ed1 = d + e;             // e^d - 1
-    const float mued = mu0 + mu0 * ed1;  // mu0 e^d, the rate at pt
+    const float mued = mu0 + mu0 * ed1;  // mu0 e^d, the rate at the point
     const float t1 = d * (y - mu0);
     const float t2 = mu0 * e;
     const float t3 = d * (d + 2.0f * x0f) * hg;
-    const float b32 = fabsf(t1) + fabsf(t2) + fabsf(t3) +
-                      ad * (y + mu0 + mued + (2.0f * fabsf(x0f) + 2.0f * ad) * hg) +
-                      amag * mu0 * fabsf(ed1) + mu0 * (2.0f + fabsf(ed1) + ad);
-    const float px = fabsf(x0f) + ad;
+    const float b20 = fabsf(t1) + fabsf(t2) + ad * (ad + 2.0f * ax) * hg;
+    const float b22 = ad * y + amag * mu0 * fabsf(ed1);
+    const float slope = y + mued + 2.0f * (ad + ax) * hg;
+    const float px = ax + ad;
     const float b64 = c64 + y * px + mued * (amag + ad) + px * px * hg;
-    *eb = 0x1p-20f * b32 + 0x1p-46f * b64;
+    float b = 0x1p-20f * b20 + 0x1p-22f * b22 + 1.25f * derr * slope + 0x1p-46f * b64;
+    if (ad >= 0.5f) b += 0x1p-21f * mu0 * (2.0f + fabsf(ed1) + ad);
+    *eb = derr < 0.1f ? b : INFINITY;
     return t1 - t2 - t3;
   }
 };
 
-// beta_gl: Delta(b) = d T - sum_j Q_j (e^{v_j d} - 1) - d (d + 2 (b0 - theta)) hs.
+// beta_gl: Delta = d D - sum_j Q_j (e^{z_j} - 1 - z_j) - d (d + 2 (b0 - theta)) hs with
+// z_j = v_j d and D = T - sum_j v_j Q_j, taken in FP64 before the loop.
 template <int NC>
 struct BetaFilterT {
-  double b0;
-  float T, bt, hs, b0f, c64;  // bt = b0 - theta; c64: log f(b0) magnitude
+  float D, bt, hs, b0f, Tm, c64;  // bt = b0 - theta; Tm >= |T|; c64: log f(b0) magnitude
   int ncls;
   float Q[NC], v[NC];
-  __device__ __forceinline__ float operator()(double b, float* eb) const {
-    const float d = (float)(b - b0);
-    const float ad = fabsf(d);
-    float s = 0.0f, sa = 0.0f, sq = 0.0f, se = 0.0f;
+  __device__ __forceinline__ float operator()(float d, float derr, float* eb) const {
+    const float ad = fabsf(d), abt = fabsf(bt);
+    float s = 0.0f, sz = 0.0f, sl = 0.0f, se = 0.0f, sx = 0.0f, big = 0.0f;
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
       if (NC < kMaxCls || j < ncls) {
-        const float z = v[j] * d;
-        const float ej1 = z + em1mx(z);  // e^z - 1
-        const float q = Q[j] * ej1;
-        s += q;
-        sa += fabsf(q);
-        sq += Q[j] * ((fabsf(v[j]) * ad + 1.0f) * (2.0f + fabsf(ej1)) + fabsf(z));
-        se += Q[j] * (2.0f + fabsf(ej1));
+        const float z = v[j] * d, az = fabsf(z), av = fabsf(v[j]);
+        const float em = em1mx(z);
+        const float ej1 = fabsf(z + em);  // |e^z - 1|
+        const float vd = av * derr;
+        s += Q[j] * em;
+        sz += Q[j] * ej1 * az;
+        sl += Q[j] * av * (ej1 + 2.0f * vd * (1.0f + ej1));
+        se += Q[j] * (2.0f + ej1);
+        if (az >= 0.5f) sx += Q[j] * (2.0f + ej1 + az);
+        big = fmaxf(big, vd);
       }
     }
-    const float t1 = d * T;
+    const float t1 = d * D;
     const float t3 = d * (d + 2.0f * bt) * hs;
-    const float b32 = fabsf(t1) + sa + fabsf(t3) +
-                      ad * (fabsf(T) + (2.0f * fabsf(bt) + 2.0f * ad) * hs) + sq;
-    const float pb = fabsf(b0f) + ad, pt = fabsf(bt) + ad;
-    const float b64 = c64 + pb * fabsf(T) + se + pt * pt * hs;
-    *eb = 0x1p-20f * b32 + 0x1p-46f * b64;
+    const float b20 = fabsf(t1) + s + ad * (ad + 2.0f * abt) * hs;
+    const float slope = fabsf(D) + sl + 2.0f * (ad + abt) * hs;
+    const float pb = fabsf(b0f) + ad, pt = abt + ad;
+    const float b64 = c64 + pb * Tm + se + pt * pt * hs;
+    const float b = 0x1p-20f * b20 + 0x1p-21f * (sz + sx) + 1.25f * derr * slope + 0x1p-46f * b64;
+    *eb = big < 0.1f ? b : INFINITY;
     return t1 - s - t3;
   }
 };
@@ -176,6 +170,29 @@ struct GamDensity {
     *aux = 0.0;
     if (!(x > 0.0)) return -INFINITY;
     return -shape1 * log(x) - B / x;
+  }
+};
+
+// gamma_g: Delta = -s1 log(1 + r) + bx r / (1 + r) with r = d / x0 and bx = B / x0; a
+// point below zero (1 + r below zero by more than its error) is never inside the
+// slice, and one within a few errors of zero is left to FP64.
+struct GamFilter {
+  float s1, bx, ix, c64;  // ix = 1 / x0
+  __device__ __forceinline__ float operator()(float d, float derr, float* eb) const {
+    const float r = d * ix, q = 1.0f + r;
+    const float dr = fmaf(0x1p-22f, 1.0f + fabsf(r), derr * ix);  // error of r and of q
+    if (q < -2.0f * dr) {
+      *eb = 0.0f;
+      return -INFINITY;
+    }
+    const float iq = 1.0f / q;
+    const float lr = log1pf(r);
+    const float t1 = s1 * lr, t2 = bx * (r * iq);
+    const float slope = (s1 + bx * iq) * iq;
+    const float b = 0x1p-20f * (fabsf(t1) + fabsf(t2)) + 1.5f * dr * slope +
+                    0x1p-46f * (c64 + fabsf(t1) + bx * iq);
+    *eb = dr < 0.1f * q ? b : INFINITY;
+    return t2 - t1;
   }
 };
 
@@ -200,195 +217,13 @@ __device__ __forceinline__ void block_sum_to(double (&v)[NV], double* out, doubl
   }
 }
 
-// ---------------------------------------------------------------- gene kernel (FP64)
-
-__global__ void __launch_bounds__(128) k_gene_f64(ModelConst mc, DevPtrs p) {
-  extern __shared__ double smem_dyn[];  // mu[n][blockDim] then reduction scratch
-  const int G = mc.G, N = mc.N, L = mc.L;
-  const Hyper* hy = p.hyp;
-  const long long it = hy->it + 1;
-  const uint32_t it32 = (uint32_t)it;
-  const long long burnin = hy->burnin, tune_start = hy->tune_start;
-  const bool mom = it > burnin;
-  const double inv_k = mom ? 1.0 / (double)(hy->n_mom + 1) : 0.0;
-  const double nu = hy->phi[0], tau = hy->phi[1];
-  const bool trace_now = mom && mc.trace_beta && p.trace_beta != nullptr &&
-                         ((it - burnin) % hy->thin == 0) && hy->trace_rows < hy->trace_cap;
-  const long long trace_row = hy->trace_rows;
-
-  double* mu = smem_dyn;  // mu[n * blockDim + tid]
-  const int tid = threadIdx.x;
-  const int g = blockIdx.x * blockDim.x + tid;
-  const bool active = g < G;
-
-  double part[kNumPart];
-#pragma unroll
-  for (int i = 0; i < kNumPart; ++i) part[i] = 0.0;
-  unsigned evals_e = 0, evals_b = 0, caps = 0, gcaps = 0, nonfin = 0;
-
-  if (active) {
-    double beta[kMaxL];
-#pragma unroll
-    for (int l = 0; l < kMaxL; ++l) beta[l] = l < L ? p.beta[(size_t)l * G + g] : 0.0;
-    double gam = p.gam[g];
-    const double hg = 0.5 / gam;
-
-    // ---- step 1: eps_gn, n = 1..N
-    double ss = 0.0;
-    for (int n = 0; n < N; ++n) {
-      const size_t e = (size_t)n * G + g;
-      double A = mc.h[n];
-#pragma unroll
-      for (int l = 0; l < kMaxL; ++l)
-        if (l < L) A += mc.X[n * kMaxL + l] * beta[l];
-      EpsDensity f{(double)p.y[e], A, hg};
-      Rng r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamEps, (uint32_t)((size_t)g * N + n), it32);
-      const double x0 = p.eps[e];
-      double w = p.w_eps[e], waux = p.waux_eps[e];
-      SliceResult s = slice_update(x0, w, f, r, mc.K, mc.shrink_max);
-      evals_e += s.evals;
-      caps += s.capped;
-      nonfin += s.nonfinite;
-      mu[n * blockDim.x + tid] = s.aux;
-      p.eps[e] = s.x;
-      if (it <= burnin) {
-        tune_width(w, waux, it, s.x, x0, burnin, tune_start);
-        p.w_eps[e] = w;
-        p.waux_eps[e] = waux;
-      }
-      ss += s.x * s.x;
-      if (mom && mc.moments_eps) {
-        const double m = p.m_eps[e], q = p.q_eps[e];
-        p.m_eps[e] = m + (s.x - m) * inv_k;
-        p.q_eps[e] = q + (s.x * s.x - q) * inv_k;
-      }
-    }
-
-    // ---- step 2: gamma_g ~ IG((N + nu)/2, (sum eps^2 + nu tau)/2)
-    {
-      Rng r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamGamma, (uint32_t)g, it32);
-      bool gcap = false;
-      const double shape = 0.5 * ((double)N + nu);
-      const double scale = 0.5 * (ss + nu * tau);
-      gam = scale / gamma_mt(shape, r, 0, &gcap);
-      gcaps += gcap;
-      p.gam[g] = gam;
-      if (mom) {
-        const double m = p.m_gam[g], q = p.q_gam[g];
-        p.m_gam[g] = m + (gam - m) * inv_k;
-        p.q_gam[g] = q + (gam * gam - q) * inv_k;
-      }
-      part[0] = log(gam);
-      part[1] = 1.0 / gam;
-    }
-
-    // ---- step 5: beta_gl, l = 1..L in order
-    for (int l = 0; l < L; ++l) {
-      const size_t e = (size_t)l * G + g;
-      const double theta = hy->phi[2 + l];
-      const double sig2 = hy->phi[2 + L + l];
-      BetaDensity f;
-      f.T = p.T[e];
-      f.b0 = beta[l];
-      f.theta = theta;
-      f.hs = 0.5 / sig2;
-      f.ncls = mc.ncls[l];
-#pragma unroll
-      for (int j = 0; j < kMaxCls; ++j) {
-        f.Q[j] = 0.0;
-        f.v[j] = mc.cval[l][j];
-        f.kind[j] = mc.ckind[l][j];
-      }
-      for (int n = 0; n < N; ++n) {
-        const int c = mc.cls[l][n];
-        const double m = mu[n * blockDim.x + tid];
-#pragma unroll
-        for (int j = 0; j < kMaxCls; ++j)
-          if (j == c) f.Q[j] += m;
-      }
-      Rng r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamBeta, (uint32_t)((size_t)g * L + l), it32);
-      const double x0 = beta[l];
-      double w = p.w_beta[e], waux = p.waux_beta[e];
-      SliceResult s = slice_update(x0, w, f, r, mc.K, mc.shrink_max);
-      evals_b += s.evals;
-      caps += s.capped;
-      nonfin += s.nonfinite;
-      // carry exp(h_n + eps_gn + X_n beta_g) to the new beta_gl
-      if (s.x != x0) {
-        const double dlt = s.x - x0;
-        double ej[kMaxCls];
-        const double z = exp(dlt);
-#pragma unroll
-        for (int j = 0; j < kMaxCls; ++j) {
-          ej[j] = 1.0;
-          if (j < f.ncls) {
-            if (f.kind[j] == kClsPlus) ej[j] = z;
-            else if (f.kind[j] == kClsMinus) ej[j] = 1.0 / z;
-            else ej[j] = exp(f.v[j] * dlt);
-          }
-        }
-        for (int n = 0; n < N; ++n) {
-          const int c = mc.cls[l][n];
-          double fac = 1.0;
-#pragma unroll
-          for (int j = 0; j < kMaxCls; ++j)
-            if (j == c) fac = ej[j];
-          mu[n * blockDim.x + tid] *= fac;
-        }
-      }
-      beta[l] = s.x;
-      p.beta[e] = s.x;
-      if (it <= burnin) {
-        tune_width(w, waux, it, s.x, x0, burnin, tune_start);
-        p.w_beta[e] = w;
-        p.waux_beta[e] = waux;
-      }
-      if (mom) {
-        const double m = p.m_beta[e], q = p.q_beta[e];
-        p.m_beta[e] = m + (s.x - m) * inv_k;
-        p.q_beta[e] = q + (s.x * s.x - q) * inv_k;
-      }
-      if (trace_now) p.trace_beta[(size_t)trace_row * L * G + e] = s.x;
-      const double dv = s.x - theta;  // shifted by the current theta_l
-      part[2 + l] = dv;
-      part[2 + kMaxL + l] = dv * dv;
-    }
-  }
-
-  // ---- per-block partial sums for steps 3, 4, 6, 7
-  double* red = smem_dyn + (size_t)N * blockDim.x;
-  block_sum_to<kNumPart>(part, p.partial + (size_t)blockIdx.x * kNumPart, red);
-
-  // ---- counters
-  unsigned long long c4[4] = {evals_e, evals_b, caps, gcaps};
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    unsigned long long x = c4[i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    c4[i] = x;
-  }
-  unsigned nf = nonfin;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) nf += __shfl_down_sync(0xffffffffu, nf, o);
-  if ((tid & 31) == 0) {
-    if (c4[0]) atomicAdd(&p.counters[FBS_CNT_EVALS_EPS], c4[0]);
-    if (c4[1]) atomicAdd(&p.counters[FBS_CNT_EVALS_BETA], c4[1]);
-    if (c4[2]) atomicAdd(&p.counters[FBS_CNT_SLICE_CAPS], c4[2]);
-    if (c4[3]) atomicAdd(&p.counters[FBS_CNT_GAMMA_CAPS], c4[3]);
-    if (nf) {
-      atomicAdd(&p.counters[FBS_CNT_NONFINITE], (unsigned long long)nf);
-      atomicOr(&p.hyp->flags, kFlagNonfinite);
-    }
-  }
-}
-
-// ---------------------------------------------------------------- split sweep kernels (FP64)
+// ---------------------------------------------------------------- sweep kernels (FP64)
 //
-// The same arithmetic as k_gene_f64 split in two launches so that every SM gets
-// work at any G and the hyperparameter kernel of sweep m can run concurrently
-// with the eps kernel of sweep m+1 (the eps conditionals involve no
-// hyperparameter).  k_gene_f64 remains for fbs_sweep_noalloc.
+// Step 1 and steps 2 and 5 are two launches, so that every SM gets work at any G
+// and the hyperparameter kernel of sweep m can run concurrently with the eps
+// kernel of sweep m+1 (the eps conditionals involve no hyperparameter).
+// fbs_sweep_noalloc, which has no room for the rates between the two, runs the
+// same device functions in one kernel (k_sweep_f64).
 
 __device__ __forceinline__ void add_counters_u(unsigned long long* base, unsigned evals_e,
                                                unsigned evals_b, unsigned caps, unsigned gcaps,
@@ -410,90 +245,131 @@ __device__ __forceinline__ void add_counters_u(unsigned long long* base, unsigne
   }
 }
 
-// Step 1: one thread per eps_gn (element e = n*G + g of the [N][G] planes).
-__global__ void __launch_bounds__(256) k_eps_f64(ModelConst mc, DevPtrs p, int seg_i) {
-  ktime_begin(p.ktime, p.ktime_n, 3 * seg_i);
+// The FP64 comparisons throughout, for starts that the FP32 filter does not cover
+// (out of line: rare, and its exponentials would double the kernels' code).
+template <class F>
+static __device__ __noinline__ SliceResult slice_update_ol(double x0, double w, const F& f, Rng& r,
+                                                           int K, int shrink_max) {
+  return slice_update(x0, w, f, r, K, shrink_max);
+}
+
+// Whether FP32 holds a slice width with room for its multiples.
+__device__ __forceinline__ bool width_fits(double w) {
+  const float wf = (float)w;
+  return wf > 1e-30f && wf < 1e30f;
+}
+
+// The iteration a launch runs and the weight 1/k of its draw in the running
+// moments (0: none), from the segment snapshot.
+__device__ __forceinline__ double eps_moment_weight(const Hyper* hy, long long it) {
+  long long before = (it - 1) - (hy->seg_it > hy->burnin ? hy->seg_it : hy->burnin);
+  if (before < 0) before = 0;
+  return 1.0 / (double)(hy->seg_nmom + before + 1);
+}
+
+// Step 1 for one eps_gn: the update, the width, the moments and the rate at the
+// new value (returned in aux).  hg = 1/(2 gamma_g) and inv_k (the weight of the
+// draw in the moments) are the same for many elements and come from the caller.
+__device__ __forceinline__ SliceResult eps_update_f64(const ModelConst& mc, const DevPtrs& p, int n,
+                                                      int g, double hg, float hgf, long long it,
+                                                      double inv_k) {
   const int G = mc.G, N = mc.N, L = mc.L;
+  const long long burnin = p.hyp->burnin, tune_start = p.hyp->tune_start;
+  const size_t e = (size_t)n * G + g;
+  double A = mc.h[n];
+#pragma unroll
+  for (int l = 0; l < kMaxL; ++l)
+    if (l < L) A += mc.X[n * kMaxL + l] * p.beta[(size_t)l * G + g];
+  EpsDensity f{p.y[e], A, hg};
+  Rng r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamEps, (uint32_t)((size_t)g * N + n), (uint32_t)it);
+  const double x0 = p.eps[e];
+  double w = p.w_eps[e];
+  // comparisons decided in FP32 where an error bound allows (the same result);
+  // a start whose rate does not fit FP32 takes the FP64 comparisons throughout
+  const float af = (float)(A + x0), yf = (float)f.y, x0f = (float)x0;
+  const float mu0f = expf(af);
+  SliceResult s;
+  if (isfinite(mu0f) && isfinite(hgf) && isfinite(x0f) && af < 80.0f && width_fits(w)) {
+    const float amag = fabsf(af) + 8.0f;
+    EpsFilter ff{yf, mu0f, x0f, hgf, amag, yf * fabsf(x0f) + mu0f * amag + x0f * x0f * hgf + 64.0f};
+    s = slice_update_filtered(x0, w, f, ff, r, mc.K, mc.shrink_max);
+    s.aux = exp(A + s.x);  // the rate at the result, as the density computes it
+  } else {
+    s = slice_update_ol(x0, w, f, r, mc.K, mc.shrink_max);
+  }
+  p.eps[e] = s.x;
+  if (it <= burnin) {
+    double waux = p.waux_eps[e];
+    tune_width(w, waux, it, s.x, x0, burnin, tune_start);
+    p.w_eps[e] = w;
+    p.waux_eps[e] = waux;
+  } else if (mc.moments_eps) {
+    const double m = p.m_eps[e], q = p.q_eps[e];
+    p.m_eps[e] = m + (s.x - m) * inv_k;
+    p.q_eps[e] = q + (s.x * s.x - q) * inv_k;
+  }
+  return s;
+}
+
+// Step 1: one thread per eps_gn, a block 32 genes and blockDim.x / 32 samples (one
+// warp each), so that 1/(2 gamma_g) and the moments' weight, an FP64 division of a
+// dozen instructions each, are taken once per block instead of by every warp.
+// Bound by the FP64 pipe (16 cycles per warp instruction; 84% busy).  N=16 G=40000
+// L=5: 188 us; 258 us with the offsets taken in FP64 per evaluation, bounds that
+// grow with the counts, and the divisions per thread.
+__global__ void __launch_bounds__(256, 3) k_eps_f64(ModelConst mc, DevPtrs p, int seg_i) {
+  __shared__ double s_hg[32], s_inv_k;
+  __shared__ float s_hgf[32];
+  ktime_begin(p.ktime, p.ktime_n, 3 * seg_i);
   const Hyper* hy = p.hyp;
   const long long it = hy->seg_it + seg_i + 1;
-  const long long burnin = hy->burnin, tune_start = hy->tune_start;
-  const bool mom = it > burnin;
-  long long before = (it - 1) - (hy->seg_it > burnin ? hy->seg_it : burnin);
-  if (before < 0) before = 0;
-  const double inv_k = mom ? 1.0 / (double)(hy->seg_nmom + before + 1) : 0.0;
-  const int n = blockIdx.y;
-  const int g = blockIdx.x * blockDim.x + threadIdx.x;
-  const size_t e = (size_t)n * G + g;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, rows = blockDim.x >> 5;
+  const int n = blockIdx.y * rows + warp;
+  const int g = blockIdx.x * 32 + lane;
+  if (warp == 0) {
+    const double hg = g < mc.G ? 0.5 / p.gam[g] : 0.0;
+    s_hg[lane] = hg;
+    s_hgf[lane] = (float)hg;
+  }
+  if (warp == rows - 1 && lane == 0) s_inv_k = it > hy->burnin ? eps_moment_weight(hy, it) : 0.0;
+  __syncthreads();
   unsigned evals = 0, caps = 0, nonfin = 0;
-  if (g < G) {
-    double A = mc.h[n];
-#pragma unroll
-    for (int l = 0; l < kMaxL; ++l)
-      if (l < L) A += mc.X[n * kMaxL + l] * p.beta[(size_t)l * G + g];
-    EpsDensity f{(double)p.y[e], A, 0.5 / p.gam[g]};
-    Rng r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamEps, (uint32_t)((size_t)g * N + n),
-          (uint32_t)it);
-    const double x0 = p.eps[e];
-    double w = p.w_eps[e];
-    // comparisons decided in FP32 where an error bound allows (the same result);
-    // a start whose rate does not fit FP32 takes the FP64 comparisons throughout
-    const float af = (float)(A + x0), hgf = (float)f.hg, yf = (float)f.y, x0f = (float)x0;
-    const float mu0f = expf(af);
-    SliceResult s;
-    if (isfinite(mu0f) && isfinite(hgf) && isfinite(x0f) && af < 80.0f) {
-      const float amag = fabsf(af) + 8.0f;
-      EpsFilter ff{x0, yf, mu0f, x0f, hgf, amag,
-                   yf * fabsf(x0f) + mu0f * amag + x0f * x0f * hgf + 64.0f};
-      s = slice_update_filtered(x0, w, f, ff, r, mc.K, mc.shrink_max);
-      s.aux = exp(A + s.x);  // the rate at the result, as the density computes it
-    } else {
-      s = slice_update(x0, w, f, r, mc.K, mc.shrink_max);
-    }
+  if (g < mc.G && n < mc.N) {
+    const SliceResult s = eps_update_f64(mc, p, n, g, s_hg[lane], s_hgf[lane], it, s_inv_k);
     evals = s.evals;
     caps = s.capped;
     nonfin = s.nonfinite;
-    p.mu[e] = s.aux;
-    p.eps[e] = s.x;
-    if (it <= burnin) {
-      double waux = p.waux_eps[e];
-      tune_width(w, waux, it, s.x, x0, burnin, tune_start);
-      p.w_eps[e] = w;
-      p.waux_eps[e] = waux;
-    }
-    if (mom && mc.moments_eps) {
-      const double m = p.m_eps[e], q = p.q_eps[e];
-      p.m_eps[e] = m + (s.x - m) * inv_k;
-      p.q_eps[e] = q + (s.x * s.x - q) * inv_k;
-    }
+    p.mu[(size_t)n * mc.G + g] = s.aux;
   }
-  add_counters_u(p.counters + ((blockIdx.x + blockIdx.y) % kCounterCopies) * FBS_NUM_COUNTERS, evals, 0, caps,
-                 0, nonfin, &p.hyp->flags);
+  add_counters_u(p.counters + ((blockIdx.x + blockIdx.y) % kCounterCopies) * FBS_NUM_COUNTERS, evals,
+                 0, caps, 0, nonfin, &p.hyp->flags);
   ktime_end(p.ktime, p.ktime_n, 3 * seg_i);
 }
 
-// Steps 2 and 5: one thread per gene, after the eps kernel of this sweep and the
-// hyperparameter kernel of the previous one.
+// What a gamma/beta launch reads and counts, per thread.
+struct GbF64 {
+  const Hyper* hy;
+  long long it, burnin, tune_start, trace_row;
+  bool mom, trace_now;
+  double inv_k;
+  unsigned evals_b, evals_g, caps, gcaps, nonfin;
+};
+
 // One slice update of beta_gl (step 5) for a column with NC value classes, with
 // the class sums of the rates in shared memory, the moments, trace and partials.
+// hs = 1/(2 sigma_l^2).
 template <int NC>
 __device__ __forceinline__ void beta_column_f64(const ModelConst& mc, const DevPtrs& p, int l,
                                                 int g, double* mu, double* bs, double* ps, int B,
-                                                int tid, const Hyper* hy, long long it,
-                                                uint32_t it32, long long burnin,
-                                                long long tune_start, bool mom, double inv_k,
-                                                bool trace_now, long long trace_row,
-                                                unsigned& evals_b, unsigned& caps,
-                                                unsigned& nonfin) {
+                                                int tid, double theta, double hs, GbF64& c) {
   const int G = mc.G, N = mc.N, L = mc.L;
   const size_t e = (size_t)l * G + g;
-  const double theta = hy->phi[2 + l];
-  const double sig2 = hy->phi[2 + L + l];
   BetaDensityT<NC> f;
   f.T = p.T[e];
   const double b_cur = bs[l * B + tid];
   f.b0 = b_cur;
   f.theta = theta;
-  f.hs = 0.5 / sig2;
+  f.hs = hs;
   f.ncls = mc.ncls[l];
 #pragma unroll
   for (int j = 0; j < NC; ++j) {
@@ -502,38 +378,43 @@ __device__ __forceinline__ void beta_column_f64(const ModelConst& mc, const DevP
     f.kind[j] = mc.ckind[l][j];
   }
   for (int n = 0; n < N; ++n) {
-    const int c = mc.cls[l][n];
-    const double m = mu[n * blockDim.x + tid];
+    const int k = mc.cls[l][n];
+    const double m = mu[n * B + tid];
 #pragma unroll
     for (int j = 0; j < NC; ++j)
-      if (j == c) f.Q[j] += m;
+      if (j == k) f.Q[j] += m;
   }
-  Rng r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamBeta, (uint32_t)((size_t)g * L + l), it32);
+  Rng r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamBeta, (uint32_t)((size_t)g * L + l),
+        (uint32_t)c.it);
   const double x0 = b_cur;
   double w = p.w_beta[e];
   // comparisons decided in FP32 where an error bound allows (the same result)
   BetaFilterT<NC> ff;
-  ff.b0 = x0;
   ff.b0f = (float)x0;
-  ff.T = (float)f.T;
   ff.bt = (float)(x0 - theta);
-  ff.hs = (float)f.hs;
+  ff.hs = (float)hs;
   ff.ncls = f.ncls;
-  bool filt = isfinite(ff.T) && isfinite(ff.bt) && isfinite(ff.hs) && isfinite(ff.b0f);
-  float qs = 0.0f;
+  float qs = 0.0f, vq = 0.0f;
+  double D = f.T;
 #pragma unroll
   for (int j = 0; j < NC; ++j) {
     ff.Q[j] = (float)f.Q[j];
-    ff.v[j] = (float)f.v[j];
-    if (NC < kMaxCls || j < f.ncls) qs += ff.Q[j];
+    ff.v[j] = mc.cvalf[l][j];
+    if (NC < kMaxCls || j < f.ncls) {
+      D -= f.v[j] * f.Q[j];
+      qs += ff.Q[j];
+      vq += fabsf(ff.v[j]) * ff.Q[j];
+    }
   }
-  filt = filt && isfinite(qs);
-  ff.c64 = fabsf(ff.b0f) * fabsf(ff.T) + qs + ff.bt * ff.bt * ff.hs + 64.0f;
-  SliceResult s = filt && isfinite(ff.c64) ? slice_update_filtered(x0, w, f, ff, r, mc.K, mc.shrink_max)
-                                           : slice_update(x0, w, f, r, mc.K, mc.shrink_max);
-  evals_b += s.evals;
-  caps += s.capped;
-  nonfin += s.nonfinite;
+  ff.D = (float)D;
+  ff.Tm = 1.01f * (fabsf(ff.D) + vq);
+  ff.c64 = fabsf(ff.b0f) * ff.Tm + qs + ff.bt * ff.bt * ff.hs + 64.0f;
+  SliceResult s = isfinite(ff.c64) && isfinite(ff.Tm) && width_fits(w)
+                      ? slice_update_filtered(x0, w, f, ff, r, mc.K, mc.shrink_max)
+                      : slice_update_ol(x0, w, f, r, mc.K, mc.shrink_max);
+  c.evals_b += s.evals;
+  c.caps += s.capped;
+  c.nonfin += s.nonfinite;
   if (s.x != x0) {
     const double dlt = s.x - x0;
     double ej[NC];
@@ -548,50 +429,175 @@ __device__ __forceinline__ void beta_column_f64(const ModelConst& mc, const DevP
       }
     }
     for (int n = 0; n < N; ++n) {
-      const int c = mc.cls[l][n];
+      const int k = mc.cls[l][n];
       double fac = 1.0;
 #pragma unroll
       for (int j = 0; j < NC; ++j)
-        if (j == c) fac = ej[j];
-      mu[n * blockDim.x + tid] *= fac;
+        if (j == k) fac = ej[j];
+      if (k >= 0) mu[n * B + tid] *= fac;
     }
   }
   bs[l * B + tid] = s.x;
   p.beta[e] = s.x;
-  if (it <= burnin) {
+  if (c.it <= c.burnin) {
     double waux = p.waux_beta[e];
-    tune_width(w, waux, it, s.x, x0, burnin, tune_start);
+    tune_width(w, waux, c.it, s.x, x0, c.burnin, c.tune_start);
     p.w_beta[e] = w;
     p.waux_beta[e] = waux;
   }
-  if (mom) {
+  if (c.mom) {
     const double m = p.m_beta[e], q = p.q_beta[e];
-    p.m_beta[e] = m + (s.x - m) * inv_k;
-    p.q_beta[e] = q + (s.x * s.x - q) * inv_k;
+    p.m_beta[e] = m + (s.x - m) * c.inv_k;
+    p.q_beta[e] = q + (s.x * s.x - q) * c.inv_k;
   }
-  if (trace_now) p.trace_beta[(size_t)trace_row * L * G + e] = s.x;
+  if (c.trace_now) p.trace_beta[(size_t)c.trace_row * L * G + e] = s.x;
   const double dv = s.x - theta;
   ps[(2 + l) * B + tid] = dv;
   ps[(2 + kMaxL + l) * B + tid] = dv * dv;
 }
 
-__global__ void __launch_bounds__(128) k_gb_f64(ModelConst mc, DevPtrs p, int seg_i) {
+// Columns of three and more classes, out of line: their register needs (up to
+// eight class sums in FP64) would otherwise be the kernel's.
+template <int NC>
+static __device__ __noinline__ void beta_column_f64_ol(const ModelConst& mc, const DevPtrs& p, int l,
+                                                       int g, double* mu, double* bs, double* ps,
+                                                       int B, int tid, double theta, double hs,
+                                                       GbF64& c) {
+  beta_column_f64<NC>(mc, p, l, g, mu, bs, ps, B, tid, theta, hs, c);
+}
+
+// The values that are the same for every gene of a launch: lane l < L of a warp
+// takes 1/(2 sigma_l^2), lane L the moments' weight (one division for all).
+struct GbUniform {
+  double hs[kMaxL], inv_k;
+};
+
+__device__ __forceinline__ void gb_uniform(const ModelConst& mc, const Hyper* hy, bool mom,
+                                           int lane, GbUniform* u) {
+  if (lane <= mc.L) {
+    const double num = lane < mc.L ? 0.5 : 1.0;
+    const double den = lane < mc.L ? hy->phi[2 + mc.L + lane] : (double)(hy->n_mom + 1);
+    const double q = num / den;
+    if (lane < mc.L) u->hs[lane] = q;
+    else u->inv_k = mom ? q : 0.0;
+  }
+}
+
+__device__ __forceinline__ GbF64 gb_begin_f64(const ModelConst& mc, const DevPtrs& p, int seg_i) {
+  const Hyper* hy = p.hyp;
+  GbF64 c;
+  c.hy = hy;
+  c.it = hy->seg_it + seg_i + 1;
+  c.burnin = hy->burnin;
+  c.tune_start = hy->tune_start;
+  c.mom = c.it > c.burnin;
+  c.trace_now = c.mom && mc.trace_beta && p.trace_beta != nullptr &&
+                ((c.it - c.burnin) % hy->thin == 0) && hy->trace_rows < hy->trace_cap;
+  c.trace_row = hy->trace_rows;
+  c.inv_k = 0.0;
+  c.evals_b = c.evals_g = c.caps = c.gcaps = c.nonfin = 0;
+  return c;
+}
+
+// Steps 2 and 5 for gene g (thread tid of the B genes whose rates mu [N][B] are in
+// shared memory): the gamma_g draw, the beta_gl, their moments and trace, and the
+// thread's terms ps [kNumPart][B] of the sums for steps 3, 4, 6, 7.
+__device__ __forceinline__ void gb_gene_f64(const ModelConst& mc, const DevPtrs& p, int g, int B,
+                                            int tid, double* mu, double* bs, double* ps,
+                                            const GbUniform& u, GbF64& c) {
+  const int G = mc.G, N = mc.N, L = mc.L;
+  const Hyper* hy = c.hy;
+  const double nu = hy->phi[0], tau = hy->phi[1];
+  for (int l = 0; l < L; ++l) bs[l * B + tid] = p.beta[(size_t)l * G + g];
+  double ss = 0.0;
+#pragma unroll 8
+  for (int n = 0; n < N; ++n) {
+    const double x = p.eps[(size_t)n * G + g];
+    ss += x * x;
+  }
+  // ---- step 2: gamma_g ~ IG((N + nu)/2, (sum eps^2 + nu tau)/2), exactly or
+  // (all_slice) by a slice update of that density with the gene's own width
+  {
+    Rng r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamGamma, (uint32_t)g, (uint32_t)c.it);
+    const double shape = 0.5 * ((double)N + nu);
+    const double scale = 0.5 * (ss + nu * tau);
+    double gam;
+    if (mc.all_slice) {
+      const double x0 = p.gam[g];
+      double w = p.w_gam[g], waux = p.waux_gam[g];
+      const GamDensity f{shape + 1.0, scale};
+      GamFilter ff;
+      const float x0f = (float)x0;
+      ff.s1 = (float)f.shape1;
+      ff.ix = 1.0f / x0f;
+      ff.bx = (float)scale * ff.ix;
+      ff.c64 = ff.s1 * (fabsf(__logf(x0f)) + 1.0f) + ff.bx + 64.0f;
+      const bool filt = x0f > 1e-30f && ff.ix > 0.0f && isfinite(ff.c64) && width_fits(w);
+      SliceResult s = filt ? slice_update_filtered(x0, w, f, ff, r, mc.K, mc.shrink_max)
+                           : slice_update_ol(x0, w, f, r, mc.K, mc.shrink_max);
+      c.evals_g += s.evals;
+      c.caps += s.capped;
+      c.nonfin += s.nonfinite;
+      gam = s.x;
+      if (c.it <= c.burnin) {
+        tune_width(w, waux, c.it, s.x, x0, c.burnin, c.tune_start);
+        p.w_gam[g] = w;
+        p.waux_gam[g] = waux;
+      }
+    } else {
+      bool gcap = false;
+      gam = scale / gamma_mt(shape, r, 0, &gcap);
+      c.gcaps += gcap;
+    }
+    p.gam[g] = gam;
+    if (c.mom) {
+      const double m = p.m_gam[g], q = p.q_gam[g];
+      p.m_gam[g] = m + (gam - m) * c.inv_k;
+      p.q_gam[g] = q + (gam * gam - q) * c.inv_k;
+    }
+    ps[0 * B + tid] = log(gam);
+    ps[1 * B + tid] = 1.0 / gam;
+  }
+
+  // ---- step 5: beta_gl, l = 1..L in order
+  for (int l = 0; l < L; ++l) {
+    const double theta = hy->phi[2 + l], hs = u.hs[l];
+    switch (mc.ncls[l]) {
+      case 1: beta_column_f64<1>(mc, p, l, g, mu, bs, ps, B, tid, theta, hs, c); break;
+      case 2: beta_column_f64<2>(mc, p, l, g, mu, bs, ps, B, tid, theta, hs, c); break;
+      case 3: beta_column_f64_ol<3>(mc, p, l, g, mu, bs, ps, B, tid, theta, hs, c); break;
+      default: beta_column_f64_ol<kMaxCls>(mc, p, l, g, mu, bs, ps, B, tid, theta, hs, c);
+    }
+  }
+  // contrast probabilities (§3.1): count the iterations whose beta_g satisfies
+  // each proposition
+  if (c.mom && p.con != nullptr) {
+    const Contrasts* cs = p.con;
+    for (int q = 0; q < cs->n; ++q) {
+      bool ok = true;
+      for (int k = 0; k < cs->terms[q] && ok; ++k) {
+        double sv = 0.0;
+        for (int l = 0; l < L; ++l) sv = __dadd_rn(sv, __dmul_rn(cs->v[q][k][l], bs[l * B + tid]));
+        ok = sv > cs->b[q][k];
+      }
+      if (ok) p.con_count[(size_t)q * G + g] += 1u;
+    }
+  }
+}
+
+// Steps 2 and 5: one thread per gene, after the eps kernel of this sweep and the
+// hyperparameter kernel of the previous one.  At most 168 registers, so that all
+// 1250 one-warp blocks of G=40000 are resident at once (at 248 eight fit an SM,
+// 1216 in all, and 34 ran alone).  N=16 G=40000 L=5: 118 us, FP64 pipe 72% busy; 301
+// us before the filter's bounds were freed of the counts.
+__global__ void __launch_bounds__(128, 3) k_gb_f64(ModelConst mc, DevPtrs p, int seg_i) {
   // shared: mu[N][B], beta[L][B], partials[kNumPart][B] (values indexed by a runtime
   // l live here rather than in local memory), then the reduction scratch
   extern __shared__ double smem_dyn[];
+  __shared__ GbUniform u;
   ktime_begin(p.ktime, p.ktime_n, 3 * seg_i + 1);
-  const int G = mc.G, N = mc.N, L = mc.L;
-  const Hyper* hy = p.hyp;
-  const long long it = hy->seg_it + seg_i + 1;
-  const uint32_t it32 = (uint32_t)it;
-  const long long burnin = hy->burnin, tune_start = hy->tune_start;
-  const bool mom = it > burnin;
-  const double inv_k = mom ? 1.0 / (double)(hy->n_mom + 1) : 0.0;
-  const double nu = hy->phi[0], tau = hy->phi[1];
-  const bool trace_now = mom && mc.trace_beta && p.trace_beta != nullptr &&
-                         ((it - burnin) % hy->thin == 0) && hy->trace_rows < hy->trace_cap;
-  const long long trace_row = hy->trace_rows;
-
+  const int G = mc.G, N = mc.N;
+  GbF64 c = gb_begin_f64(mc, p, seg_i);
   const int B = blockDim.x;
   double* mu = smem_dyn;
   double* bs = mu + (size_t)N * B;
@@ -599,100 +605,95 @@ __global__ void __launch_bounds__(128) k_gb_f64(ModelConst mc, DevPtrs p, int se
   const int tid = threadIdx.x;
   const int g = blockIdx.x * B + tid;
   const bool active = g < G;
-
+  if (active) {
+#pragma unroll 8
+    for (int n = 0; n < N; ++n) mu[n * B + tid] = p.mu[(size_t)n * G + g];
+  }
 #pragma unroll
   for (int i = 0; i < kNumPart; ++i) ps[i * B + tid] = 0.0;
-  unsigned evals_b = 0, evals_g = 0, caps = 0, gcaps = 0, nonfin = 0;
-
-  if (active) {
-    for (int l = 0; l < L; ++l) bs[l * B + tid] = p.beta[(size_t)l * G + g];
-    double ss = 0.0;
-#pragma unroll 4
-    for (int n = 0; n < N; ++n) {
-      const size_t e = (size_t)n * G + g;
-      const double x = p.eps[e];
-      ss += x * x;
-      mu[n * blockDim.x + tid] = p.mu[e];
-    }
-
-    // ---- step 2: gamma_g ~ IG((N + nu)/2, (sum eps^2 + nu tau)/2), exactly or
-    // (all_slice) by a slice update of that density with the gene's own width
-    {
-      Rng r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamGamma, (uint32_t)g, it32);
-      const double shape = 0.5 * ((double)N + nu);
-      const double scale = 0.5 * (ss + nu * tau);
-      double gam;
-      if (mc.all_slice) {
-        const double x0 = p.gam[g];
-        double w = p.w_gam[g], waux = p.waux_gam[g];
-        SliceResult s = slice_update(x0, w, GamDensity{shape + 1.0, scale}, r, mc.K, mc.shrink_max);
-        evals_g += s.evals;
-        caps += s.capped;
-        nonfin += s.nonfinite;
-        gam = s.x;
-        if (it <= burnin) {
-          tune_width(w, waux, it, s.x, x0, burnin, tune_start);
-          p.w_gam[g] = w;
-          p.waux_gam[g] = waux;
-        }
-      } else {
-        bool gcap = false;
-        gam = scale / gamma_mt(shape, r, 0, &gcap);
-        gcaps += gcap;
-      }
-      p.gam[g] = gam;
-      if (mom) {
-        const double m = p.m_gam[g], q = p.q_gam[g];
-        p.m_gam[g] = m + (gam - m) * inv_k;
-        p.q_gam[g] = q + (gam * gam - q) * inv_k;
-      }
-      ps[0 * B + tid] = log(gam);
-      ps[1 * B + tid] = 1.0 / gam;
-    }
-
-    // ---- step 5: beta_gl, l = 1..L in order
-    for (int l = 0; l < L; ++l) {
-      switch (mc.ncls[l]) {
-        case 1:
-          beta_column_f64<1>(mc, p, l, g, mu, bs, ps, B, tid, hy, it, it32, burnin, tune_start, mom, inv_k,
-                               trace_now, trace_row, evals_b, caps, nonfin);
-          break;
-        case 2:
-          beta_column_f64<2>(mc, p, l, g, mu, bs, ps, B, tid, hy, it, it32, burnin, tune_start, mom, inv_k,
-                               trace_now, trace_row, evals_b, caps, nonfin);
-          break;
-        case 3:
-          beta_column_f64<3>(mc, p, l, g, mu, bs, ps, B, tid, hy, it, it32, burnin, tune_start, mom, inv_k,
-                               trace_now, trace_row, evals_b, caps, nonfin);
-          break;
-        default:
-          beta_column_f64<kMaxCls>(mc, p, l, g, mu, bs, ps, B, tid, hy, it, it32, burnin, tune_start, mom, inv_k,
-                               trace_now, trace_row, evals_b, caps, nonfin);
-      }
-    }
-    // contrast probabilities (§3.1): count the iterations whose beta_g satisfies
-    // each proposition
-    if (mom && p.con != nullptr) {
-      const Contrasts* cs = p.con;
-      for (int q = 0; q < cs->n; ++q) {
-        bool ok = true;
-        for (int k = 0; k < cs->terms[q] && ok; ++k) {
-          double sv = 0.0;
-          for (int l = 0; l < L; ++l) sv = __dadd_rn(sv, __dmul_rn(cs->v[q][k][l], bs[l * B + tid]));
-          ok = sv > cs->b[q][k];
-        }
-        if (ok) p.con_count[(size_t)q * G + g] += 1u;
-      }
-    }
-  }
+  if (tid < 32) gb_uniform(mc, c.hy, c.mom, tid, &u);
+  __syncthreads();
+  c.inv_k = u.inv_k;
+  if (active) gb_gene_f64(mc, p, g, B, tid, mu, bs, ps, u, c);
 
   double part[kNumPart];
 #pragma unroll
   for (int i = 0; i < kNumPart; ++i) part[i] = ps[i * B + tid];
   double* red = ps + (size_t)kNumPart * B;
   block_sum_to<kNumPart>(part, p.partial + (size_t)blockIdx.x * kNumPart, red);
-  add_counters_u(p.counters, 0, evals_b, caps, gcaps, nonfin, &p.hyp->flags, evals_g);
+  add_counters_u(p.counters, 0, c.evals_b, c.caps, c.gcaps, c.nonfin, &p.hyp->flags, c.evals_g);
   ktime_end(p.ktime, p.ktime_n, 3 * seg_i + 1);
+}
+
+// Steps 1, 2 and 5 in one launch for fbs_sweep_noalloc: a block takes 32 genes, its
+// four warps the samples' eps updates in turn with the rates kept in shared
+// memory, then the first warp the genes' gamma and beta updates.  The four blocks
+// of a cluster are the 128 genes of one row of partial sums (what the fixed
+// scratch has rows for) and add their sums in order through distributed shared
+// memory.  32 genes per block, not 128: N=16 G=20011 is 626 blocks for 152 SMs
+// instead of 157, and a few blocks share an SM, so that the one's serial gene
+// phase runs beside the other's eps phase.  Bound by the FP64 pipe.  One sweep of
+// N=16 G=20011 L=5: 659 us with one thread per gene making its 16 eps updates in a
+// row in FP64, 290 us so.
+constexpr int kSweepWarps = 4, kSweepCluster = 4;
+
+__global__ void __cluster_dims__(kSweepCluster, 1, 1) __launch_bounds__(32 * kSweepWarps, 3)
+    k_sweep_f64(ModelConst mc, DevPtrs p) {
+  extern __shared__ double smem_dyn[];  // mu[N][32], beta[kMaxL][32], partials[kNumPart][32]
+  __shared__ GbUniform u;
+  __shared__ double s_hg[32], s_inv_k, s_sum[kNumPart];
+  __shared__ float s_hgf[32];
+  const int G = mc.G, N = mc.N;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g = blockIdx.x * 32 + lane;
+  double* mu = smem_dyn;
+  double* bs = mu + (size_t)N * 32;
+  double* ps = bs + (size_t)kMaxL * 32;
+  GbF64 c = gb_begin_f64(mc, p, 0);
+  if (warp == 0) {
+    const double hg = g < G ? 0.5 / p.gam[g] : 0.0;
+    s_hg[lane] = hg;
+    s_hgf[lane] = (float)hg;
+  } else if (warp == 1) {
+    gb_uniform(mc, c.hy, c.mom, lane, &u);
+  } else if (warp == 2) {
+    if (lane == 0) s_inv_k = c.mom ? eps_moment_weight(c.hy, c.it) : 0.0;
+#pragma unroll
+    for (int i = 0; i < kNumPart; ++i) ps[i * 32 + lane] = 0.0;
+  }
+  __syncthreads();
+  unsigned evals_e = 0;
+  if (g < G) {
+    for (int n = warp; n < N; n += kSweepWarps) {
+      const SliceResult s = eps_update_f64(mc, p, n, g, s_hg[lane], s_hgf[lane], c.it, s_inv_k);
+      evals_e += s.evals;
+      c.caps += s.capped;
+      c.nonfin += s.nonfinite;
+      mu[n * 32 + lane] = s.aux;
+    }
+  }
+  __syncthreads();
+  if (warp == 0) {
+    c.inv_k = u.inv_k;
+    if (g < G) gb_gene_f64(mc, p, g, 32, lane, mu, bs, ps, u, c);
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < kNumPart; ++i) {
+      double x = ps[i * 32 + lane];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+      if (lane == 0) s_sum[i] = x;
+    }
+  }
+  add_counters_u(p.counters, evals_e, c.evals_b, c.caps, c.gcaps, c.nonfin, &p.hyp->flags, c.evals_g);
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  if (cl.block_rank() == 0 && threadIdx.x < kNumPart) {
+    double sum = 0.0;
+    for (unsigned r = 0; r < kSweepCluster; ++r) sum += cl.map_shared_rank(s_sum, r)[threadIdx.x];
+    p.partial[(size_t)(blockIdx.x / kSweepCluster) * kNumPart + threadIdx.x] = sum;
+  }
+  cl.sync();  // the other blocks' sums stay until they are read
 }
 
 __global__ void __launch_bounds__(kHyperThreads) k_hyper(ModelConst mc, DevPtrs p, int nblk) {
@@ -1018,13 +1019,10 @@ __global__ void k_uniforms(uint32_t seed_lo, uint32_t seed_hi, uint32_t chain, u
 
 // ---------------------------------------------------------------- launchers
 
-size_t gene_smem_bytes(int N, int block) {
-  return (size_t)N * block * sizeof(double) + (size_t)(block / 32) * kNumPart * sizeof(double);
-}
-
-cudaError_t launch_gene(const ModelConst& mc, const DevPtrs& p, int block, cudaStream_t s) {
-  const int nblk = (mc.G + block - 1) / block;
-  k_gene_f64<<<nblk, block, gene_smem_bytes(mc.N, block), s>>>(mc, p);
+cudaError_t launch_sweep_f64(const ModelConst& mc, const DevPtrs& p, cudaStream_t s) {
+  const int nblk = (mc.G + 127) / 128 * kSweepCluster;
+  const size_t smem = ((size_t)mc.N + kMaxL + kNumPart) * 32 * sizeof(double);
+  k_sweep_f64<<<nblk, 32 * kSweepWarps, smem, s>>>(mc, p);
   return cudaGetLastError();
 }
 
@@ -1039,12 +1037,6 @@ size_t gb_smem_bytes_f64(int N, int block) {
 }
 
 cudaError_t prepare_gene_kernel(int N, int block) {
-  const size_t smem = gene_smem_bytes(N, block);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k_gene_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess) return e;
-  }
   const size_t smem_gb = gb_smem_bytes_f64(N, block);
   if (smem_gb > 48 * 1024)
     return cudaFuncSetAttribute(k_gb_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1053,9 +1045,10 @@ cudaError_t prepare_gene_kernel(int N, int block) {
 }
 
 cudaError_t launch_eps_f64(const ModelConst& mc, const DevPtrs& p, int seg_i, cudaStream_t s) {
-  const int blk = 256;
-  const dim3 grid((unsigned)((mc.G + blk - 1) / blk), (unsigned)mc.N);
-  k_eps_f64<<<grid, blk, 0, s>>>(mc, p, seg_i);
+  // as few idle warps as blocks of up to eight samples leave
+  const int groups = (mc.N + 7) / 8, rows = (mc.N + groups - 1) / groups;
+  const dim3 grid((unsigned)((mc.G + 31) / 32), (unsigned)groups);
+  k_eps_f64<<<grid, 32 * rows, 0, s>>>(mc, p, seg_i);
   return cudaGetLastError();
 }
 

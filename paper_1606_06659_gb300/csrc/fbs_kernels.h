@@ -12,9 +12,9 @@ namespace fbs {
 
 constexpr int kDefaultBlock = 128;
 
-size_t gene_smem_bytes(int N, int block);
 cudaError_t prepare_gene_kernel(int N, int block);
-cudaError_t launch_gene(const ModelConst& mc, const DevPtrs& p, int block, cudaStream_t s);
+// Steps 1, 2 and 5 in one launch, the rates kept on chip; partial sums per 128 genes.
+cudaError_t launch_sweep_f64(const ModelConst& mc, const DevPtrs& p, cudaStream_t s);
 cudaError_t launch_hyper(const ModelConst& mc, const DevPtrs& p, int nblk, cudaStream_t s);
 cudaError_t launch_eps_f64(const ModelConst& mc, const DevPtrs& p, int seg_i, cudaStream_t s);
 cudaError_t launch_gb_f64(const ModelConst& mc, const DevPtrs& p, int block, int seg_i,

@@ -87,8 +87,8 @@ __global__ void k_noalloc_begin(Hyper* hy, unsigned long long* cnt, const double
   if (tid == 0) {
     hy->w_nu = hyp[P];
     hy->waux_nu = hyp[P + 1];
-    hy->it = it - 1;
-    hy->n_mom = n_mom;
+    hy->it = hy->seg_it = it - 1;
+    hy->n_mom = hy->seg_nmom = n_mom;
     hy->burnin = burnin;
     hy->tune_start = burnin / 2;
     hy->thin = 1;
@@ -193,6 +193,7 @@ int fbs_sweep_noalloc(const fbs_sweep_args* a) {
         if (nc == kMaxCls)
           return fail_na(FBS_E_ARG, "a column of X has more than FBS_MAX_CLASSES distinct values");
         mc.cval[l][nc] = v;
+        mc.cvalf[l][nc] = (float)v;
         mc.ckind[l][nc] = v == 1.0 ? kClsPlus : (v == -1.0 ? kClsMinus : kClsOther);
         ++nc;
       }
@@ -237,8 +238,7 @@ int fbs_sweep_noalloc(const fbs_sweep_args* a) {
   k_noalloc_begin<<<1, 64, 0, s>>>(d_hyp, d_cnt, a->hyp, m_phi, q_phi, P, a->it, a->n_mom,
                                    a->burnin);
   NA_CUDA(cudaGetLastError());
-  NA_CUDA(prepare_gene_kernel(N, kNoAllocBlock));
-  NA_CUDA(launch_gene(mc, p, kNoAllocBlock, s));
+  NA_CUDA(launch_sweep_f64(mc, p, s));
   NA_CUDA(launch_hyper(mc, p, (G + kNoAllocBlock - 1) / kNoAllocBlock, s));
   k_noalloc_end<<<1, 64, 0, s>>>(d_hyp, d_cnt, a->hyp, m_phi, q_phi, P,
                                  reinterpret_cast<unsigned long long*>(a->status));

@@ -61,24 +61,34 @@ struct Rng {
       : key0(seed_lo), key1(seed_hi), index(index_), sblk(stream << 24), iter(iter_),
         chain(chain_), cached(0xFFFFFFFFu), w(make_uint4(0, 0, 0, 0)) {}
 
-  __device__ __forceinline__ double u(uint32_t k) {
+  // The 64 random bits of uniform k.
+  __device__ __forceinline__ unsigned long long bits(uint32_t k) {
     const uint32_t blk = k >> 1;
     if (blk != cached) {
       w = philox4x32_10(make_uint4(index, sblk | blk, iter, chain), key0, key1);
       cached = blk;
     }
-    const unsigned long long x = (k & 1u)
-                                     ? ((unsigned long long)w.w << 32 | w.z)
-                                     : ((unsigned long long)w.y << 32 | w.x);
-    // (floor(x / 2^12) + 1/2) / 2^52 = v / 2^53 with v = 2 floor(x / 2^12) + 1, an odd
-    // integer below 2^53, so the double is assembled from integer operations: the
-    // leading bit of v moved to bit 52 gives the mantissa, its position the exponent
+    return (k & 1u) ? ((unsigned long long)w.w << 32 | w.z)
+                    : ((unsigned long long)w.y << 32 | w.x);
+  }
+
+  // (floor(x / 2^12) + 1/2) / 2^52 = v / 2^53 with v = 2 floor(x / 2^12) + 1, an odd
+  // integer below 2^53, so the double is assembled from integer operations: the
+  // leading bit of v moved to bit 52 gives the mantissa, its position the exponent
+  static __device__ __forceinline__ double to_u(unsigned long long x) {
     const unsigned long long v = ((x >> 12) << 1) | 1ull;
     const int sh = __clzll((long long)v) - 11;
-    const unsigned long long bits =
+    const unsigned long long b =
         ((unsigned long long)(1022 - sh) << 52) | ((v << sh) & 0xFFFFFFFFFFFFFull);
-    return __longlong_as_double((long long)bits);
+    return __longlong_as_double((long long)b);
   }
+
+  // The uniform of the bits x in FP32, within 2^-24 of itself plus 2^-33.
+  static __device__ __forceinline__ float to_f(unsigned long long x) {
+    return __fmul_rn(__fadd_rn(__uint2float_rn((uint32_t)(x >> 32)), 0.5f), 0x1p-32f);
+  }
+
+  __device__ __forceinline__ double u(uint32_t k) { return to_u(bits(k)); }
 };
 
 // Box-Muller normal from uniforms k0, k0+1 (cosine branch).
@@ -185,17 +195,42 @@ __device__ __forceinline__ SliceResult slice_update(double x0, double w, const F
   return res;
 }
 
+// K_L = min(floor((K+1) U), K) of Algorithm 2, rounded as the FP64 product of K + 1
+// and the uniform of the bits x: from the exact 128-bit product, unless that lies
+// so close below an integer that the FP64 product may round up to it.
+__device__ __forceinline__ int step_split(int K, unsigned long long x) {
+  const unsigned long long a = ((unsigned long long)K + 1ull) << 11, v = ((x >> 12) << 1) | 1ull;
+  // (K+1) U = a v / 2^64, below 2^32, so half an ulp of it is at most 2^-22
+  int KL = (int)__umul64hi(a, v);
+  if (a * v > ~0ull - (1ull << 42)) KL = (int)__dmul_rn((double)(K + 1), Rng::to_u(x));
+  return KL > K ? K : KL;
+}
+
 // slice_update (Algorithm 2, steps 1-6) with every comparison "log u < log f(p)"
-// first decided in FP32.  ff(p, &bound) returns Delta(p) = log f(p) - log f(x0)
-// in FP32 and a bound on the sum of its error and of the error with which the
-// FP64 evaluation (f) of the same comparison is made; with the FP32 level
-// log U_0, a gap beyond the two bounds decides the comparison exactly as the
-// FP64 arithmetic would, and only a gap inside them evaluates f in FP64 (the
-// level log f(x0) + log U_0 is then computed once).  The uniforms, the interval
-// arithmetic (FP64, rounded step by step), the evaluation count, the result and
-// its flags are those of slice_update; the caller computes the auxiliary value
-// at the result.  ff must be usable only where f(x0) is finite (the caller
-// checks this and otherwise calls slice_update), so nonfinite is false.
+// first decided in FP32, at the offset d = p - x0.  ff(d, derr, &bound) returns
+// Delta = log f(x0 + d) - log f(x0) in FP32 and a bound on the sum of its error,
+// given that d is within derr of p - x0, and of the error with which the FP64
+// evaluation (f) of the same comparison is made; with the FP32 level log U_0, a
+// gap beyond the two bounds decides the comparison exactly as the FP64 arithmetic
+// would, and only a gap inside them evaluates f in FP64 (the level log f(x0) +
+// log U_0 is then computed once).  The uniforms, the interval arithmetic (FP64,
+// rounded step by step), the evaluation count, the result and its flags are those
+// of slice_update; the caller computes the auxiliary value at the result.  ff must
+// be usable only where f(x0) is finite (the caller checks this and otherwise calls
+// slice_update), so nonfinite is false.
+//
+// A warp's FP64 instruction holds the SM's FP64 pipe for 16 cycles, so the offsets
+// are carried in FP32 beside the FP64 end points instead of being taken from them
+// (a subtraction and a conversion per evaluation): an evaluation costs the one
+// FP64 operation that moves the end point, or the three that make the proposal.
+// Errors, with e = 2^-24: the ends -w U_1 and w (1 - U_1) are products of two
+// rounded numbers (the second from the complement of the bits), within 4 e w; k
+// steps of w add the rounding of w, k w e <= e |d|, and one of the sum; the
+// proposal d = dlo + (dhi - dlo) u is a convex combination of the ends (their
+// error) plus at most 4 e (dhi - dlo) for the roundings of the length, u and the
+// sum.  The FP64 points themselves are rounded up to K + 1 times in stepping out
+// (2^-44 |x0| covers K <= 100; more steps are charged to it too) and three times
+// per proposal (2^-50 |x0|).
 template <class F, class FF>
 __device__ __forceinline__ SliceResult slice_update_filtered(double x0, double w, const F& f,
                                                              const FF& ff, Rng& r, int K,
@@ -204,49 +239,72 @@ __device__ __forceinline__ SliceResult slice_update_filtered(double x0, double w
   res.evals = 1;
   res.nonfinite = false;
   res.aux = 0.0;
-  const double u0 = r.u(0);
-  const float lu = logf((float)u0);
+  const unsigned long long b0 = r.bits(0);
+  const float u0f = b0 >= (1ull << 56) ? Rng::to_f(b0) : (float)Rng::to_u(b0);
+  const float lu = logf(u0f);
   // error of lu: the rounding of u0 to FP32 and logf's (ulp) error, with margin
   const float lu_err = 0x1p-20f * (fabsf(lu) + 1.0f);
+  const float wf = (float)w, x0m = fabsf((float)x0);
   double logu = 0.0;
   bool have_level = false;
-  auto above = [&](double pt) -> bool {  // the FP64 comparison logu < f(pt)
+  auto above = [&](double pt, float d, float derr) -> bool {  // the FP64 comparison logu < f(pt)
     float eb;
-    const float gap = ff(pt, &eb) - lu;
+    const float gap = ff(d, derr, &eb) - lu;
     const float tol = eb + lu_err;
     if (gap > tol) return true;
     if (gap < -tol) return false;
     if (!have_level) {
       double a0;
-      logu = __dadd_rn(f(x0, &a0), log(u0));
+      logu = __dadd_rn(f(x0, &a0), log(Rng::to_u(b0)));
       have_level = true;
     }
     double a;
     return logu < f(pt, &a);
   };
-  const double v = __dmul_rn(w, r.u(1));
+  const unsigned long long b1 = r.bits(1);
+  const double v = __dmul_rn(w, Rng::to_u(b1));
   double lo = __dsub_rn(x0, v);
   double hi = __dadd_rn(lo, w);
-  int KL = (int)__dmul_rn((double)(K + 1), r.u(2));
-  if (KL > K) KL = K;
+  const float dlo0 = -(wf * Rng::to_f(b1)), dhi0 = wf * Rng::to_f(~b1);
+  const int KL = step_split(K, r.bits(2));
   const int KR = K - KL;
-  for (int k = 0; k < KL; ++k) {
+  const float e64 = 0x1p-44f * (1.0f + 0x1p-6f * (float)K) * x0m;
+  const float derr0 = fmaf(0x1p-22f, wf, e64);
+  float dlo = dlo0, dhi = dhi0;
+  for (int k = 0; k < KL;) {
     ++res.evals;
-    if (above(lo)) lo = __dsub_rn(lo, w); else break;
+    if (!above(lo, dlo, fmaf(0x1p-22f, -dlo, derr0))) break;
+    lo = __dsub_rn(lo, w);
+    ++k;
+    dlo = fmaf(-(float)k, wf, dlo0);
   }
-  for (int k = 0; k < KR; ++k) {
+  for (int k = 0; k < KR;) {
     ++res.evals;
-    if (above(hi)) hi = __dadd_rn(hi, w); else break;
+    if (!above(hi, dhi, fmaf(0x1p-22f, dhi, derr0))) break;
+    hi = __dadd_rn(hi, w);
+    ++k;
+    dhi = fmaf((float)k, wf, dhi0);
   }
+  float derr = fmaf(0x1p-22f, dhi - dlo, derr0);
   for (int j = 0; j < shrink_max; ++j) {
-    const double xs = __dadd_rn(lo, __dmul_rn(__dsub_rn(hi, lo), r.u(3u + (uint32_t)j)));
+    const unsigned long long b = r.bits(3u + (uint32_t)j);
+    const double xs = __dadd_rn(lo, __dmul_rn(__dsub_rn(hi, lo), Rng::to_u(b)));
+    const float len = dhi - dlo;
+    const float d = fmaf(len, Rng::to_f(b), dlo);
+    derr = fmaf(0x1p-22f, len, fmaf(0x1p-50f, x0m, derr));
     ++res.evals;
-    if (above(xs)) {
+    if (above(xs, d, derr)) {
       res.x = xs;
       res.capped = false;
       return res;
     }
-    if (xs > x0) hi = xs; else lo = xs;
+    if (fabsf(d) > derr ? d > 0.0f : xs > x0) {
+      hi = xs;
+      dhi = d;
+    } else {
+      lo = xs;
+      dlo = d;
+    }
   }
   res.x = x0;
   res.capped = true;
