@@ -315,8 +315,9 @@ __device__ __forceinline__ SliceResult eps_update_f64(const ModelConst& mc, cons
 // warp each), so that 1/(2 gamma_g) and the moments' weight, an FP64 division of a
 // dozen instructions each, are taken once per block instead of by every warp.
 // Bound by the FP64 pipe (16 cycles per warp instruction; 84% busy).  N=16 G=40000
-// L=5: 188 us; 258 us with the offsets taken in FP64 per evaluation, bounds that
-// grow with the counts, and the divisions per thread.
+// L=5: 88 us; 258 us with the offsets taken in FP64 per evaluation, bounds that
+// grow with the counts, the divisions per thread and the level's density and log
+// in every update.
 __global__ void __launch_bounds__(256, 3) k_eps_f64(ModelConst mc, DevPtrs p, int seg_i) {
   __shared__ double s_hg[32], s_inv_k;
   __shared__ float s_hgf[32];
@@ -588,8 +589,8 @@ __device__ __forceinline__ void gb_gene_f64(const ModelConst& mc, const DevPtrs&
 // Steps 2 and 5: one thread per gene, after the eps kernel of this sweep and the
 // hyperparameter kernel of the previous one.  At most 168 registers, so that all
 // 1250 one-warp blocks of G=40000 are resident at once (at 248 eight fit an SM,
-// 1216 in all, and 34 ran alone).  N=16 G=40000 L=5: 118 us, FP64 pipe 72% busy; 301
-// us before the filter's bounds were freed of the counts.
+// 1216 in all, and 34 ran alone).  N=16 G=40000 L=5: 92 us; 301 us before the filter's
+// bounds were freed of the counts and the level taken only when needed.
 __global__ void __launch_bounds__(128, 3) k_gb_f64(ModelConst mc, DevPtrs p, int seg_i) {
   // shared: mu[N][B], beta[L][B], partials[kNumPart][B] (values indexed by a runtime
   // l live here rather than in local memory), then the reduction scratch
@@ -634,7 +635,7 @@ __global__ void __launch_bounds__(128, 3) k_gb_f64(ModelConst mc, DevPtrs p, int
 // instead of 157, and a few blocks share an SM, so that the one's serial gene
 // phase runs beside the other's eps phase.  Bound by the FP64 pipe.  One sweep of
 // N=16 G=20011 L=5: 659 us with one thread per gene making its 16 eps updates in a
-// row in FP64, 290 us so.
+// row in FP64, 205 us so.
 constexpr int kSweepWarps = 4, kSweepCluster = 4;
 
 __global__ void __cluster_dims__(kSweepCluster, 1, 1) __launch_bounds__(32 * kSweepWarps, 3)
