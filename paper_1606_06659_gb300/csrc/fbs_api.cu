@@ -89,7 +89,7 @@ Layout make_layout(int N, int G, int L, int nblk, long long trace_cap, int trace
 
 // FP32 form: per-gene state in FP32, four FP32 moment planes per parameter.
 struct LayoutF32 {
-  size_t y, T, eps, w_eps, waux_eps, mom_eps, mu, beta, w_beta, waux_beta, mom_beta, gam, mom_gam;
+  size_t y, T, asinh_T, eps, w_eps, waux_eps, mom_eps, mu, beta, w_beta, waux_beta, mom_beta, gam, mom_gam;
   size_t partial, hyp, trace_phi, trace_beta, counters, pinv, gsync, total;
 };
 
@@ -104,6 +104,7 @@ LayoutF32 make_layout_f32(int N, int G, int L, int nblk, long long trace_cap, in
   const size_t NG = (size_t)N * G, LG = (size_t)L * G, P = 2 * (size_t)L + 2;
   o.y = take(NG * sizeof(int32_t));
   o.T = take(LG * 8);
+  o.asinh_T = take(LG * 4);
   o.eps = take(NG * 4);
   o.w_eps = take(NG * 4);
   o.waux_eps = take(NG * 4);
@@ -305,6 +306,7 @@ DevPtrsF32 carve_f32_ptrs(char* base, const LayoutF32& o32, int trace_beta) {
   f.tc_polls = kTcWaitPolls;
   f.y = (const int32_t*)(base + o32.y);
   f.T = (const double*)(base + o32.T);
+  f.asinh_T = (float*)(base + o32.asinh_T);
   f.eps = (float*)(base + o32.eps);
   f.w_eps = (float*)(base + o32.w_eps);
   f.waux_eps = (float*)(base + o32.waux_eps);
@@ -618,9 +620,12 @@ int build_model(const int32_t* y, int N, int G, const double* X, int L, const do
     }
     mc.ncls[l] = nc;
   }
+  for (int l = 0; l < L; ++l)
+    mc.ncl[l] = (uint8_t)order_runs(N, kMaxCls, [&](int n) { return (int)mc.cls[l][n]; },
+                                    mc.cord[l], mc.cinfo[l]);
   // distinct rows of X, for the FP32 beta columns' per-pattern rate sums
   {
-    int rep[kMaxPat];
+    int rep[kMaxPat], pat[kMaxN];
     mc.npat = 0;
     for (int n = 0; n < N && mc.npat <= kMaxPat; ++n) {
       int r = 0;
@@ -632,11 +637,14 @@ int build_model(const int32_t* y, int N, int G, const double* X, int L, const do
         }
         rep[mc.npat++] = n;
       }
-      mc.pat[n] = (int8_t)r;
+      pat[n] = r;
     }
-    for (int l = 0; l < kMaxL; ++l)
-      for (int r = 0; r < kMaxPat; ++r)
-        mc.pcls[l][r] = (l < L && r < mc.npat && mc.npat <= kMaxPat) ? mc.cls[l][rep[r]] : -1;
+    if (mc.npat <= kMaxPat) {
+      order_runs(N, mc.npat, [&](int n) { return pat[n]; }, mc.pord, mc.pinfo);
+      for (int l = 0; l < L; ++l)
+        for (int r = 0; r < mc.npat; ++r)
+          if (mc.cls[l][rep[r]] >= 0) mc.pmask[l][mc.cls[l][rep[r]]] |= (uint8_t)(1u << r);
+    }
   }
   if (!pseudo_inverse(X, N, L, pinv)) return fail(FBS_E_ARG, "X^T X is singular");
   return FBS_OK;
@@ -747,7 +755,7 @@ int fbs_init(fbs_handle** out, const int32_t* y, int N, int G, int gene_major, c
     d_pinv = (double*)(base + o32.pinv);
     h->stage = (char*)f.mu;
     h->stage_cap = std::max((size_t)N * G * 4, kPackBytes);
-    if ((e = prepare_gene_kernel_f32(N, h->block)) != cudaSuccess)
+    if ((e = prepare_gene_kernel_f32(mc, h->block)) != cudaSuccess)
       return bail(FBS_E_CUDA, std::string("kernel attribute: ") + cudaGetErrorString(e));
   } else {
     h->p = carve(base, h->lay, mc.trace_beta);
@@ -1894,8 +1902,8 @@ struct fbs_batch {
   int* d_nblk = nullptr;         // [C] gamma/beta blocks per dataset
   int4* d_eps_tab = nullptr;
   int2* d_gb_tab = nullptr;
-  int n_eps = 0, n_gb = 0, eps_block = 256, gb_block = 128, max_N = 0, seg = 100;
-  size_t eps_cap = 0, gb_cap = 0;
+  int n_eps = 0, n_gb = 0, eps_block = 256, gb_block = 128, seg = 100;
+  size_t eps_cap = 0, gb_cap = 0, gb_smem = 0;
   cudaStream_t user = nullptr, s = nullptr, s2 = nullptr;
   cudaEvent_t ev_in = nullptr, ev_out = nullptr, ev_g = nullptr, ev_h = nullptr;
   cudaGraphExec_t exec = nullptr;
@@ -1956,7 +1964,9 @@ int batch_tables(fbs_batch* b, int eps_block, int gb_block) {
   FBS_CUDA(cudaMemcpyAsync(b->d_nblk, nblk.data(), nblk.size() * sizeof(int),
                            cudaMemcpyHostToDevice, b->s));
   FBS_CUDA(cudaStreamSynchronize(b->s));
-  FBS_CUDA(prepare_batch_kernels(b->max_N, gb_block));
+  b->gb_smem = 0;
+  for (const ModelConst& mc : b->mcs) b->gb_smem = std::max(b->gb_smem, gb_smem_f32(mc, gb_block, false));
+  FBS_CUDA(prepare_batch_kernels(b->gb_smem));
   b->n_eps = (int)et.size();
   b->n_gb = (int)gt.size();
   b->eps_block = eps_block;
@@ -1974,7 +1984,7 @@ cudaError_t batch_sweeps_direct(fbs_batch* b, int64_t n_iter) {
   for (int64_t i = 0; i < n_iter && e == cudaSuccess; ++i) {
     e = launch_eps_f32_batch(b->d_mc, b->d_pf, b->d_eps_tab, b->n_eps, b->eps_block, (int)i, b->s);
     if (e == cudaSuccess)
-      e = launch_gb_f32_batch(b->d_mc, b->d_pf, b->d_gb_tab, b->n_gb, b->gb_block, b->max_N,
+      e = launch_gb_f32_batch(b->d_mc, b->d_pf, b->d_gb_tab, b->n_gb, b->gb_block, b->gb_smem,
                               (int)i, b->s);
     if (e == cudaSuccess) e = launch_hyper_batch(b->d_mc, b->d_pf, b->d_nblk, b->C, b->s);
     if (e == cudaSuccess && b->three_level)
@@ -1990,7 +2000,7 @@ cudaError_t batch_capture(fbs_batch* b) {
     e = launch_eps_f32_batch(b->d_mc, b->d_pf, b->d_eps_tab, b->n_eps, b->eps_block, i, b->s);
     if (e != cudaSuccess) return e;
     if (i > 0 && (e = cudaStreamWaitEvent(b->s, b->ev_h, 0)) != cudaSuccess) return e;
-    e = launch_gb_f32_batch(b->d_mc, b->d_pf, b->d_gb_tab, b->n_gb, b->gb_block, b->max_N, i,
+    e = launch_gb_f32_batch(b->d_mc, b->d_pf, b->d_gb_tab, b->n_gb, b->gb_block, b->gb_smem, i,
                             b->s);
     if (e != cudaSuccess) return e;
     if ((e = cudaEventRecord(b->ev_g, b->s)) != cudaSuccess) return e;
@@ -2052,7 +2062,6 @@ int fbs_batch_init(fbs_batch** out, int C, const fbs_dataset* sets, const fbs_op
     integral[c] = integ;
     b->G[c] = ds.G;
     b->N[c] = ds.N;
-    b->max_N = std::max(b->max_N, ds.N);
     lay[c] = make_layout_f32(ds.N, ds.G, ds.L, (ds.G + 31) / 32, o->trace_cap,
                              b->mcs[c].trace_beta);
     off[c] = total;
@@ -2082,8 +2091,6 @@ int fbs_batch_init(fbs_batch** out, int C, const fbs_dataset* sets, const fbs_op
                 std::string("cudaMalloc: ") + cudaGetErrorString(e));
   if ((e = cudaEventRecord(b->ev_in, b->user)) != cudaSuccess ||
       (e = cudaStreamWaitEvent(b->s, b->ev_in, 0)) != cudaSuccess)
-    return bail(FBS_E_CUDA, cudaGetErrorString(e));
-  if ((e = prepare_gene_kernel_f32(b->max_N, 128)) != cudaSuccess)
     return bail(FBS_E_CUDA, cudaGetErrorString(e));
   for (int c = 0; c < C; ++c) {
     const fbs_dataset& ds = sets[c];

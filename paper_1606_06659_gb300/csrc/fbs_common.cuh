@@ -50,6 +50,10 @@ constexpr int kMaxOut = FBS_MAX_L + FBS_MAX_L * (FBS_MAX_L + 1) / 2;
 // Class of a non-zero value of one column of X: +1, -1 or any other value.
 enum : int8_t { kClsPlus = 1, kClsMinus = 2, kClsOther = 0 };
 
+// Marks of a sample in an order by runs (classes, patterns): the run begins, ends
+// there; its number from bit kRunShift on.
+enum : unsigned { kRunFirst = 1u, kRunLast = 2u, kRunShift = 2u };
+
 // Model constants, passed to every kernel by value (kernel-parameter space).
 struct ModelConst {
   int N, G, L, P;
@@ -73,12 +77,20 @@ struct ModelConst {
   float hf[kMaxN];
   float Xf[kMaxN * kMaxL];
   float cvalf[kMaxL][kMaxCls];
-  // Distinct rows of X (patterns): pat[n] = pattern of sample n, pcls[l][r] =
-  // class of pattern r in column l (-1 for a zero); npat = kMaxPat + 1 when X
-  // has more distinct rows (the FP32 beta columns then sum over samples).
+  // The samples of column l in the order of their classes (the ncl[l] with a
+  // non-zero value), and for each whether its class begins or ends there and
+  // which it is (kRunFirst, kRunLast, class << kRunShift).
+  uint8_t ncl[kMaxL];
+  uint8_t cord[kMaxL][kMaxN];
+  uint8_t cinfo[kMaxL][kMaxN];
+  // Distinct rows of X (patterns): all samples in the order of their patterns, with
+  // the same marks; bit r of pmask[l][j]: pattern r has class j in column l.
+  // npat = kMaxPat + 1 when X has more distinct rows (the FP32 beta columns then sum
+  // over samples).
   int npat;
-  int8_t pat[kMaxN];
-  int8_t pcls[kMaxL][kMaxPat];
+  uint8_t pord[kMaxN];
+  uint8_t pinfo[kMaxN];
+  uint8_t pmask[kMaxL][kMaxCls];
 };
 
 // Propositions of the contrast probabilities, in device memory: proposition q
@@ -162,6 +174,7 @@ struct DevPtrs {
 struct DevPtrsF32 {
   const int32_t* y;   // [N][G]
   const double* T;    // [L][G] (exact count sums, kept for fbs_count_sums)
+  float* asinh_T;     // [L][G] their asinh, a feature of the learned proposal
   float* eps;         // [N][G]
   float* w_eps;
   float* waux_eps;

@@ -20,6 +20,8 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "fbs_common.cuh"
 #include "fbs_kernels.h"
 #include "fbs_rng.cuh"
@@ -32,22 +34,28 @@ namespace fbs {
 
 // The uniforms of one random variable in the FP32 form: uniform k is word k%4 of
 // Philox block k/4, as ((w >> 9) + 1/2) / 2^23 (exact in FP32, inside (0,1)).
-struct Rng4 {
+//
+// OL: the Philox rounds as a call.  The gamma/beta kernels draw at a dozen places,
+// and with two warps per scheduler they wait for instructions a quarter of the
+// time: one copy of the rounds stays in the instruction cache.  The eps kernel,
+// which issues in most cycles, has them inline.
+static __device__ __noinline__ uint4 philox_ol(uint4 c, uint32_t k0, uint32_t k1) {
+  return philox4x32_10(c, k0, k1);
+}
+
+template <bool OL>
+struct Rng4T {
   uint32_t key0, key1, index, sblk, iter, chain;
   uint32_t cached;
   uint4 w;
 
-  __device__ __forceinline__ Rng4(uint32_t seed_lo, uint32_t seed_hi, uint32_t chain_,
+  __device__ __forceinline__ Rng4T(uint32_t seed_lo, uint32_t seed_hi, uint32_t chain_,
                                   uint32_t stream, uint32_t index_, uint32_t iter_)
       : key0(seed_lo), key1(seed_hi), index(index_), sblk(stream << 24), iter(iter_),
         chain(chain_), cached(0xFFFFFFFFu), w(make_uint4(0, 0, 0, 0)) {}
 
   __device__ __forceinline__ float u(uint32_t k) {
-    const uint32_t blk = k >> 2;
-    if (blk != cached) {
-      w = philox4x32_10(make_uint4(index, sblk | blk, iter, chain), key0, key1);
-      cached = blk;
-    }
+    block(k >> 2);
     const uint32_t j = k & 3u;
     const uint32_t x = j == 0 ? w.x : (j == 1 ? w.y : (j == 2 ? w.z : w.w));
     return word(x);
@@ -61,27 +69,31 @@ struct Rng4 {
   // Philox block blk (uniforms 4 blk .. 4 blk + 3), cached.
   __device__ __forceinline__ uint4 block(uint32_t blk) {
     if (blk != cached) {
-      w = philox4x32_10(make_uint4(index, sblk | blk, iter, chain), key0, key1);
+      const uint4 c = make_uint4(index, sblk | blk, iter, chain);
+      w = OL ? philox_ol(c, key0, key1) : philox4x32_10(c, key0, key1);
       cached = blk;
     }
     return w;
   }
 };
+using Rng4 = Rng4T<false>;
+using Rng4OL = Rng4T<true>;
 
-__device__ __forceinline__ float normal_bm_f(Rng4& r, uint32_t k0) {
-  const float u1 = r.u(k0), u2 = r.u(k0 + 1);
+__device__ __forceinline__ float normal_bm_f(float u1, float u2) {
   return sqrtf(-2.0f * __logf(u1)) * __cosf(6.2831853071795865f * u2);
 }
 
 // Gamma(shape, 1), Marsaglia & Tsang (2000), uniform layout as in the FP64 form.
-__device__ __forceinline__ float gamma_mt_f(float shape, Rng4& r, uint32_t k0, bool* capped) {
+template <class R>
+__device__ __forceinline__ float gamma_mt_f(float shape, R& r, uint32_t k0, bool* capped) {
   const float alpha = shape < 1.0f ? shape + 1.0f : shape;
   const float dd = alpha - (1.0f / 3.0f);
   const float cc = rsqrtf(9.0f * dd);
   float boost = 1.0f;
   if (shape < 1.0f) boost = __powf(r.u(k0 + 3), 1.0f / shape);
   for (uint32_t j = 0; j < (uint32_t)kGammaAttempts; ++j) {
-    const float x = normal_bm_f(r, k0 + 4 * j);
+    const float u1 = r.u(k0 + 4 * j), u2 = r.u(k0 + 4 * j + 1);
+    const float x = normal_bm_f(u1, u2);
     float v = 1.0f + cc * x;
     if (v <= 0.0f) continue;
     v = v * v * v;
@@ -139,9 +151,9 @@ struct SliceResultF {
 
 // Algorithm 2, steps 1-6, on Delta (Delta(x0) = 0): level log U_0, interval from
 // U_1, K_L from U_2, the j-th shrinkage proposal from U_{3+j}.
-template <class F>
+template <class F, class R>
 __device__ __forceinline__ SliceResultF slice_update_f(float x0, float aux0, float w, const F& f,
-                                                       Rng4& r, int K, int shrink_max) {
+                                                       R& r, int K, int shrink_max) {
   SliceResultF res;
   res.evals = 0;
   res.nonfinite = !(isfinite(x0) && isfinite(aux0));
@@ -203,11 +215,23 @@ __device__ __forceinline__ void tune_width_f(float& w, float& waux, long long it
   }
 }
 
-// Welford update of a Kahan-compensated FP32 pair (m, c) representing m - c.
-__device__ __forceinline__ void welford_kahan(float* base, size_t plane, size_t e, float x,
-                                              float inv_k) {
-  float m = base[e], c = base[plane + e];
-  float q = base[2 * plane + e], cq = base[3 * plane + e];
+// Welford update of a Kahan-compensated FP32 pair (m, c) representing m - c, of the
+// mean and the mean square: the four planes' values v of one element.
+struct KahanMoments {
+  float v[4];
+  __device__ __forceinline__ void load(const float* base, size_t plane, size_t e) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = base[i * plane + e];
+  }
+  __device__ __forceinline__ void store(float* base, size_t plane, size_t e) const {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) base[i * plane + e] = v[i];
+  }
+  __device__ __forceinline__ void update(float x, float inv_k);
+};
+
+__device__ __forceinline__ void KahanMoments::update(float x, float inv_k) {
+  float &m = v[0], &c = v[1], &q = v[2], &cq = v[3];
   {
     const float inc = (x - (m - c)) * inv_k;
     const float y = inc - c;
@@ -222,10 +246,14 @@ __device__ __forceinline__ void welford_kahan(float* base, size_t plane, size_t 
     cq = __fsub_rn(__fsub_rn(t, q), y);
     q = t;
   }
-  base[e] = m;
-  base[plane + e] = c;
-  base[2 * plane + e] = q;
-  base[3 * plane + e] = cq;
+}
+
+__device__ __forceinline__ void welford_kahan(float* base, size_t plane, size_t e, float x,
+                                              float inv_k) {
+  KahanMoments m;
+  m.load(base, plane, e);
+  m.update(x, inv_k);
+  m.store(base, plane, e);
 }
 
 // Error-free FP32 pair addition (Knuth's TwoSum).
@@ -342,77 +370,98 @@ __device__ __forceinline__ int move_kind(const DevPtrsF32& p, int g, long long i
 // genes whose conditional is close to the prior (very large gamma_g), where the
 // network, trained mostly on typical genes, extrapolates poorly.  Either way
 // the proposal depends only on quantities the move keeps.
-// The network's outputs are read from prop[k pstride + pidx].  Returns true
-// when accepted.
+// The network's outputs are read from prop[k pstride + pidx]; es holds the gene's
+// eps ([N][B], changed in place when accepted).  Returns true when accepted.
 constexpr int kTDof = 8;
+constexpr int kGbBatch = 16;  // samples whose rate, count and eps are in flight at a time
 
-__device__ __forceinline__ bool mh_move_f32(const ModelConst& mc, const DevPtrsF32& p, int g,
-                                            uint32_t it32, float* bs, int B, int tid,
-                                            const Hyper* hy, float hg, int kind,
-                                            const float* prop, size_t pstride, int pidx) {
-  const int G = mc.G, N = mc.N, L = mc.L;
-  float mu[kMaxL], C[kMaxL][kMaxL], xi[kMaxL], bn[kMaxL], d[kMaxL];
-#pragma unroll
-  for (int i = 0; i < kMaxL; ++i) {
-    mu[i] = 0.0f;
-#pragma unroll
-    for (int j = 0; j < kMaxL; ++j) C[i][j] = 0.0f;
+// The hyperparameters of a gamma/beta launch in FP32, once per block: the
+// conversions run on the FP64 pipe and every thread used to make them per column.
+struct GbHyper {
+  float th[kMaxL], s2[kMaxL], hs[kMaxL];  // theta_l, sigma_l^2, 1/(2 sigma_l^2)
+  float nu, tau, inv_k;                   // inv_k: weight of the draw in the moments
+};
+
+__device__ __forceinline__ void gb_hyper_load(const ModelConst& mc, const Hyper* hy, bool mom,
+                                              int tid, GbHyper* u) {
+  if (tid < mc.L) {
+    const float s2 = (float)hy->phi[2 + mc.L + tid];
+    u->th[tid] = (float)hy->phi[2 + tid];
+    u->s2[tid] = s2;
+    u->hs[tid] = 0.5f / s2;
+  } else if (tid == kMaxL) {
+    u->nu = (float)hy->phi[0];
+    u->tau = (float)hy->phi[1];
+    u->inv_k = mom ? 1.0f / (float)(hy->n_mom + 1) : 0.0f;
   }
-  int k = 2 * L;
+}
+
+template <int L>
+__device__ __forceinline__ bool mh_move_l(const ModelConst& mc, int g, uint32_t it32, float* bs,
+                                          float* es, int B, int tid, const GbHyper& u_, float hg,
+                                          int kind, const float* prop, size_t pstride, int pidx) {
+  const int N = mc.N;
+  float mu[L], C[L][L], xi[L], bn[L], d[L];
 #pragma unroll
-  for (int i = 0; i < kMaxL; ++i) {
-    if (i < L) {
-      if (kind == kMoveNet) {
-        mu[i] = prop[(size_t)i * pstride + pidx];
-        C[i][i] = expf(prop[(size_t)(L + i) * pstride + pidx]);
+  for (int i = 0; i < L; ++i) {
+    mu[i] = u_.th[i];  // the prior's centre and scales
 #pragma unroll
-        for (int j = 0; j < kMaxL; ++j)
-          if (j < i) C[i][j] = prop[(size_t)(k++) * pstride + pidx];
-      } else {  // the prior's centre and scales
-        mu[i] = (float)hy->phi[2 + i];
-        C[i][i] = sqrtf((float)hy->phi[2 + L + i]);
-      }
+    for (int j = 0; j < L; ++j) C[i][j] = 0.0f;
+    C[i][i] = sqrtf(u_.s2[i]);
+  }
+  if (kind == kMoveNet) {
+    int k = 2 * L;
+#pragma unroll
+    for (int i = 0; i < L; ++i) {
+      mu[i] = prop[(size_t)i * pstride + pidx];
+      C[i][i] = expf(prop[(size_t)(L + i) * pstride + pidx]);
+#pragma unroll
+      for (int j = 0; j < i; ++j) C[i][j] = prop[(size_t)(k++) * pstride + pidx];
     }
   }
-  Rng4 r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamMH, (uint32_t)g, it32);
+  // the 2L + 5 uniforms, block by block
+  constexpr int kU = 2 * L + 5, kBlk = (kU + 3) / 4;
+  float un[4 * kBlk];
+  Rng4OL r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamMH, (uint32_t)g, it32);
+#pragma unroll
+  for (int b = 0; b < kBlk; ++b) {
+    const uint4 q = r.block((uint32_t)b);
+    un[4 * b] = Rng4OL::word(q.x);
+    un[4 * b + 1] = Rng4OL::word(q.y);
+    un[4 * b + 2] = Rng4OL::word(q.z);
+    un[4 * b + 3] = Rng4OL::word(q.w);
+  }
   float lp = 0.0f;  // log prior ratio of beta
   float xx = 0.0f;  // |xi|^2
 #pragma unroll
-  for (int i = 0; i < kMaxL; ++i) {
-    xi[i] = 0.0f;
-    if (i < L) xi[i] = normal_bm_f(r, 2 * i);
+  for (int i = 0; i < L; ++i) {
+    xi[i] = normal_bm_f(un[2 * i], un[2 * i + 1]);
     xx += xi[i] * xi[i];
   }
-  const float log_u = __logf(r.u(2u * (uint32_t)L));
-  const uint32_t kc = 2u * (uint32_t)L + 1u;
-  const float chi2 = -2.0f * (logf(r.u(kc)) + logf(r.u(kc + 1u)) + logf(r.u(kc + 2u)) +
-                              logf(r.u(kc + 3u)));
+  const float log_u = __logf(un[2 * L]);
+  const float chi2 = -2.0f * (logf(un[2 * L + 1]) + logf(un[2 * L + 2]) + logf(un[2 * L + 3]) +
+                              logf(un[2 * L + 4]));
   const float st = sqrtf((float)kTDof / chi2);
 #pragma unroll
-  for (int i = 0; i < kMaxL; ++i) {
+  for (int i = 0; i < L; ++i) {
     float v = 0.0f;
 #pragma unroll
-    for (int j = 0; j < kMaxL; ++j)
-      if (j <= i) v += C[i][j] * xi[j];
+    for (int j = 0; j <= i; ++j) v += C[i][j] * xi[j];
     v = mu[i] + st * v;
     bn[i] = v;
-    d[i] = i < L ? v - bs[i * B + tid] : 0.0f;
+    d[i] = v - bs[i * B + tid];
   }
-  float u[kMaxL];
+  float u[L];
   float uu = 0.0f;  // |C^-1 (beta - mu)|^2
 #pragma unroll
-  for (int i = 0; i < kMaxL; ++i) {
-    u[i] = 0.0f;
-    if (i < L) {
-      float v = bs[i * B + tid] - mu[i];
+  for (int i = 0; i < L; ++i) {
+    float v = bs[i * B + tid] - mu[i];
 #pragma unroll
-      for (int j = 0; j < kMaxL; ++j)
-        if (j < i) v -= C[i][j] * u[j];
-      u[i] = v / C[i][i];
-      uu += u[i] * u[i];
-      const float bt = bs[i * B + tid] - (float)hy->phi[2 + i];
-      lp -= d[i] * (d[i] + 2.0f * bt) * (0.5f / (float)hy->phi[2 + L + i]);
-    }
+    for (int j = 0; j < i; ++j) v -= C[i][j] * u[j];
+    u[i] = v / C[i][i];
+    uu += u[i] * u[i];
+    const float bt = bs[i * B + tid] - u_.th[i];
+    lp -= d[i] * (d[i] + 2.0f * bt) * u_.hs[i];
   }
   // log q(beta) - log q(beta*), with C^-1 (beta* - mu) = st xi
   const float inv_dof = 1.0f / (float)kTDof;
@@ -420,88 +469,119 @@ __device__ __forceinline__ bool mh_move_f32(const ModelConst& mc, const DevPtrsF
                    (log1pf(uu * inv_dof) - log1pf(st * st * xx * inv_dof));
   // eps prior ratio: sum_n [eps_n^2 - (eps_n - X_n d)^2] / (2 gamma)
   float se = 0.0f;
+#pragma unroll 4
   for (int n = 0; n < N; ++n) {
     float xd = 0.0f;
 #pragma unroll
-    for (int l = 0; l < kMaxL; ++l)
-      if (l < L) xd += mc.Xf[n * kMaxL + l] * d[l];
-    se += xd * (2.0f * p.eps[(size_t)n * G + g] - xd);
+    for (int l = 0; l < L; ++l) xd += mc.Xf[n * kMaxL + l] * d[l];
+    se += xd * (2.0f * es[n * B + tid] - xd);
   }
   const float la = se * hg + lp + lq;
   const bool acc = log_u < la;
   if (acc) {
+#pragma unroll 4
     for (int n = 0; n < N; ++n) {
       float xd = 0.0f;
 #pragma unroll
-      for (int l = 0; l < kMaxL; ++l)
-        if (l < L) xd += mc.Xf[n * kMaxL + l] * d[l];
-      p.eps[(size_t)n * G + g] -= xd;
+      for (int l = 0; l < L; ++l) xd += mc.Xf[n * kMaxL + l] * d[l];
+      es[n * B + tid] -= xd;
     }
 #pragma unroll
-    for (int i = 0; i < kMaxL; ++i)
-      if (i < L) bs[i * B + tid] = bn[i];
+    for (int i = 0; i < L; ++i) bs[i * B + tid] = bn[i];
   }
   return acc;
 }
 
-// One slice update of beta_gl (step 5) for a column with NC value classes:
-// class sums Q_j (rates) and Y_j (counts) from the per-thread rows in shared
-// memory, the update, and the rates carried to the new value.
+// One copy of the move per number of columns: with L a constant its matrices are
+// registers and its 2L + 5 uniforms are drawn block by block (with L a variable
+// every uniform had its own copy of the generator behind a test: 17 000 cycles
+// per move at L = 5).
+__device__ __forceinline__ bool mh_move_f32(const ModelConst& mc, int g, uint32_t it32, float* bs,
+                                            float* es, int B, int tid, const GbHyper& u, float hg,
+                                            int kind, const float* prop, size_t pstride,
+                                            int pidx) {
+  static_assert(kMaxL == 8, "one case per number of columns");
+  switch (mc.L) {
+    case 1: return mh_move_l<1>(mc, g, it32, bs, es, B, tid, u, hg, kind, prop, pstride, pidx);
+    case 2: return mh_move_l<2>(mc, g, it32, bs, es, B, tid, u, hg, kind, prop, pstride, pidx);
+    case 3: return mh_move_l<3>(mc, g, it32, bs, es, B, tid, u, hg, kind, prop, pstride, pidx);
+    case 4: return mh_move_l<4>(mc, g, it32, bs, es, B, tid, u, hg, kind, prop, pstride, pidx);
+    case 5: return mh_move_l<5>(mc, g, it32, bs, es, B, tid, u, hg, kind, prop, pstride, pidx);
+    case 6: return mh_move_l<6>(mc, g, it32, bs, es, B, tid, u, hg, kind, prop, pstride, pidx);
+    case 7: return mh_move_l<7>(mc, g, it32, bs, es, B, tid, u, hg, kind, prop, pstride, pidx);
+    default: return mh_move_l<8>(mc, g, it32, bs, es, B, tid, u, hg, kind, prop, pstride, pidx);
+  }
+}
+
+// One slice update of beta_gl (step 5) for a column with NC value classes: class
+// sums Q_j (rates) and Y_j (counts), the update, and the rates carried to the new
+// value.  With use_pat the sums run over the row patterns' sums E and Yp, picked
+// by the classes' pattern masks (one constant each; a class number per pattern
+// made every addition wait for a constant load and a branch: 1500 cycles per
+// column); else over the class's samples in the per-thread rows in shared memory,
+// the samples in the order of their classes, each class's sums left in the
+// scratch rows qs [kMaxCls] and qs + kMaxCls rows as it ends.
 template <int NC>
 __device__ __forceinline__ void beta_column_f32(const ModelConst& mc, const DevPtrsF32& p, int l,
-                                                int g, float* mu, const float* ys, float* bs,
-                                                int B, int tid, const Hyper* hy, long long it,
-                                                uint32_t it32, long long burnin,
-                                                long long tune_start, unsigned& evals_b,
-                                                unsigned& caps, unsigned& nonfin, bool use_pat,
-                                                float* E, const float* Yp) {
-  const int G = mc.G, N = mc.N, L = mc.L;
-  const size_t e = (size_t)l * G + g;
-  const float theta = (float)hy->phi[2 + l];
-  const float sig2 = (float)hy->phi[2 + L + l];
+                                                int g, float* mu, const float* ys, float* qs,
+                                                float* bs, const float* ws, int B, int tid,
+                                                const GbHyper& u, long long it, uint32_t it32,
+                                                long long burnin, long long tune_start,
+                                                unsigned& evals_b, unsigned& caps,
+                                                unsigned& nonfin, bool use_pat, float* E,
+                                                const float* Yp) {
+  const int G = mc.G, L = mc.L;
   BetaDensityFT<NC> f;
   const float b_cur = bs[l * B + tid];
   f.b0 = b_cur;
-  f.bt = b_cur - theta;
-  f.hs = 0.5f / sig2;
+  f.bt = b_cur - u.th[l];
+  f.hs = u.hs[l];
   f.ncls = mc.ncls[l];
   float Y[NC];
+  unsigned mask[NC];
 #pragma unroll
   for (int j = 0; j < NC; ++j) {
     f.Q[j] = 0.0f;
     Y[j] = 0.0f;
     f.v[j] = mc.cvalf[l][j];
+    mask[j] = mc.pmask[l][j];
   }
+  const int nk = mc.ncl[l];
   if (use_pat) {
 #pragma unroll
-    for (int r = 0; r < kMaxPat; ++r)
-      if (r < mc.npat) {
-        const int c = mc.pcls[l][r];
+    for (int j = 0; j < NC; ++j)
 #pragma unroll
-        for (int j = 0; j < NC; ++j)
-          if (j == c) {
-            f.Q[j] += E[r];
-            Y[j] += Yp[r];
-          }
-      }
-  } else {
-    for (int n = 0; n < N; ++n) {
-      const int c = mc.cls[l][n];
-      const float m = mu[n * B + tid];
-      const float yv = ys[n * B + tid];
-#pragma unroll
-      for (int j = 0; j < NC; ++j)
-        if (j == c) {
-          f.Q[j] += m;
-          Y[j] += yv;
+      for (int r = 0; r < kMaxPat; ++r)
+        if (mask[j] & (1u << r)) {
+          f.Q[j] += E[r];
+          Y[j] += Yp[r];
         }
+  } else {
+    float am = 0.0f, ay = 0.0f;
+#pragma unroll 4
+    for (int k = 0; k < nk; ++k) {
+      const unsigned c = mc.cinfo[l][k];
+      const int n = mc.cord[l][k];
+      if (c & kRunFirst) am = ay = 0.0f;
+      am += mu[n * B + tid];
+      ay += ys[n * B + tid];
+      if (c & kRunLast) {
+        qs[(c >> kRunShift) * B + tid] = am;
+        qs[((c >> kRunShift) + kMaxCls) * B + tid] = ay;
+      }
     }
+#pragma unroll
+    for (int j = 0; j < NC; ++j)
+      if (j < f.ncls) {
+        f.Q[j] = qs[j * B + tid];
+        Y[j] = qs[(j + kMaxCls) * B + tid];
+      }
   }
 #pragma unroll
   for (int j = 0; j < NC; ++j) f.D[j] = Y[j] - f.Q[j];
-  Rng4 r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamBeta, (uint32_t)((size_t)g * L + l), it32);
+  Rng4OL r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamBeta, (uint32_t)((size_t)g * L + l), it32);
   const float x0 = b_cur;
-  float w = p.w_beta[e];
+  float w = ws[l * B + tid];
   SliceResultF s = slice_update_f(x0, 0.0f, w, f, r, mc.K, mc.shrink_max);
   evals_b += s.evals;
   caps += s.capped;
@@ -516,28 +596,21 @@ __device__ __forceinline__ void beta_column_f32(const ModelConst& mc, const DevP
     }
     if (use_pat) {
 #pragma unroll
-      for (int r = 0; r < kMaxPat; ++r)
-        if (r < mc.npat) {
-          const int c = mc.pcls[l][r];
-          float fc = 1.0f;
+      for (int j = 0; j < NC; ++j)
 #pragma unroll
-          for (int j = 0; j < NC; ++j)
-            if (j == c) fc = fac[j];
-          E[r] *= fc;
-        }
+        for (int r = 0; r < kMaxPat; ++r)
+          if (mask[j] & (1u << r)) E[r] *= fac[j];
     } else {
-      for (int n = 0; n < N; ++n) {
-        const int c = mc.cls[l][n];
-        float fc = 1.0f;
 #pragma unroll
-        for (int j = 0; j < NC; ++j)
-          if (j == c) fc = fac[j];
-        mu[n * B + tid] *= fc;
-      }
+      for (int j = 0; j < NC; ++j) qs[j * B + tid] = fac[j];
+#pragma unroll 4
+      for (int k = 0; k < nk; ++k)
+        mu[mc.cord[l][k] * B + tid] *= qs[(mc.cinfo[l][k] >> kRunShift) * B + tid];
     }
   }
   bs[l * B + tid] = s.x;
   if (it <= burnin) {
+    const size_t e = (size_t)l * G + g;
     float waux = p.waux_beta[e];
     tune_width_f(w, waux, it, s.x, x0, burnin, tune_start);
     p.w_beta[e] = w;
@@ -545,11 +618,41 @@ __device__ __forceinline__ void beta_column_f32(const ModelConst& mc, const DevP
   }
 }
 
-// Shared memory of the gamma/beta updates for blocks of B threads: mu, y [N][B],
-// beta [kMaxL][B], partials [kNumPart][B] (floats), then FP64 warp sums.
-__host__ __device__ inline size_t gb_smem_bytes_f32(int N, int B) {
-  return ((2 * (size_t)N + kMaxL + kNumPart) * B + 2) * sizeof(float) +
+// Shared memory of the gamma/beta updates for blocks of B threads, in rows of B
+// floats: the partials ps [kNumPart] (until they are written, the row patterns'
+// sums, or a column's class sums), beta and its widths [2 kMaxL], the running
+// moments of beta and gamma [4 (L + 1)], with the learned move eps [N], without
+// row patterns the rates mu and counts y [2 N]; then FP64 warp sums.  Threads only
+// touch their own column of the rows, but for the partials at the end.
+struct GbLayout {
+  int bs, ws, mom, es, mu, rows;
+};
+
+__host__ __device__ inline GbLayout gb_layout_f32(int N, int L, bool pat, bool move) {
+  GbLayout o;
+  o.bs = kNumPart;
+  o.ws = o.bs + kMaxL;
+  o.mom = o.ws + kMaxL;
+  o.es = o.mom + 4 * (L + 1);
+  o.mu = o.es + (move ? N : 0);
+  o.rows = o.mu + (pat ? 0 : 2 * N);
+  return o;
+}
+
+__host__ __device__ inline size_t gb_smem_bytes_f32(int N, int L, int B, bool pat, bool move) {
+  return ((size_t)gb_layout_f32(N, L, pat, move).rows * B + 2) * sizeof(float) +
          (size_t)(B / 32) * kNumPart * sizeof(double);
+}
+
+// A thread's own copy of one word into its shared memory, without a register and
+// without waiting (cp_wait).
+__device__ __forceinline__ void cp_word(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 // Steps 2 and 5 of Algorithm 1 in the FP32 form: one thread per gene.  The
@@ -560,104 +663,151 @@ __host__ __device__ inline size_t gb_smem_bytes_f32(int N, int B) {
 // net_ok: false when this block's network pass gave up (its genes then skip the
 // network's move); prop_s: the network's outputs of the block's genes in shared
 // memory ([K][B]), or nullptr (the move reads p.prop, [K][G]).
+//
+// Bound by latency (2 warps per scheduler at G = 40000), so everything a thread
+// reads is under way before it waits for any of it: the state and the moments as
+// asynchronous copies, the rates and counts 16 samples at a time, in the order of
+// the row patterns, whose sums they are added into on arrival.  N=16 G=40000 L=5:
+// 19.5 us (21.9 with a column's loads behind its stores, one wait each, and a
+// constant load and branch per addition).
+template <bool kMove>
 __device__ __forceinline__ void gb_f32_body(const ModelConst& mc, const DevPtrsF32& p, int seg_i,
                                             int blk, bool net_ok = true,
                                             const float* prop_s = nullptr) {
-  // shared: mu[N][B], y[N][B], beta[L][B], partials[kNumPart][B] (per-thread values
-  // indexed by a runtime l live here rather than in local memory); then FP64 warp sums
   extern __shared__ float smem_f[];
+  __shared__ GbHyper u;
   const int G = mc.G, N = mc.N, L = mc.L;
   const Hyper* hy = p.hyp;
   const long long it = hy->seg_it + seg_i + 1;
   const uint32_t it32 = (uint32_t)it;
   const long long burnin = hy->burnin, tune_start = hy->tune_start;
   const bool mom = it > burnin;
-  const float inv_k = mom ? 1.0f / (float)(hy->n_mom + 1) : 0.0f;
-  const float nu = (float)hy->phi[0], tau = (float)hy->phi[1];
   const bool trace_now = mom && mc.trace_beta && p.trace_beta != nullptr &&
                          ((it - burnin) % hy->thin == 0) && hy->trace_rows < hy->trace_cap;
   const long long trace_row = hy->trace_rows;
   const size_t LG = (size_t)L * G;
 
   const int B = blockDim.x;
-  float* mu = smem_f;
+  const bool use_pat = mc.npat <= kMaxPat;
+  const GbLayout lay = gb_layout_f32(N, L, use_pat, kMove);
+  float* ps = smem_f;
+  float* bs = smem_f + (size_t)lay.bs * B;
+  float* ws = smem_f + (size_t)lay.ws * B;
+  float* ms = smem_f + (size_t)lay.mom * B;
+  float* es = smem_f + (size_t)lay.es * B;
+  float* mu = smem_f + (size_t)lay.mu * B;
   float* ys = mu + (size_t)N * B;
-  float* bs = ys + (size_t)N * B;
-  float* ps = bs + (size_t)kMaxL * B;
   const int tid = threadIdx.x;
   const int g = blk * B + tid;
   const bool active = g < G;
-
-#pragma unroll
-  for (int i = 0; i < kNumPart; ++i) ps[i * B + tid] = 0.0f;
   unsigned evals_b = 0, caps = 0, gcaps = 0, nonfin = 0;
+  float ss = 0.0f;
+  float E[kMaxPat], Yp[kMaxPat];
 
   if (active) {
-    for (int l = 0; l < L; ++l) bs[l * B + tid] = p.beta[(size_t)l * G + g];
-    // 16 samples' loads in flight at a time (at N = 16 the whole gene; 8 or 4 lost
-    // 0.3-1.4 us of the kernel at N=16 G=40000)
-#pragma unroll 16
-    for (int n = 0; n < N; ++n) {
-      const size_t e = (size_t)n * G + g;
-      mu[n * B + tid] = p.mu[e];
-      ys[n * B + tid] = (float)p.y[e];
+    for (int l = 0; l < L; ++l) {
+      cp_word(bs + l * B + tid, p.beta + (size_t)l * G + g);
+      cp_word(ws + l * B + tid, p.w_beta + (size_t)l * G + g);
     }
-
-    // per-pattern sums of the rates and counts, in registers, when X has at most
-    // kMaxPat distinct rows (the move below keeps every rate)
-    const bool use_pat = mc.npat <= kMaxPat;
-    float E[kMaxPat], Yp[kMaxPat];
+    if (kMove)
+      for (int n = 0; n < N; ++n) cp_word(es + n * B + tid, p.eps + (size_t)n * G + g);
+    cp_commit();
+    float am = 0.0f, ay = 0.0f;  // sums of the pattern being read
+    for (int k0 = 0; k0 < N; k0 += kGbBatch) {
+      float m[kGbBatch], x[kGbBatch];
+      int32_t y[kGbBatch];
 #pragma unroll
-    for (int r = 0; r < kMaxPat; ++r) {
-      E[r] = 0.0f;
-      Yp[r] = 0.0f;
-    }
-    if (use_pat) {
-      for (int n = 0; n < N; ++n) {
-        const int pr = mc.pat[n];
-        const float m = mu[n * B + tid], yv = ys[n * B + tid];
+      for (int i = 0; i < kGbBatch; ++i)
+        if (k0 + i < N) {
+          // the samples in the patterns' order, the eps (whose squares are added
+          // in the samples' order) in theirs
+          const size_t e = (size_t)(use_pat ? mc.pord[k0 + i] : k0 + i) * G + g;
+          m[i] = p.mu[e];
+          y[i] = p.y[e];
+          if (!kMove) x[i] = p.eps[(size_t)(k0 + i) * G + g];
+        }
+      if (k0 == 0 && mom) {
+        for (int l = 0; l < L; ++l)
 #pragma unroll
-        for (int r = 0; r < kMaxPat; ++r)
-          if (r == pr) {
-            E[r] += m;
-            Yp[r] += yv;
+          for (int i = 0; i < 4; ++i)
+            cp_word(ms + (4 * l + i) * B + tid, p.mom_beta + i * LG + (size_t)l * G + g);
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+          cp_word(ms + (4 * L + i) * B + tid, p.mom_gam + (size_t)i * G + g);
+      }
+#pragma unroll
+      for (int i = 0; i < kGbBatch; ++i)
+        if (k0 + i < N) {
+          const float yf = (float)y[i];
+          if (!kMove) ss += x[i] * x[i];
+          if (use_pat) {
+            const unsigned c = mc.pinfo[k0 + i];
+            if (c & kRunFirst) am = ay = 0.0f;
+            am += m[i];
+            ay += yf;
+            if (c & kRunLast) {
+              ps[(c >> kRunShift) * B + tid] = am;
+              ps[((c >> kRunShift) + kMaxPat) * B + tid] = ay;
+            }
+          } else {
+            mu[(k0 + i) * B + tid] = m[i];
+            ys[(k0 + i) * B + tid] = yf;
           }
+        }
+    }
+    cp_commit();
+  }
+  gb_hyper_load(mc, hy, mom, tid, &u);
+  cp_wait<1>();     // beta, its widths and eps; the moments are still on their way
+  __syncthreads();  // the block's hyperparameters
+  const float inv_k = u.inv_k;
+  // the per-pattern sums of the rates and counts, in registers, when X has at most
+  // kMaxPat distinct rows (the move keeps every rate)
+#pragma unroll
+  for (int r = 0; r < kMaxPat; ++r) {
+    const bool on = active && use_pat && r < mc.npat;
+    E[r] = on ? ps[r * B + tid] : 0.0f;
+    Yp[r] = on ? ps[(r + kMaxPat) * B + tid] : 0.0f;
+  }
+
+  if (active) {
+    // ---- learned-proposal move (keeps every log-rate, so mu stays valid)
+    bool mh_gene = false;
+    if constexpr (kMove) {
+      int kind = move_kind(p, g, it);
+      if (kind == kMoveNet && !net_ok) kind = 0;
+      mh_gene = kind != 0;
+      if (mh_gene) {
+        const float hg = 0.5f / p.gam[g];
+        const size_t ci = (size_t)(kind - 1) * G + g;
+        const unsigned tried = p.mh_try[ci], accepted = p.mh_acc[ci];
+        const bool in_smem = prop_s != nullptr;
+        const bool acc = mh_move_f32(mc, g, it32, bs, es, B, tid, u, hg, kind,
+                                     in_smem ? prop_s : p.prop, in_smem ? (size_t)B : (size_t)G,
+                                     in_smem ? tid : g);
+        p.mh_try[ci] = tried + 1u;
+        if (acc) {
+          p.mh_acc[ci] = accepted + 1u;
+          for (int n = 0; n < N; ++n) p.eps[(size_t)n * G + g] = es[n * B + tid];
+        }
+      }
+#pragma unroll 8
+      for (int n = 0; n < N; ++n) {
+        const float x = es[n * B + tid];
+        ss += x * x;
       }
     }
 
-    // ---- learned-proposal move (keeps every log-rate, so mu stays valid)
-    int kind = p.prop != nullptr ? move_kind(p, g, it) : 0;
-    if (kind == kMoveNet && !net_ok) kind = 0;
-    const bool mh_gene = kind != 0;
-    if (mh_gene) {
-      const bool acc =
-          prop_s != nullptr
-              ? mh_move_f32(mc, p, g, it32, bs, B, tid, hy, 0.5f / p.gam[g], kind, prop_s,
-                            (size_t)B, tid)
-              : mh_move_f32(mc, p, g, it32, bs, B, tid, hy, 0.5f / p.gam[g], kind, p.prop,
-                            (size_t)G, g);
-      const size_t ci = (size_t)(kind - 1) * G + g;
-      p.mh_try[ci] += 1u;
-      p.mh_acc[ci] += acc ? 1u : 0u;
-    }
-
-    float ss = 0.0f;
-#pragma unroll 16
-    for (int n = 0; n < N; ++n) {
-      const float x = p.eps[(size_t)n * G + g];
-      ss += x * x;
-    }
-
     // ---- step 2: gamma_g ~ IG((N + nu)/2, (sum eps^2 + nu tau)/2)
+    float gam;
     {
-      Rng4 r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamGamma, (uint32_t)g, it32);
+      Rng4OL r(mc.seed_lo, mc.seed_hi, mc.chain, kStreamGamma, (uint32_t)g, it32);
       bool gcap = false;
-      const float shape = 0.5f * ((float)N + nu);
-      const float scale = 0.5f * (ss + nu * tau);
-      const float gam = scale / gamma_mt_f(shape, r, 0, &gcap);
+      const float shape = 0.5f * ((float)N + u.nu);
+      const float scale = 0.5f * (ss + u.nu * u.tau);
+      gam = scale / gamma_mt_f(shape, r, 0, &gcap);
       gcaps += gcap;
       p.gam[g] = gam;
-      if (mom) welford_kahan(p.mom_gam, (size_t)G, (size_t)g, gam, inv_k);
       ps[0 * B + tid] = __logf(gam);
       ps[1 * B + tid] = 1.0f / gam;
     }
@@ -667,34 +817,44 @@ __device__ __forceinline__ void gb_f32_body(const ModelConst& mc, const DevPtrsF
     for (int l = 0; l < L && !skip_slices; ++l) {
       switch (mc.ncls[l]) {
         case 1:
-          beta_column_f32<1>(mc, p, l, g, mu, ys, bs, B, tid, hy, it, it32, burnin, tune_start,
-                             evals_b, caps, nonfin, use_pat, E, Yp);
+          beta_column_f32<1>(mc, p, l, g, mu, ys, ps + 2 * B, bs, ws, B, tid, u, it, it32, burnin,
+                             tune_start, evals_b, caps, nonfin, use_pat, E, Yp);
           break;
         case 2:
-          beta_column_f32<2>(mc, p, l, g, mu, ys, bs, B, tid, hy, it, it32, burnin, tune_start,
-                             evals_b, caps, nonfin, use_pat, E, Yp);
+          beta_column_f32<2>(mc, p, l, g, mu, ys, ps + 2 * B, bs, ws, B, tid, u, it, it32, burnin,
+                             tune_start, evals_b, caps, nonfin, use_pat, E, Yp);
           break;
         case 3:
-          beta_column_f32<3>(mc, p, l, g, mu, ys, bs, B, tid, hy, it, it32, burnin, tune_start,
-                             evals_b, caps, nonfin, use_pat, E, Yp);
+          beta_column_f32<3>(mc, p, l, g, mu, ys, ps + 2 * B, bs, ws, B, tid, u, it, it32, burnin,
+                             tune_start, evals_b, caps, nonfin, use_pat, E, Yp);
           break;
         default:
-          beta_column_f32<kMaxCls>(mc, p, l, g, mu, ys, bs, B, tid, hy, it, it32, burnin,
-                                   tune_start, evals_b, caps, nonfin, use_pat, E, Yp);
+          beta_column_f32<kMaxCls>(mc, p, l, g, mu, ys, ps + 2 * B, bs, ws, B, tid, u, it, it32,
+                                   burnin, tune_start, evals_b, caps, nonfin, use_pat, E, Yp);
       }
     }
 
     // ---- the new beta_g: state, moments, trace, partial sums for steps 6-7
+    cp_wait<0>();
+    if (mom) {
+      for (int l = 0; l <= L; ++l) {  // the columns, then gamma
+        KahanMoments m;
+        m.load(ms + (size_t)4 * l * B, (size_t)B, (size_t)tid);
+        m.update(l < L ? bs[l * B + tid] : gam, inv_k);
+        if (l < L) m.store(p.mom_beta, LG, (size_t)l * G + g);
+        else m.store(p.mom_gam, (size_t)G, (size_t)g);
+      }
+    }
     for (int l = 0; l < L; ++l) {
       const size_t e = (size_t)l * G + g;
       const float b = bs[l * B + tid];
       p.beta[e] = b;
-      if (mom) welford_kahan(p.mom_beta, LG, e, b, inv_k);
       if (trace_now) p.trace_beta[(size_t)trace_row * LG + e] = (double)b;
-      const float dv = b - (float)hy->phi[2 + l];
+      const float dv = b - u.th[l];
       ps[(2 + l) * B + tid] = dv;
       ps[(2 + kMaxL + l) * B + tid] = dv * dv;
     }
+    for (int l = L; l < kMaxL; ++l) ps[(2 + l) * B + tid] = ps[(2 + kMaxL + l) * B + tid] = 0.0f;
     // contrast probabilities (§3.1), evaluated in FP32
     if (mom && p.con != nullptr) {
       const Contrasts* cs = p.con;
@@ -710,16 +870,21 @@ __device__ __forceinline__ void gb_f32_body(const ModelConst& mc, const DevPtrsF
     }
   }
 
+  if (!active) {
+#pragma unroll
+    for (int i = 0; i < kNumPart; ++i) ps[i * B + tid] = 0.0f;
+  }
+
   // ---- partial sums: error-free FP32 pair sums within the warp, FP64 beyond.
   // Lane i < kNumPart sums row i of the warp's 32 values (read in an order
   // rotated by i, so that the lanes hit distinct shared-memory banks).
   const int lane = tid & 31, warp = tid >> 5, nwarp = B >> 5;
-  double* red = reinterpret_cast<double*>(
-      smem_f + (((2 * (size_t)N + kMaxL + kNumPart) * B + 1) & ~(size_t)1));
+  double* red = reinterpret_cast<double*>(smem_f + (((size_t)lay.rows * B + 1) & ~(size_t)1));
   __syncwarp();
   if (lane < kNumPart) {
     const float* row = ps + (size_t)lane * B + warp * 32;
     float sm = 0.0f, c = 0.0f;
+#pragma unroll 8
     for (int j = 0; j < 32; ++j) {
       float t, e;
       two_sum(sm, row[(j + lane) & 31], t, e);
@@ -739,7 +904,15 @@ __device__ __forceinline__ void gb_f32_body(const ModelConst& mc, const DevPtrsF
 
 __global__ void __launch_bounds__(128) k_gb_f32(ModelConst mc, DevPtrsF32 p, int seg_i) {
   ktime_begin(p.ktime, p.ktime_n, 3 * seg_i + 1);
-  gb_f32_body(mc, p, seg_i, blockIdx.x);
+  gb_f32_body<false>(mc, p, seg_i, blockIdx.x);
+  ktime_end(p.ktime, p.ktime_n, 3 * seg_i + 1);
+}
+
+// With the learned move, the network's outputs read from global memory (block
+// sizes other than 128, or the network in a kernel of its own).
+__global__ void __launch_bounds__(128) k_gb_move_f32(ModelConst mc, DevPtrsF32 p, int seg_i) {
+  ktime_begin(p.ktime, p.ktime_n, 3 * seg_i + 1);
+  gb_f32_body<true>(mc, p, seg_i, blockIdx.x);
   ktime_end(p.ktime, p.ktime_n, 3 * seg_i + 1);
 }
 
@@ -751,7 +924,8 @@ __global__ void __launch_bounds__(128) k_gb_f32(ModelConst mc, DevPtrsF32 p, int
 __host__ __device__ inline size_t gb_net_stash_offset(int N, int L) {
   size_t off_a;
   tc_smem_layout(L, &off_a);
-  const size_t gb = gb_smem_bytes_f32(N, 128);
+  const size_t gb = std::max(gb_smem_bytes_f32(N, L, 128, true, true),
+                             gb_smem_bytes_f32(N, L, 128, false, true));
   return ((off_a > gb ? off_a : gb) + 15) & ~(size_t)15;
 }
 
@@ -778,7 +952,9 @@ __global__ void __launch_bounds__(128) k_gb_net_f32(ModelConst mc, DevPtrsF32 p,
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort;
     const TcShape t = tc_shape(mc.L);
+    __shared__ NetHyper nh;
     if (threadIdx.x == 0) s_abort = 0;
+    net_hyper_load(mc, p.hyp, (int)threadIdx.x, &nh);
     TcBlock c;
     tc_begin(c, bars, &tmem_slot, img, sm_tc, t.bytes, p.tc_polls);
     if (!c.w_ok) s_abort = 1;
@@ -786,7 +962,7 @@ __global__ void __launch_bounds__(128) k_gb_net_f32(ModelConst mc, DevPtrsF32 p,
     const int g = blockIdx.x * 128 + (int)threadIdx.x;
     prop_s = reinterpret_cast<float*>(sm_tc + gb_net_stash_offset(mc.N, mc.L));
     if (!s_abort)
-      tc_tile(c, mc, p, t, sm_tc, g, net_gene(p, g, mc.G), prop_s, 128, (int)threadIdx.x,
+      tc_tile(c, mc, p, nh, t, sm_tc, g, net_gene(p, g, mc.G), prop_s, 128, (int)threadIdx.x,
               &s_abort);
     __syncthreads();
     net_ok = s_abort == 0;
@@ -794,28 +970,34 @@ __global__ void __launch_bounds__(128) k_gb_net_f32(ModelConst mc, DevPtrsF32 p,
     fence_async_smem();
     __syncthreads();  // below the outputs, the shared memory is the gamma/beta updates' from here on
   }
-  gb_f32_body(mc, p, seg_i, blockIdx.x, net_ok, prop_s);
+  gb_f32_body<true>(mc, p, seg_i, blockIdx.x, net_ok, prop_s);
   ktime_end(p.ktime, p.ktime_n, 3 * seg_i + 1);
 }
 
 // The learned move alone, at the current state, for the genes that use it (every
 // gene when p.mh_all), with the random numbers of iteration `it`.
 __global__ void __launch_bounds__(128) k_mh_step_f32(ModelConst mc, DevPtrsF32 p, long long it) {
+  extern __shared__ float es[];  // [N][128]
   __shared__ float bs[kMaxL * 128];
+  __shared__ GbHyper u;
   const int B = blockDim.x, tid = threadIdx.x;
   const int g = blockIdx.x * B + tid;
+  gb_hyper_load(mc, p.hyp, false, tid, &u);
+  __syncthreads();
   if (g >= mc.G) return;
   const int kind = move_kind(p, g, it);
   if (kind == 0) return;
-  const int G = mc.G, L = mc.L;
+  const int G = mc.G, N = mc.N, L = mc.L;
   for (int l = 0; l < L; ++l) bs[l * B + tid] = p.beta[(size_t)l * G + g];
-  const bool acc = mh_move_f32(mc, p, g, (uint32_t)it, bs, B, tid, p.hyp, 0.5f / p.gam[g], kind,
+  for (int n = 0; n < N; ++n) es[n * B + tid] = p.eps[(size_t)n * G + g];
+  const bool acc = mh_move_f32(mc, g, (uint32_t)it, bs, es, B, tid, u, 0.5f / p.gam[g], kind,
                                p.prop, (size_t)G, g);
   const size_t ci = (size_t)(kind - 1) * G + g;
   p.mh_try[ci] += 1u;
   if (acc) {
     p.mh_acc[ci] += 1u;
     for (int l = 0; l < L; ++l) p.beta[(size_t)l * G + g] = bs[l * B + tid];
+    for (int n = 0; n < N; ++n) p.eps[(size_t)n * G + g] = es[n * B + tid];
   }
 }
 
@@ -903,7 +1085,7 @@ __global__ void __launch_bounds__(128, 4) k_sweeps_f32(ModelConst mc, DevPtrsF32
     }
     if (!grid_sync(gs, &p.hyp->flags, &s_ok)) return;
     for (int b = blockIdx.x; b < nblk; b += gridDim.x) {
-      gb_f32_body(mc, p, i, b);
+      gb_f32_body<false>(mc, p, i, b);
       __syncthreads();  // the next gene block reuses the shared memory
     }
     if (!grid_sync(gs, &p.hyp->flags, &s_ok)) return;
@@ -915,9 +1097,9 @@ cudaError_t launch_sweeps_f32(const ModelConst& mc, const DevPtrsF32& p, const D
                               int n_sweeps, void* gsync, cudaStream_t s, int* grid_out) {
   const int block = 128;
   const int nblk = (mc.G + block - 1) / block;
-  const size_t smem = gene_smem_bytes_f32(mc.N, block);
+  const size_t smem = gb_smem_f32(mc, block, false);
   cudaError_t e = cudaFuncSetAttribute(k_sweeps_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)gene_smem_bytes_f32(FBS_MAX_N, block));
+                                       (int)gb_smem_bytes_f32(FBS_MAX_N, FBS_MAX_L, block, false, false));
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -958,11 +1140,11 @@ __global__ void __launch_bounds__(256, 5) k_eps_f32_batch(const ModelConst* __re
   eps_f32_body(mcs[t.x], ps[t.x], seg_i, t.y, t.z * blockDim.x + threadIdx.x, t.w);
 }
 
-__global__ void __launch_bounds__(128) k_gb_f32_batch(const ModelConst* __restrict__ mcs,
+__global__ void __launch_bounds__(128, 4) k_gb_f32_batch(const ModelConst* __restrict__ mcs,
                                                       const DevPtrsF32* __restrict__ ps,
                                                       const int2* __restrict__ tab, int seg_i) {
   const int2 t = tab[blockIdx.x];  // dataset, gene block within the dataset
-  gb_f32_body(mcs[t.x], ps[t.x], seg_i, t.y);
+  gb_f32_body<false>(mcs[t.x], ps[t.x], seg_i, t.y);
 }
 
 // One block per dataset.
@@ -1051,8 +1233,7 @@ __global__ void k_set_run_batch(const DevPtrsF32* __restrict__ ps, int C, long l
   }
 }
 
-cudaError_t prepare_batch_kernels(int max_N, int gb_block) {
-  const size_t smem = gene_smem_bytes_f32(max_N, gb_block);
+cudaError_t prepare_batch_kernels(size_t smem) {
   if (smem > 48 * 1024)
     return cudaFuncSetAttribute(k_gb_f32_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)smem);
@@ -1066,8 +1247,8 @@ cudaError_t launch_eps_f32_batch(const ModelConst* mcs, const DevPtrsF32* ps, co
 }
 
 cudaError_t launch_gb_f32_batch(const ModelConst* mcs, const DevPtrsF32* ps, const int2* tab,
-                                int n_blocks, int block, int max_N, int seg_i, cudaStream_t s) {
-  k_gb_f32_batch<<<n_blocks, block, gene_smem_bytes_f32(max_N, block), s>>>(mcs, ps, tab, seg_i);
+                                int n_blocks, int block, size_t smem, int seg_i, cudaStream_t s) {
+  k_gb_f32_batch<<<n_blocks, block, smem, s>>>(mcs, ps, tab, seg_i);
   return cudaGetLastError();
 }
 
@@ -1116,6 +1297,7 @@ __global__ void k_init_genes_f32(ModelConst mc, DevPtrsF32 p, const int32_t* y_i
     }
     for (int l = 0; l < L; ++l) {
       const_cast<double*>(p.T)[(size_t)l * G + g] = T[l];
+      p.asinh_T[(size_t)l * G + g] = asinhf((float)T[l]);
       if (set_state) {
         double s = 0.0;
         for (int n = 0; n < N; ++n) s += pinv[l * kMaxN + n] * r[n];
@@ -1145,15 +1327,19 @@ __global__ void k_zero_moments_f32(ModelConst mc, DevPtrsF32 p) {
   }
 }
 
-cudaError_t prepare_gene_kernel_f32(int N, int block) {
-  const size_t smem = gene_smem_bytes_f32(N, block);
-  if (smem > 48 * 1024)
-    return cudaFuncSetAttribute(k_gb_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem);
-  return cudaSuccess;
+size_t gb_smem_f32(const ModelConst& mc, int block, bool move) {
+  return gb_smem_bytes_f32(mc.N, mc.L, block, mc.npat <= kMaxPat, move);
 }
 
-size_t gene_smem_bytes_f32(int N, int block) { return gb_smem_bytes_f32(N, block); }
+cudaError_t prepare_gene_kernel_f32(const ModelConst& mc, int block) {
+  const size_t smem = gb_smem_f32(mc, block, true);  // with the learned move or without
+  if (smem <= 48 * 1024) return cudaSuccess;
+  cudaError_t e = cudaFuncSetAttribute(k_gb_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)smem);
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(k_gb_move_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return e;
+}
 
 cudaError_t launch_eps_f32(const ModelConst& mc, const DevPtrsF32& p, int seg_i,
                            cudaStream_t s) {
@@ -1166,7 +1352,7 @@ cudaError_t launch_eps_f32(const ModelConst& mc, const DevPtrsF32& p, int seg_i,
 cudaError_t launch_gb_f32(const ModelConst& mc, const DevPtrsF32& p, int block, int seg_i,
                           cudaStream_t s, const void* img) {
   const int nblk = (mc.G + block - 1) / block;
-  size_t smem = gene_smem_bytes_f32(mc.N, block);
+  size_t smem = gb_smem_f32(mc, block, p.prop != nullptr);
   if (img != nullptr) {
     if (block != 128) return cudaErrorInvalidValue;  // one thread per gene of a 128-gene tile
     smem = gb_net_smem_bytes(mc.N, mc.L);
@@ -1180,6 +1366,7 @@ cudaError_t launch_gb_f32(const ModelConst& mc, const DevPtrsF32& p, int block, 
     if (e != cudaSuccess) return e;
   }
   if (img != nullptr) k_gb_net_f32<<<nblk, block, smem, s>>>(mc, p, seg_i, (const uint8_t*)img);
+  else if (p.prop != nullptr) k_gb_move_f32<<<nblk, block, smem, s>>>(mc, p, seg_i);
   else k_gb_f32<<<nblk, block, smem, s>>>(mc, p, seg_i);
   return cudaGetLastError();
 }
@@ -1187,7 +1374,8 @@ cudaError_t launch_gb_f32(const ModelConst& mc, const DevPtrsF32& p, int block, 
 cudaError_t launch_mh_step_f32(const ModelConst& mc, const DevPtrsF32& p, long long it,
                               cudaStream_t s) {
   const int block = 128;
-  k_mh_step_f32<<<(mc.G + block - 1) / block, block, 0, s>>>(mc, p, it);
+  k_mh_step_f32<<<(mc.G + block - 1) / block, block, (size_t)mc.N * block * sizeof(float), s>>>(
+      mc, p, it);
   return cudaGetLastError();
 }
 

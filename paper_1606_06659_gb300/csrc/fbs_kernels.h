@@ -12,6 +12,27 @@ namespace fbs {
 
 constexpr int kDefaultBlock = 128;
 
+// Puts the samples 0..N-1 whose run(n) is 0..runs-1 in the order of their runs:
+// their numbers, and the marks kRunFirst, kRunLast and run << kRunShift.  Returns
+// how many there are.
+template <class Run>
+inline int order_runs(int N, int runs, Run run, uint8_t* order, uint8_t* info) {
+  int k = 0;
+  for (int r = 0; r < runs; ++r) {
+    const int k0 = k;
+    for (int n = 0; n < N; ++n)
+      if (run(n) == r) {
+        order[k] = (uint8_t)n;
+        info[k++] = (uint8_t)(r << kRunShift);
+      }
+    if (k > k0) {
+      info[k0] |= kRunFirst;
+      info[k - 1] |= kRunLast;
+    }
+  }
+  return k;
+}
+
 cudaError_t prepare_gene_kernel(int N, int block);
 // Steps 1, 2 and 5 in one launch, the rates kept on chip; partial sums per 128 genes.
 cudaError_t launch_sweep_f64(const ModelConst& mc, const DevPtrs& p, cudaStream_t s);
@@ -30,8 +51,9 @@ cudaError_t launch_init_hyper(const ModelConst& mc, Hyper* hy, const double* bet
 cudaError_t launch_init_run(Hyper* hy, long long trace_cap, cudaStream_t s);
 
 // FP32 form (fbs_gene_f32.cu)
-size_t gene_smem_bytes_f32(int N, int block);
-cudaError_t prepare_gene_kernel_f32(int N, int block);
+// Shared memory of the gamma/beta kernel for one dataset's layout.
+size_t gb_smem_f32(const ModelConst& mc, int block, bool move);
+cudaError_t prepare_gene_kernel_f32(const ModelConst& mc, int block);
 cudaError_t launch_eps_f32(const ModelConst& mc, const DevPtrsF32& p, int seg_i, cudaStream_t s);
 // img: null, or the learned proposal's weight image, whose network the kernel
 // then evaluates for its own genes first (block must be 128)
@@ -126,11 +148,11 @@ size_t tc_image_bytes(int L);
 cudaError_t launch_pack_image(const float* params, void* img, int L, cudaStream_t s);
 
 // batched FP32 kernels (fbs_gene_f32.cu)
-cudaError_t prepare_batch_kernels(int max_N, int gb_block);
+cudaError_t prepare_batch_kernels(size_t gb_smem);
 cudaError_t launch_eps_f32_batch(const ModelConst* mcs, const DevPtrsF32* ps, const int4* tab,
                                  int n_blocks, int block, int seg_i, cudaStream_t s);
 cudaError_t launch_gb_f32_batch(const ModelConst* mcs, const DevPtrsF32* ps, const int2* tab,
-                                int n_blocks, int block, int max_N, int seg_i, cudaStream_t s);
+                                int n_blocks, int block, size_t smem, int seg_i, cudaStream_t s);
 cudaError_t launch_hyper_batch(const ModelConst* mcs, const DevPtrsF32* ps, const int* nblk,
                                int C, cudaStream_t s);
 cudaError_t launch_seg_begin_batch(const DevPtrsF32* ps, int C, cudaStream_t s);

@@ -98,14 +98,16 @@ __global__ void __launch_bounds__(kTcThreads) k_proposal_tc(ModelConst mc, DevPt
   __shared__ uint32_t tmem_slot;
   __shared__ int s_abort;
   const TcShape t = tc_shape(mc.L);
+  __shared__ NetHyper nh;
   if (threadIdx.x == 0) s_abort = 0;
+  net_hyper_load(mc, p.hyp, (int)threadIdx.x, &nh);
   TcBlock c;
   tc_begin(c, bars, &tmem_slot, img_g, sm, t.bytes, p.tc_polls);
   if (!c.w_ok) s_abort = 1;
   __syncthreads();
   for (int tile = blockIdx.x; tile < ntiles && !s_abort; tile += gridDim.x) {
     const int g = tile * 128 + (int)threadIdx.x;
-    if (!tc_tile(c, mc, p, t, sm, g, net_gene(p, g, mc.G), out, (size_t)mc.G, g, &s_abort))
+    if (!tc_tile(c, mc, p, nh, t, sm, g, net_gene(p, g, mc.G), out, (size_t)mc.G, g, &s_abort))
       break;
   }
   tc_end(c, s_abort != 0, &p.hyp->flags);
@@ -113,16 +115,37 @@ __global__ void __launch_bounds__(kTcThreads) k_proposal_tc(ModelConst mc, DevPt
 
 // Training pairs from the current state of every gene: features [M][F] and
 // beta [M][L] rows starting at `row`.
+template <int L>
+__device__ __forceinline__ void collect_gene(const ModelConst& mc, const DevPtrsF32& p,
+                                             const NetHyper& u, int g, float* __restrict__ feat,
+                                             float* __restrict__ beta, size_t r) {
+  constexpr int F = 4 * L + 1;
+  float f[F];
+  gene_features_l<L>(mc, p, u, g, f);
+#pragma unroll
+  for (int i = 0; i < F; ++i) feat[r * F + i] = f[i];
+#pragma unroll
+  for (int l = 0; l < L; ++l) beta[r * L + l] = p.beta[(size_t)l * mc.G + g];
+}
+
 __global__ void k_collect_f32(ModelConst mc, DevPtrsF32 p, float* __restrict__ feat,
                               float* __restrict__ beta, long long row) {
+  __shared__ NetHyper u;
+  net_hyper_load(mc, p.hyp, (int)threadIdx.x, &u);
+  __syncthreads();
   const int g = blockIdx.x * blockDim.x + threadIdx.x;
   if (g >= mc.G) return;
-  const int F = 4 * mc.L + 1, L = mc.L;
-  float f[kMaxFeat];
-  gene_features(mc, p, g, p.hyp, f);
   const size_t r = (size_t)(row + g);
-  for (int i = 0; i < F; ++i) feat[r * F + i] = f[i];
-  for (int l = 0; l < L; ++l) beta[r * L + l] = p.beta[(size_t)l * mc.G + g];
+  switch (mc.L) {
+    case 1: collect_gene<1>(mc, p, u, g, feat, beta, r); break;
+    case 2: collect_gene<2>(mc, p, u, g, feat, beta, r); break;
+    case 3: collect_gene<3>(mc, p, u, g, feat, beta, r); break;
+    case 4: collect_gene<4>(mc, p, u, g, feat, beta, r); break;
+    case 5: collect_gene<5>(mc, p, u, g, feat, beta, r); break;
+    case 6: collect_gene<6>(mc, p, u, g, feat, beta, r); break;
+    case 7: collect_gene<7>(mc, p, u, g, feat, beta, r); break;
+    default: collect_gene<8>(mc, p, u, g, feat, beta, r); break;
+  }
 }
 
 // ---------------------------------------------------------------- training
