@@ -1089,7 +1089,7 @@ __global__ void __launch_bounds__(128, 4) k_sweeps_f32(ModelConst mc, DevPtrsF32
       __syncthreads();  // the next gene block reuses the shared memory
     }
     if (!grid_sync(gs, &p.hyp->flags, &s_ok)) return;
-    if (blockIdx.x == 0) hyper_body(mc, hp.partial, hp.hyp, hp.trace_phi, hp.counters, nblk);
+    if (blockIdx.x == 0) hyper_body<128>(mc, hp.partial, hp.hyp, hp.trace_phi, hp.counters, nblk);
   }
 }
 
@@ -1153,7 +1153,7 @@ __global__ void __launch_bounds__(kHyperThreads) k_hyper_batch(const ModelConst*
                                                                const int* __restrict__ nblk) {
   const int c = blockIdx.x;
   const DevPtrsF32& p = ps[c];
-  hyper_body(mcs[c], p.partial, p.hyp, p.trace_phi, p.counters, nblk[c], p.psi);
+  hyper_body<kHyperThreads>(mcs[c], p.partial, p.hyp, p.trace_phi, p.counters, nblk[c], p.psi);
 }
 
 // Top level of the three-level model, one warp, after the datasets' hyper

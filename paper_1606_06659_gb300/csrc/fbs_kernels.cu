@@ -701,7 +701,7 @@ __global__ void __launch_bounds__(kHyperThreads) k_hyper(ModelConst mc, DevPtrs 
   // the sweep of the segment this launch completes (probe slot only)
   const int slot = p.ktime ? 3 * (int)(p.hyp->it - p.hyp->seg_it) + 2 : 0;
   ktime_begin(p.ktime, p.ktime_n, slot);
-  hyper_body(mc, p.partial, p.hyp, p.trace_phi, p.counters, nblk);
+  hyper_body<kHyperThreads>(mc, p.partial, p.hyp, p.trace_phi, p.counters, nblk);
   ktime_end(p.ktime, p.ktime_n, slot);
 }
 
