@@ -131,12 +131,35 @@ struct BetaDensityFT {
   __device__ __forceinline__ float operator()(float b, float* aux) const {
     const float d = b - b0;
     float s = 0.0f;
+    if constexpr (NC <= 3) {
 #pragma unroll
-    for (int j = 0; j < NC; ++j) {
-      if (NC < kMaxCls || j < ncls) {
+      for (int j = 0; j < NC; ++j) {
         const float z = v[j] * d;
         s += z * D[j] - Q[j] * em1mx(z);
       }
+    } else {
+      // with many classes the exponentials are worth a branch (N=22 G=9973 with an
+      // eight-level covariate: gamma/beta 21.2 -> 19.0 us; with two they are not)
+      float e[NC];
+      bool big = false;
+#pragma unroll
+      for (int j = 0; j < NC; ++j) {
+        e[j] = em1mx_series(v[j] * d);
+        big |= !(fabsf(v[j] * d) < 0.5f);
+      }
+      if (big) {
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+          const float z = v[j] * d, t = em1mx_direct(z);
+          e[j] = fabsf(z) < 0.5f ? e[j] : t;
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < NC; ++j)
+        if (j < ncls) {
+          const float z = v[j] * d;
+          s += z * D[j] - Q[j] * e[j];
+        }
     }
     *aux = d;
     return s - d * (d + 2.0f * bt) * hs;
@@ -398,8 +421,9 @@ __device__ __forceinline__ void gb_hyper_load(const ModelConst& mc, const Hyper*
 
 template <int L>
 __device__ __forceinline__ bool mh_move_l(const ModelConst& mc, int g, uint32_t it32, float* bs,
-                                          float* es, int B, int tid, const GbHyper& u_, float hg,
-                                          int kind, const float* prop, size_t pstride, int pidx) {
+                                          float* es, int B, int tid,
+                                          const GbHyper& u_, float hg, int kind,
+                                          const float* prop, size_t pstride, int pidx) {
   const int N = mc.N;
   float mu[L], C[L][L], xi[L], bn[L], d[L];
 #pragma unroll
@@ -468,24 +492,23 @@ __device__ __forceinline__ bool mh_move_l(const ModelConst& mc, int g, uint32_t 
   const float lq = -0.5f * (float)(kTDof + L) *
                    (log1pf(uu * inv_dof) - log1pf(st * st * xx * inv_dof));
   // eps prior ratio: sum_n [eps_n^2 - (eps_n - X_n d)^2] / (2 gamma)
-  float se = 0.0f;
-#pragma unroll 4
-  for (int n = 0; n < N; ++n) {
+  auto shift = [&](int n) {  // X_n d
     float xd = 0.0f;
 #pragma unroll
     for (int l = 0; l < L; ++l) xd += mc.Xf[n * kMaxL + l] * d[l];
+    return xd;
+  };
+  float se = 0.0f;
+#pragma unroll 4
+  for (int n = 0; n < N; ++n) {
+    const float xd = shift(n);
     se += xd * (2.0f * es[n * B + tid] - xd);
   }
   const float la = se * hg + lp + lq;
   const bool acc = log_u < la;
   if (acc) {
 #pragma unroll 4
-    for (int n = 0; n < N; ++n) {
-      float xd = 0.0f;
-#pragma unroll
-      for (int l = 0; l < L; ++l) xd += mc.Xf[n * kMaxL + l] * d[l];
-      es[n * B + tid] -= xd;
-    }
+    for (int n = 0; n < N; ++n) es[n * B + tid] -= shift(n);
 #pragma unroll
     for (int i = 0; i < L; ++i) bs[i * B + tid] = bn[i];
   }
@@ -497,9 +520,9 @@ __device__ __forceinline__ bool mh_move_l(const ModelConst& mc, int g, uint32_t 
 // every uniform had its own copy of the generator behind a test: 17 000 cycles
 // per move at L = 5).
 __device__ __forceinline__ bool mh_move_f32(const ModelConst& mc, int g, uint32_t it32, float* bs,
-                                            float* es, int B, int tid, const GbHyper& u, float hg,
-                                            int kind, const float* prop, size_t pstride,
-                                            int pidx) {
+                                            float* es, int B, int tid,
+                                            const GbHyper& u, float hg, int kind,
+                                            const float* prop, size_t pstride, int pidx) {
   static_assert(kMaxL == 8, "one case per number of columns");
   switch (mc.L) {
     case 1: return mh_move_l<1>(mc, g, it32, bs, es, B, tid, u, hg, kind, prop, pstride, pidx);
@@ -902,7 +925,9 @@ __device__ __forceinline__ void gb_f32_body(const ModelConst& mc, const DevPtrsF
   add_counters(p.counters, 0, evals_b, caps, gcaps, nonfin, &p.hyp->flags);
 }
 
-__global__ void __launch_bounds__(128) k_gb_f32(ModelConst mc, DevPtrsF32 p, int seg_i) {
+// At most 128 registers: four blocks per SM, which G = 200000 needs (80 against 90 us
+// at N = 32 with three).
+__global__ void __launch_bounds__(128, 4) k_gb_f32(ModelConst mc, DevPtrsF32 p, int seg_i) {
   ktime_begin(p.ktime, p.ktime_n, 3 * seg_i + 1);
   gb_f32_body<false>(mc, p, seg_i, blockIdx.x);
   ktime_end(p.ktime, p.ktime_n, 3 * seg_i + 1);
@@ -921,17 +946,16 @@ __global__ void __launch_bounds__(128) k_gb_move_f32(ModelConst mc, DevPtrsF32 p
 // arrays from offset 0, and
 // the network's outputs of the block's genes ([K][128] floats) at
 // gb_net_stash_offset, past both the weight image and those arrays.
-__host__ __device__ inline size_t gb_net_stash_offset(int N, int L) {
+__host__ __device__ inline size_t gb_net_stash_offset(const ModelConst& mc) {
   size_t off_a;
-  tc_smem_layout(L, &off_a);
-  const size_t gb = std::max(gb_smem_bytes_f32(N, L, 128, true, true),
-                             gb_smem_bytes_f32(N, L, 128, false, true));
+  tc_smem_layout(mc.L, &off_a);
+  const size_t gb = gb_smem_bytes_f32(mc.N, mc.L, 128, mc.npat <= kMaxPat, true);
   return ((off_a > gb ? off_a : gb) + 15) & ~(size_t)15;
 }
 
-size_t gb_net_smem_bytes(int N, int L) {
-  const size_t tc = tc_smem_layout(L, nullptr);
-  const size_t st = gb_net_stash_offset(N, L) + (size_t)tc_shape(L).K * 128 * sizeof(float);
+static size_t gb_net_smem_bytes(const ModelConst& mc) {
+  const size_t tc = tc_smem_layout(mc.L, nullptr);
+  const size_t st = gb_net_stash_offset(mc) + (size_t)tc_shape(mc.L).K * 128 * sizeof(float);
   return tc > st ? tc : st;
 }
 
@@ -940,8 +964,12 @@ size_t gb_net_smem_bytes(int N, int L) {
 // same threads in the move: a round trip through global memory less), then frees
 // the tensor memory and reuses the shared memory below the outputs for the
 // gamma/beta updates.  A kernel of its own, so that the plain gamma/beta kernel
-// keeps its own register allocation.
-__global__ void __launch_bounds__(128) k_gb_net_f32(ModelConst mc, DevPtrsF32 p, int seg_i,
+// keeps its own register allocation.  kBlocks: resident blocks per SM it is
+// compiled for: 3 (154 registers) while the genes fit them, else 4 (128, a few
+// spilled).  N=16 L=5: 34.6 against 35.7 us at G = 40000, 61.9 against 41.7 at 59500
+// (one block more than 3 per SM hold), 99 against 79 at 120000.
+template <int kBlocks>
+__global__ void __launch_bounds__(128, kBlocks) k_gb_net_f32(ModelConst mc, DevPtrsF32 p, int seg_i,
                                                     const uint8_t* __restrict__ img) {
   ktime_begin(p.ktime, p.ktime_n, 3 * seg_i + 1);
   bool net_ok;
@@ -960,7 +988,7 @@ __global__ void __launch_bounds__(128) k_gb_net_f32(ModelConst mc, DevPtrsF32 p,
     if (!c.w_ok) s_abort = 1;
     __syncthreads();
     const int g = blockIdx.x * 128 + (int)threadIdx.x;
-    prop_s = reinterpret_cast<float*>(sm_tc + gb_net_stash_offset(mc.N, mc.L));
+    prop_s = reinterpret_cast<float*>(sm_tc + gb_net_stash_offset(mc));
     if (!s_abort)
       tc_tile(c, mc, p, nh, t, sm_tc, g, net_gene(p, g, mc.G), prop_s, 128, (int)threadIdx.x,
               &s_abort);
@@ -990,8 +1018,8 @@ __global__ void __launch_bounds__(128) k_mh_step_f32(ModelConst mc, DevPtrsF32 p
   const int G = mc.G, N = mc.N, L = mc.L;
   for (int l = 0; l < L; ++l) bs[l * B + tid] = p.beta[(size_t)l * G + g];
   for (int n = 0; n < N; ++n) es[n * B + tid] = p.eps[(size_t)n * G + g];
-  const bool acc = mh_move_f32(mc, g, (uint32_t)it, bs, es, B, tid, u, 0.5f / p.gam[g], kind,
-                               p.prop, (size_t)G, g);
+  const bool acc = mh_move_f32(mc, g, (uint32_t)it, bs, es, B, tid, u,
+                               0.5f / p.gam[g], kind, p.prop, (size_t)G, g);
   const size_t ci = (size_t)(kind - 1) * G + g;
   p.mh_try[ci] += 1u;
   if (acc) {
@@ -1352,21 +1380,21 @@ cudaError_t launch_eps_f32(const ModelConst& mc, const DevPtrsF32& p, int seg_i,
 cudaError_t launch_gb_f32(const ModelConst& mc, const DevPtrsF32& p, int block, int seg_i,
                           cudaStream_t s, const void* img) {
   const int nblk = (mc.G + block - 1) / block;
-  size_t smem = gb_smem_f32(mc, block, p.prop != nullptr);
   if (img != nullptr) {
     if (block != 128) return cudaErrorInvalidValue;  // one thread per gene of a 128-gene tile
-    smem = gb_net_smem_bytes(mc.N, mc.L);
-    size_t most = 0;
-    for (int L = 1; L <= FBS_MAX_L; ++L) {
-      const size_t b = gb_net_smem_bytes(FBS_MAX_N, L);
-      if (b > most) most = b;
-    }
-    cudaError_t e = cudaFuncSetAttribute(k_gb_net_f32,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
+    const size_t smem = gb_net_smem_bytes(mc);
+    const auto kernel = nblk <= 3 * sms ? k_gb_net_f32<3> : k_gb_net_f32<4>;
+    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    kernel<<<nblk, block, smem, s>>>(mc, p, seg_i, (const uint8_t*)img);
+    return cudaGetLastError();
   }
-  if (img != nullptr) k_gb_net_f32<<<nblk, block, smem, s>>>(mc, p, seg_i, (const uint8_t*)img);
-  else if (p.prop != nullptr) k_gb_move_f32<<<nblk, block, smem, s>>>(mc, p, seg_i);
+  const size_t smem = gb_smem_f32(mc, block, p.prop != nullptr);
+  if (p.prop != nullptr) k_gb_move_f32<<<nblk, block, smem, s>>>(mc, p, seg_i);
   else k_gb_f32<<<nblk, block, smem, s>>>(mc, p, seg_i);
   return cudaGetLastError();
 }

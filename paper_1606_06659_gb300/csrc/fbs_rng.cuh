@@ -22,7 +22,7 @@ constexpr uint32_t kTruncStride = 256;  // uniforms reserved per truncated-draw 
 // truncation error below 3e-9), expf otherwise.  Both are evaluated: most warps
 // have lanes on either side, and side by side they cost less than a branch and
 // one after the other.
-__device__ __forceinline__ float em1mx(float z) {
+__device__ __forceinline__ float em1mx_series(float z) {
   float p = 1.0f / 362880.0f;
   p = fmaf(p, z, 1.0f / 40320.0f);
   p = fmaf(p, z, 1.0f / 5040.0f);
@@ -31,8 +31,13 @@ __device__ __forceinline__ float em1mx(float z) {
   p = fmaf(p, z, 1.0f / 24.0f);
   p = fmaf(p, z, 1.0f / 6.0f);
   p = fmaf(p, z, 0.5f);
-  const float series = z * z * p;
-  const float direct = expf(z) - 1.0f - z;
+  return z * z * p;
+}
+
+__device__ __forceinline__ float em1mx_direct(float z) { return expf(z) - 1.0f - z; }
+
+__device__ __forceinline__ float em1mx(float z) {
+  const float series = em1mx_series(z), direct = em1mx_direct(z);
   return fabsf(z) < 0.5f ? series : direct;
 }
 
