@@ -139,6 +139,16 @@ int block_of(const fbs_options* o) {
 
 void fbs::set_last_error(const std::string& msg) { g_err = msg; }
 
+// Scratch of one training step for batch size B; flags: the tensor-core wait
+// flag word of the step's kernels; img: the training kernel's weight image; stat:
+// scratch of the column statistics.
+struct TrainBufs {
+  float *fb, *yb, *part, *grad, *loss;
+  unsigned* flags;
+  void* img;
+  double* stat;
+};
+
 // Learned beta_g proposal of one FP32 handle.
 struct LearnedState {
   int L = 0, F = 0, K = 0, np = 0;
@@ -156,9 +166,20 @@ struct LearnedState {
   float* pair_beta = nullptr;  // [cap][L]
   long long pair_cap = 0, pairs = 0;
   int mode = 0;                // 1: genes with use_mh take the learned move
+  struct TrainBufs* bufs = nullptr;  // scratch of the training steps, kept between calls
+  int bufs_batch = 0;
   bool trained = false;
   bool fused = true;           // the gamma/beta kernel runs the network pass itself
 };
+
+static void train_bufs_free(TrainBufs& t) {
+  cudaFree(t.fb);
+  cudaFree(t.img);
+  cudaFree(t.stat);
+  t.fb = nullptr;
+  t.img = nullptr;
+  t.stat = nullptr;
+}
 
 struct fbs_handle {
   ModelConst mc;
@@ -1179,6 +1200,10 @@ void fbs_free(fbs_handle* h) {
     cudaFree(ls->stats);
     cudaFree(ls->pair_feat);
     cudaFree(ls->pair_beta);
+    if (ls->bufs) {
+      train_bufs_free(*ls->bufs);
+      delete ls->bufs;
+    }
     delete ls;
   }
   if (h->seg_exec) cudaGraphExecDestroy(h->seg_exec);
@@ -1272,21 +1297,6 @@ void learned_apply(fbs_handle* h, int mode, int mh_all) {
 
 constexpr int kTrainGraphSteps = 8;  // training steps per replayed graph
 
-// Scratch of one training step for batch size B; flags: the tensor-core wait
-// flag word of the step's kernels (zeroed here).
-struct TrainBufs {
-  float *fb, *yb, *part, *grad, *loss;
-  unsigned* flags;
-  void* img;  // the training kernel's weight image (zeroed)
-};
-
-void train_bufs_free(TrainBufs& t) {
-  cudaFree(t.fb);
-  cudaFree(t.img);
-  t.fb = nullptr;
-  t.img = nullptr;
-}
-
 // Gradient and summed loss of the minibatch in t.fb / t.yb at params.
 int mlp_step(const float* params, int L, int B, TrainBufs& t, cudaStream_t s) {
   FBS_CUDA(launch_mlp_grad(params, L, B, t.fb, t.yb, t.part, t.grad, t.loss, t.img, t.flags,
@@ -1312,6 +1322,7 @@ int train_bufs_alloc(TrainBufs& t, int L, int B) {
   cudaError_t e = cudaMemset(t.flags, 0, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMalloc(&t.img, train_image_bytes(L));
   if (e == cudaSuccess) e = cudaMemset(t.img, 0, train_image_bytes(L));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&t.stat, col_stats_bytes(L));
   if (e != cudaSuccess) train_bufs_free(t);
   FBS_CUDA(e);
   return FBS_OK;
@@ -1373,9 +1384,19 @@ int fbs_proposal_train(fbs_handle* h, int epochs, int batch, double lr, uint64_t
   LearnedState* ls = h->learned;
   if (ls->pairs < 1) return fail(FBS_E_ARG, "no training pairs: call fbs_proposal_collect first");
   if (epochs < 1 || batch < 32 || !(lr > 0.0)) return fail(FBS_E_ARG, "bad epochs, batch or lr");
-  TrainBufs t;
-  rc = train_bufs_alloc(t, ls->L, batch);
-  if (rc) return rc;
+  if (ls->bufs && ls->bufs_batch != batch) {
+    train_bufs_free(*ls->bufs);
+    delete ls->bufs;
+    ls->bufs = nullptr;
+  }
+  if (!ls->bufs) {
+    TrainBufs fresh;
+    rc = train_bufs_alloc(fresh, ls->L, batch);
+    if (rc) return rc;
+    ls->bufs = new TrainBufs(fresh);
+    ls->bufs_batch = batch;
+  }
+  TrainBufs& t = *ls->bufs;
   const long long steps_per_epoch = (ls->pairs + batch - 1) / batch;
   const long long steps = steps_per_epoch * epochs;
   const int F = ls->F, L = ls->L;
@@ -1383,7 +1404,9 @@ int fbs_proposal_train(fbs_handle* h, int epochs, int batch, double lr, uint64_t
   // already trained (or set) move to those coordinates first, the initial ones
   // are drawn for them.
   std::vector<float> st_h(2 * F + 2 * L);
-  cudaError_t e = launch_col_stats(ls->pair_feat, ls->pair_beta, ls->pairs, F, L, ls->stats, h->s);
+  cudaError_t e = cudaMemsetAsync(t.flags, 0, sizeof(unsigned), h->s);
+  if (e == cudaSuccess)
+    e = launch_col_stats(ls->pair_feat, ls->pair_beta, ls->pairs, F, L, t.stat, ls->stats, h->s);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(st_h.data(), ls->stats, sizeof(float) * st_h.size(),
                         cudaMemcpyDeviceToHost, h->s);
@@ -1392,9 +1415,9 @@ int fbs_proposal_train(fbs_handle* h, int epochs, int batch, double lr, uint64_t
   double log_scale = 0.0;  // NLL of raw beta = NLL of standardised beta + sum log s_beta
   for (int l = 0; l < L; ++l) log_scale += log((double)st_h[2 * F + L + l]);
   // Training steps (minibatch gather, forward, backward, Adam, bookkeeping) are
-  // captured once, kTrainGraphSteps of them in one graph and one alone, and
-  // replayed to make `steps`; the step counter, the Adam scalars and the loss
-  // sum live in a device control block.
+  // captured, kTrainGraphSteps of them in one graph, and replayed to make `steps`;
+  // the rest are launched one by one.  The step counter, the Adam scalars and the
+  // loss sum live in a device control block.
   TrainCtl ctl;
   memset(&ctl, 0, sizeof(ctl));
   ctl.t = (unsigned long long)ls->adam_t;
@@ -1404,35 +1427,35 @@ int fbs_proposal_train(fbs_handle* h, int epochs, int batch, double lr, uint64_t
   ctl.b1 = 0.9f;
   ctl.b2 = 0.999f;
   TrainCtl* d_ctl = nullptr;
-  cudaGraphExec_t exec[2] = {nullptr, nullptr};  // kTrainGraphSteps steps, one step
+  cudaGraphExec_t exec = nullptr;
   if (e == cudaSuccess) e = cudaMalloc((void**)&d_ctl, sizeof(TrainCtl));
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_ctl, &ctl, sizeof(ctl), cudaMemcpyHostToDevice, h->s);
   if (e == cudaSuccess) e = launch_pack_train_image(ls->params, L, t.img, h->s);
-  for (int gi = 0; gi < 2 && e == cudaSuccess; ++gi) {
+  auto step = [&] {
+    return launch_train_step(ls->params, L, batch, ls->pair_feat, ls->pair_beta, ls->pairs, seed,
+                             d_ctl, ls->stats, t.part, t.grad, t.loss, ls->adam_m, ls->adam_v,
+                             t.img, t.flags, h->pf.tc_polls, h->s);
+  };
+  if (e == cudaSuccess && steps >= kTrainGraphSteps) {
     cudaGraph_t graph = nullptr;
     e = cudaStreamBeginCapture(h->s, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
       cudaError_t ce = cudaSuccess;
-      for (int k = 0; k < (gi == 0 ? kTrainGraphSteps : 1) && ce == cudaSuccess; ++k)
-        ce = launch_train_step(ls->params, L, batch, ls->pair_feat, ls->pair_beta, ls->pairs,
-                               seed, d_ctl, ls->stats, t.part, t.grad, t.loss, ls->adam_m,
-                               ls->adam_v, t.img, t.flags, h->pf.tc_polls, h->s);
+      for (int k = 0; k < kTrainGraphSteps && ce == cudaSuccess; ++k) ce = step();
       e = cudaStreamEndCapture(h->s, &graph);
       if (e == cudaSuccess) e = ce;
     }
-    if (e == cudaSuccess && rc == FBS_OK) e = cudaGraphInstantiate(&exec[gi], graph, 0);
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&exec, graph, 0);
     if (graph) cudaGraphDestroy(graph);
   }
-  for (long long st = 0; st < steps / kTrainGraphSteps && rc == FBS_OK && e == cudaSuccess; ++st)
-    e = cudaGraphLaunch(exec[0], h->s);
-  for (long long st = 0; st < steps % kTrainGraphSteps && rc == FBS_OK && e == cudaSuccess; ++st)
-    e = cudaGraphLaunch(exec[1], h->s);
+  for (long long st = 0; st < steps / kTrainGraphSteps && e == cudaSuccess; ++st)
+    e = cudaGraphLaunch(exec, h->s);
+  for (long long st = 0; st < steps % kTrainGraphSteps && e == cudaSuccess; ++st) e = step();
   if (e == cudaSuccess && rc == FBS_OK)
     e = cudaMemcpyAsync(&ctl, d_ctl, sizeof(ctl), cudaMemcpyDeviceToHost, h->s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->s);
-  for (cudaGraphExec_t x : exec)
-    if (x) cudaGraphExecDestroy(x);
+  if (exec) cudaGraphExecDestroy(exec);
   cudaFree(d_ctl);
   // a step whose tensor-core wait gave up left the parameters as they were; the
   // parameters still go back to raw coordinates before the error is returned
@@ -1443,7 +1466,6 @@ int fbs_proposal_train(fbs_handle* h, int epochs, int batch, double lr, uint64_t
   if (e == cudaSuccess && rc == FBS_OK) e = launch_fold(ls->params, ls->stats, L, 1, h->s);
   if (e == cudaSuccess && rc == FBS_OK) e = launch_pack_image(ls->params, ls->w_image, ls->L, h->s);
   if (e == cudaSuccess && rc == FBS_OK) e = cudaStreamSynchronize(h->s);
-  train_bufs_free(t);
   if (rc) return rc;
   FBS_CUDA(e);
   ls->trained = true;  // raw coordinates from here on, even after a failed wait

@@ -132,8 +132,10 @@ cudaError_t launch_proposal_f32(const ModelConst& mc, const DevPtrsF32& p, const
                                 float* out, cudaStream_t s);
 cudaError_t launch_collect_f32(const ModelConst& mc, const DevPtrsF32& p, float* feat,
                                float* beta, long long row, cudaStream_t s);
+// part: col_stats_bytes(L) of scratch
+size_t col_stats_bytes(int L);
 cudaError_t launch_col_stats(const float* feat, const float* beta, long long M, int F, int L,
-                             float* st, cudaStream_t s);
+                             double* part, float* st, cudaStream_t s);
 cudaError_t launch_fold(float* params, const float* st, int L, int to_raw, cudaStream_t s);
 // one training step's gradient: fused forward/backward per block of 128 rows on
 // the tensor cores, then the blocks' partial sums in block order (part:
