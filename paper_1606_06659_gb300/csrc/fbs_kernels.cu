@@ -500,16 +500,15 @@ __device__ __forceinline__ GbF64 gb_begin_f64(const ModelConst& mc, const DevPtr
   return c;
 }
 
-// Steps 2 and 5 for gene g (thread tid of the B genes whose rates mu [N][B] are in
-// shared memory): the gamma_g draw, the beta_gl, their moments and trace, and the
-// thread's terms ps [kNumPart][B] of the sums for steps 3, 4, 6, 7.
-__device__ __forceinline__ void gb_gene_f64(const ModelConst& mc, const DevPtrs& p, int g, int B,
-                                            int tid, double* mu, double* bs, double* ps,
-                                            const GbUniform& u, GbF64& c) {
-  const int G = mc.G, N = mc.N, L = mc.L;
+// Step 2 for gene g (column tid of the B genes of ps [kNumPart][B], the terms of
+// the sums for steps 3, 4, 6, 7): the gamma_g draw and its moments.  It and the beta
+// updates need the sweep's eps and the hyperparameters but not each other, so they
+// may run on different warps.
+__device__ __forceinline__ void gb_gamma_f64(const ModelConst& mc, const DevPtrs& p, int g, int B,
+                                             int tid, double* ps, GbF64& c) {
+  const int G = mc.G, N = mc.N;
   const Hyper* hy = c.hy;
   const double nu = hy->phi[0], tau = hy->phi[1];
-  for (int l = 0; l < L; ++l) bs[l * B + tid] = p.beta[(size_t)l * G + g];
   double ss = 0.0;
 #pragma unroll 8
   for (int n = 0; n < N; ++n) {
@@ -559,10 +558,17 @@ __device__ __forceinline__ void gb_gene_f64(const ModelConst& mc, const DevPtrs&
     ps[0 * B + tid] = log(gam);
     ps[1 * B + tid] = 1.0 / gam;
   }
+}
 
-  // ---- step 5: beta_gl, l = 1..L in order
+// Step 5 for gene g, whose rates mu [N][B] are in shared memory: the beta_gl, l =
+// 1..L in order, with their moments, trace and terms of the sums.
+__device__ __forceinline__ void gb_beta_f64(const ModelConst& mc, const DevPtrs& p, int g, int B,
+                                            int tid, double* mu, double* bs, double* ps,
+                                            const GbUniform& u, GbF64& c) {
+  const int G = mc.G, L = mc.L;
+  for (int l = 0; l < L; ++l) bs[l * B + tid] = p.beta[(size_t)l * G + g];
   for (int l = 0; l < L; ++l) {
-    const double theta = hy->phi[2 + l], hs = u.hs[l];
+    const double theta = c.hy->phi[2 + l], hs = u.hs[l];
     switch (mc.ncls[l]) {
       case 1: beta_column_f64<1>(mc, p, l, g, mu, bs, ps, B, tid, theta, hs, c); break;
       case 2: beta_column_f64<2>(mc, p, l, g, mu, bs, ps, B, tid, theta, hs, c); break;
@@ -583,6 +589,18 @@ __device__ __forceinline__ void gb_gene_f64(const ModelConst& mc, const DevPtrs&
       }
       if (ok) p.con_count[(size_t)q * G + g] += 1u;
     }
+  }
+}
+
+// The sum over a warp's 32 genes of every row of ps, on lane 0.
+template <class Store>
+__device__ __forceinline__ void warp_sums(const double* ps, int lane, Store store) {
+#pragma unroll
+  for (int i = 0; i < kNumPart; ++i) {
+    double x = ps[i * 32 + lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+    if (lane == 0) store(i, x);
   }
 }
 
@@ -615,7 +633,10 @@ __global__ void __launch_bounds__(128, 3) k_gb_f64(ModelConst mc, DevPtrs p, int
   if (tid < 32) gb_uniform(mc, c.hy, c.mom, tid, &u);
   __syncthreads();
   c.inv_k = u.inv_k;
-  if (active) gb_gene_f64(mc, p, g, B, tid, mu, bs, ps, u, c);
+  if (active) {
+    gb_gamma_f64(mc, p, g, B, tid, ps, c);
+    gb_beta_f64(mc, p, g, B, tid, mu, bs, ps, u, c);
+  }
 
   double part[kNumPart];
 #pragma unroll
@@ -626,16 +647,61 @@ __global__ void __launch_bounds__(128, 3) k_gb_f64(ModelConst mc, DevPtrs p, int
   ktime_end(p.ktime, p.ktime_n, 3 * seg_i + 1);
 }
 
+// k_gb_f64 for blocks of 32 genes with the beta updates on one warp and the gamma
+// draws on another, for datasets whose blocks leave parts of the SMs idle: a
+// warp's FP64 instructions take 64 cycles each, on its quarter of the SM alone, so
+// the kernel lasts as long as its longest warp.  N=4 G=1000 L=2: 33.4 -> 22.6 us; N=16
+// L=5: 58.6 -> 49.3 at G=5000, 71.5 -> 69.6 at 29000, where its two warps per block
+// still all fit (beyond that the one-warp blocks have twice the genes resident).
+constexpr int kSplitBlocks = 6;  // resident blocks per SM
+
+__global__ void __launch_bounds__(64, kSplitBlocks) k_gb_split_f64(ModelConst mc, DevPtrs p,
+                                                                  int seg_i) {
+  extern __shared__ double smem_dyn[];  // mu[N][32], beta[kMaxL][32], partials[kNumPart][32]
+  __shared__ GbUniform u;
+  ktime_begin(p.ktime, p.ktime_n, 3 * seg_i + 1);
+  const int G = mc.G, N = mc.N;
+  GbF64 c = gb_begin_f64(mc, p, seg_i);
+  double* mu = smem_dyn;
+  double* bs = mu + (size_t)N * 32;
+  double* ps = bs + (size_t)kMaxL * 32;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int g = blockIdx.x * 32 + lane;
+  if (warp == 0) {
+    if (g < G) {
+#pragma unroll 8
+      for (int n = 0; n < N; ++n) mu[n * 32 + lane] = p.mu[(size_t)n * G + g];
+    }
+#pragma unroll
+    for (int i = 0; i < kNumPart; ++i) ps[i * 32 + lane] = 0.0;
+  } else {
+    gb_uniform(mc, c.hy, c.mom, lane, &u);
+  }
+  __syncthreads();
+  c.inv_k = u.inv_k;
+  if (g < G) {
+    if (warp == 0) gb_beta_f64(mc, p, g, 32, lane, mu, bs, ps, u, c);
+    else gb_gamma_f64(mc, p, g, 32, lane, ps, c);
+  }
+  __syncthreads();
+  if (warp == 0)
+    warp_sums(ps, lane,
+              [&](int i, double x) { p.partial[(size_t)blockIdx.x * kNumPart + i] = 0.0 + x; });
+  add_counters_u(p.counters, 0, c.evals_b, c.caps, c.gcaps, c.nonfin, &p.hyp->flags, c.evals_g);
+  ktime_end(p.ktime, p.ktime_n, 3 * seg_i + 1);
+}
+
 // Steps 1, 2 and 5 in one launch for fbs_sweep_noalloc: a block takes 32 genes, its
 // four warps the samples' eps updates in turn with the rates kept in shared
-// memory, then the first warp the genes' gamma and beta updates.  The four blocks
+// memory, then the first warp the genes' beta updates beside the second's gamma
+// draws.  The four blocks
 // of a cluster are the 128 genes of one row of partial sums (what the fixed
 // scratch has rows for) and add their sums in order through distributed shared
 // memory.  32 genes per block, not 128: N=16 G=20011 is 626 blocks for 152 SMs
 // instead of 157, and a few blocks share an SM, so that the one's serial gene
 // phase runs beside the other's eps phase.  Bound by the FP64 pipe.  One sweep of
 // N=16 G=20011 L=5: 659 us with one thread per gene making its 16 eps updates in a
-// row in FP64, 205 us so.
+// row in FP64, 182 us so.
 constexpr int kSweepWarps = 4, kSweepCluster = 4;
 
 __global__ void __cluster_dims__(kSweepCluster, 1, 1) __launch_bounds__(32 * kSweepWarps, 3)
@@ -674,18 +740,13 @@ __global__ void __cluster_dims__(kSweepCluster, 1, 1) __launch_bounds__(32 * kSw
     }
   }
   __syncthreads();
-  if (warp == 0) {
-    c.inv_k = u.inv_k;
-    if (g < G) gb_gene_f64(mc, p, g, 32, lane, mu, bs, ps, u, c);
-    __syncwarp();
-#pragma unroll
-    for (int i = 0; i < kNumPart; ++i) {
-      double x = ps[i * 32 + lane];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-      if (lane == 0) s_sum[i] = x;
-    }
+  c.inv_k = u.inv_k;
+  if (g < G) {
+    if (warp == 0) gb_beta_f64(mc, p, g, 32, lane, mu, bs, ps, u, c);
+    else if (warp == 1) gb_gamma_f64(mc, p, g, 32, lane, ps, c);
   }
+  __syncthreads();
+  if (warp == 0) warp_sums(ps, lane, [&](int i, double x) { s_sum[i] = x; });
   add_counters_u(p.counters, evals_e, c.evals_b, c.caps, c.gcaps, c.nonfin, &p.hyp->flags, c.evals_g);
   cg::cluster_group cl = cg::this_cluster();
   cl.sync();
@@ -1056,6 +1117,15 @@ cudaError_t launch_eps_f64(const ModelConst& mc, const DevPtrs& p, int seg_i, cu
 cudaError_t launch_gb_f64(const ModelConst& mc, const DevPtrs& p, int block, int seg_i,
                           cudaStream_t s) {
   const int nblk = (mc.G + block - 1) / block;
+  int dev = 0, sms = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  // split while all its blocks are resident (both measured at k_gb_split_f64)
+  if (block == 32 && nblk <= kSplitBlocks * sms) {
+    k_gb_split_f64<<<nblk, 64, gb_smem_bytes_f64(mc.N, 32), s>>>(mc, p, seg_i);
+    return cudaGetLastError();
+  }
   k_gb_f64<<<nblk, block, gb_smem_bytes_f64(mc.N, block), s>>>(mc, p, seg_i);
   return cudaGetLastError();
 }
