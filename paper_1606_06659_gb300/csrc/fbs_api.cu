@@ -1420,7 +1420,7 @@ int fbs_proposal_train(fbs_handle* h, int epochs, int batch, double lr, uint64_t
   // loss sum live in a device control block.
   TrainCtl ctl;
   memset(&ctl, 0, sizeof(ctl));
-  ctl.t = (unsigned long long)ls->adam_t;
+  ctl.t = ctl.t0 = (unsigned long long)ls->adam_t;
   ctl.steps = steps;
   ctl.epoch_steps = steps_per_epoch;
   ctl.lr = lr;
@@ -1432,9 +1432,9 @@ int fbs_proposal_train(fbs_handle* h, int epochs, int batch, double lr, uint64_t
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_ctl, &ctl, sizeof(ctl), cudaMemcpyHostToDevice, h->s);
   if (e == cudaSuccess) e = launch_pack_train_image(ls->params, L, t.img, h->s);
-  auto step = [&] {
+  auto step = [&](int k, int n) {
     return launch_train_step(ls->params, L, batch, ls->pair_feat, ls->pair_beta, ls->pairs, seed,
-                             d_ctl, ls->stats, t.part, t.grad, t.loss, ls->adam_m, ls->adam_v,
+                             d_ctl, k, n, ls->stats, t.part, t.grad, t.loss, ls->adam_m, ls->adam_v,
                              t.img, t.flags, h->pf.tc_polls, h->s);
   };
   if (e == cudaSuccess && steps >= kTrainGraphSteps) {
@@ -1442,7 +1442,8 @@ int fbs_proposal_train(fbs_handle* h, int epochs, int batch, double lr, uint64_t
     e = cudaStreamBeginCapture(h->s, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
       cudaError_t ce = cudaSuccess;
-      for (int k = 0; k < kTrainGraphSteps && ce == cudaSuccess; ++k) ce = step();
+      for (int k = 0; k < kTrainGraphSteps && ce == cudaSuccess; ++k)
+        ce = step(k, kTrainGraphSteps);
       e = cudaStreamEndCapture(h->s, &graph);
       if (e == cudaSuccess) e = ce;
     }
@@ -1451,7 +1452,8 @@ int fbs_proposal_train(fbs_handle* h, int epochs, int batch, double lr, uint64_t
   }
   for (long long st = 0; st < steps / kTrainGraphSteps && e == cudaSuccess; ++st)
     e = cudaGraphLaunch(exec, h->s);
-  for (long long st = 0; st < steps % kTrainGraphSteps && e == cudaSuccess; ++st) e = step();
+  const int rest = (int)(steps % kTrainGraphSteps);
+  for (int k = 0; k < rest && e == cudaSuccess; ++k) e = step(k, rest);
   if (e == cudaSuccess && rc == FBS_OK)
     e = cudaMemcpyAsync(&ctl, d_ctl, sizeof(ctl), cudaMemcpyDeviceToHost, h->s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(h->s);

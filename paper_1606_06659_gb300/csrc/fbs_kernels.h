@@ -109,6 +109,7 @@ cudaError_t launch_estimates(const RhatInput& in, double z, double* out, cudaStr
 // Training control block in device memory (one Adam step per captured replay).
 struct TrainCtl {
   unsigned long long t;      // Adam steps done before the current step
+  unsigned long long t0;     // the same before the current group of steps
   long long k, steps, epoch_steps;  // step within the call, steps of the call, of an epoch
   double lr, loss_sum;       // base step size; loss summed over the last epoch's steps
   float b1, b2;
@@ -121,10 +122,14 @@ struct TrainCtl {
 // img: the step's weight image (train_image_bytes(L), zeroed when allocated,
 // packed from params by launch_pack_train_image before the first step); the
 // Adam update rewrites it for the next step.
+// The step is number `step` of a group of `steps` launched one after the other: its
+// rows are drawn for step t0 + step + 1, so that it may begin beside the update of
+// the step before it, and the last of the group advances t0.
 cudaError_t launch_train_step(float* params, int L, int Bsz, const float* feat, const float* beta,
-                              long long M, uint64_t seed, TrainCtl* ctl, const float* st,
-                              float* part, float* grad, float* loss, float* adam_m, float* adam_v,
-                              void* img, unsigned* flags, unsigned polls, cudaStream_t s);
+                              long long M, uint64_t seed, TrainCtl* ctl, int step, int steps,
+                              const float* st, float* part, float* grad, float* loss,
+                              float* adam_m, float* adam_v, void* img, unsigned* flags,
+                              unsigned polls, cudaStream_t s);
 size_t train_image_bytes(int L);
 cudaError_t launch_pack_train_image(const float* params, int L, void* img, cudaStream_t s);
 int mlp_param_count(int L);

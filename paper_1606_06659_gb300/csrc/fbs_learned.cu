@@ -396,6 +396,15 @@ __global__ void k_pack_train_image(const float* __restrict__ w, int L, uint8_t* 
     train_img_put(img, t, p, w[p]);
 }
 
+// Programmatic dependent launch: wait for the kernels before this one (at once when
+// it was launched without the attribute), and let the next one begin.
+__device__ __forceinline__ void grid_dep_wait() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void grid_dep_launch() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 constexpr uint32_t kTrainTmemCols = 512;
 constexpr int kTrainOutPad = (kMaxOut + 15) & ~15;
 
@@ -548,8 +557,9 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
     int L, int Bsz, const float* __restrict__ fb,
     const float* __restrict__ yb, const float* __restrict__ feat,
     const float* __restrict__ beta, long long M, uint32_t seed_lo, uint32_t seed_hi,
-    const TrainCtl* __restrict__ ctl, const float* __restrict__ st, float* __restrict__ part,
-    const uint8_t* __restrict__ img, unsigned* __restrict__ flags, unsigned polls) {
+    const TrainCtl* __restrict__ ctl, int step, const float* __restrict__ st,
+    float* __restrict__ part, const uint8_t* __restrict__ img, unsigned* __restrict__ flags,
+    unsigned polls) {
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ __align__(8) uint64_t bars[2];
   __shared__ uint32_t tmem_slot;
@@ -583,16 +593,6 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c.bar_w) : "memory");
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(c.bar_m) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    // the weight image (written by the previous step's Adam update, or packed
-    // before the first step): one bulk copy, waited for before the first product
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(c.bar_w),
-                 "r"(t.img_bytes)
-                 : "memory");
-    asm volatile(
-        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
-            "r"(smem_u32(sm)),
-        "l"(img), "r"(t.img_bytes), "r"(c.bar_w)
-        : "memory");
   }
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
@@ -605,7 +605,8 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
   // this thread's row: features and the column of ones (split into bufF), beta
   long long srow = 0;
   if (feat != nullptr && row_ok) {
-    Rng rg(seed_lo, seed_hi, 0u, kStreamTrain, (uint32_t)(r0 + tid), (uint32_t)(ctl->t + 1));
+    Rng rg(seed_lo, seed_hi, 0u, kStreamTrain, (uint32_t)(r0 + tid),
+           (uint32_t)(ctl->t0 + (unsigned long long)step + 1));
     const long long m = (long long)(rg.u(0) * (double)M);
     srow = m >= M ? M - 1 : m;
   }
@@ -635,6 +636,21 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
       if (q < t.cx) store_split8_ch(bF, t.sbo_f, tid, 8 + q, 8 + q + half, x + 8 * q);
   }
 
+  // Up to here nothing depends on the previous step, and the launch may have begun
+  // beside its update; from here on everything does.  The weight image (written by
+  // that update, or packed before the first step): one bulk copy, waited for before
+  // the first product.
+  grid_dep_wait();
+  if (tid == 0) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(c.bar_w),
+                 "r"(t.img_bytes)
+                 : "memory");
+    asm volatile(
+        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::
+            "r"(smem_u32(sm)),
+        "l"(img), "r"(t.img_bytes), "r"(c.bar_w)
+        : "memory");
+  }
   c.w_ok = mbar_wait(c.bar_w, 0, c.polls);
   if (!c.w_ok) s_abort = 1;
   tc_fence_before();
@@ -747,6 +763,7 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
                   128);
     });
   }
+  grid_dep_launch();  // the reduction's blocks get ready while the sums are written
   // ---- this block's sums, in parameter order: W1 [64][F], b1, W2 [64][64], b2,
   // W3 [K][64], b3, loss
   if (ok) {
@@ -822,7 +839,7 @@ __device__ __forceinline__ void adam_scalars(const TrainCtl* c, float* c1, float
 // and warp 0 adds the eight warp sums in order.  With a control block it also
 // applies Adam to w, m, v, writes the new w into the training kernel's weight
 // image img and, in the last block to finish (ticket counter, no waiting), adds
-// the loss to the last epoch's sum and advances t and k.  Does
+// the loss to the last epoch's sum and advances t and k, and t0 by `advance`.  Does
 // nothing once *flags is set (a tensor-core wait of the forward and backward
 // pass gave up, so the partials are incomplete).
 __global__ void __launch_bounds__(256) k_reduce_adam(const float* __restrict__ part, int nblk,
@@ -830,7 +847,9 @@ __global__ void __launch_bounds__(256) k_reduce_adam(const float* __restrict__ p
                                                      float* __restrict__ loss, float* w, float* m,
                                                      float* v, TrainCtl* ctl, int B, float eps,
                                                      const unsigned* __restrict__ flags,
-                                                     uint8_t* __restrict__ img, int L) {
+                                                     uint8_t* __restrict__ img, int L, int advance) {
+  grid_dep_wait();
+  grid_dep_launch();  // the next step draws and gathers its rows meanwhile
   if (*(volatile const unsigned*)flags != 0u) return;
   __shared__ float red[8][33];
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -875,6 +894,7 @@ __global__ void __launch_bounds__(256) k_reduce_adam(const float* __restrict__ p
       if (ctl->k >= ctl->steps - ctl->epoch_steps) ctl->loss_sum += (double)lv / (double)B;
       ctl->t += 1;
       ctl->k += 1;
+      ctl->t0 += (unsigned long long)advance;
       ctl->done = 0;
     }
   }
@@ -948,6 +968,24 @@ cudaError_t launch_pack_train_image(const float* params, int L, void* img, cudaS
   return cudaGetLastError();
 }
 
+// A launch that may begin before the kernel in front of it in the stream has ended
+// (its grid_dep_wait makes up for it).
+template <class... Par, class... Arg>
+static cudaError_t launch_overlapped(void (*kernel)(Par...), int grid, int block, size_t smem,
+                                     cudaStream_t s, bool overlap, Arg... arg) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, Par(arg)...);
+}
+
 cudaError_t launch_mlp_grad(const float* params, int L, int Bsz, const float* fb, const float* yb,
                             float* part, float* grad, float* loss, void* img, unsigned* flags,
                             unsigned polls, cudaStream_t s) {
@@ -955,26 +993,33 @@ cudaError_t launch_mlp_grad(const float* params, int L, int Bsz, const float* fb
   const int np = mlp_param_count(L);
   k_pack_train_image<<<32, 256, 0, s>>>(params, L, (uint8_t*)img);
   k_mlp_tc<<<nblk, 128, train_smem_bytes(L), s>>>(L, Bsz, fb, yb, nullptr, nullptr, 0,
-                                                  0u, 0u, nullptr, nullptr, part,
+                                                  0u, 0u, nullptr, 0, nullptr, part,
                                                   (const uint8_t*)img, flags, polls);
   k_reduce_adam<<<(np + 1 + 31) / 32, 256, 0, s>>>(part, nblk, np, grad, loss, nullptr, nullptr,
-                                                   nullptr, nullptr, Bsz, 0.0f, flags, nullptr, L);
+                                                   nullptr, nullptr, Bsz, 0.0f, flags, nullptr, L,
+                                                   0);
   return cudaGetLastError();
 }
 
+// A step's kernels overlap at their edges: the reduction's blocks are launched
+// while the gradient kernel writes its sums, and the next step's blocks draw,
+// gather and split their rows beside the reduction.  33.8 -> 29.5 us per step
+// of 8192 rows at L = 5.
 cudaError_t launch_train_step(float* params, int L, int Bsz, const float* feat, const float* beta,
-                              long long M, uint64_t seed, TrainCtl* ctl, const float* st,
-                              float* part, float* grad, float* loss, float* adam_m, float* adam_v,
-                              void* img, unsigned* flags, unsigned polls, cudaStream_t s) {
+                              long long M, uint64_t seed, TrainCtl* ctl, int step, int steps,
+                              const float* st, float* part, float* grad, float* loss,
+                              float* adam_m, float* adam_v, void* img, unsigned* flags,
+                              unsigned polls, cudaStream_t s) {
   const int nblk = train_blocks(Bsz);
   const int np = mlp_param_count(L);
-  k_mlp_tc<<<nblk, 128, train_smem_bytes(L), s>>>(L, Bsz, nullptr, nullptr, feat, beta, M,
-                                                  (uint32_t)seed, (uint32_t)(seed >> 32), ctl, st,
-                                                  part, (const uint8_t*)img, flags, polls);
-  k_reduce_adam<<<(np + 1 + 31) / 32, 256, 0, s>>>(part, nblk, np, grad, loss, params, adam_m,
-                                                   adam_v, ctl, Bsz, 1e-8f, flags,
-                                                   (uint8_t*)img, L);
-  return cudaGetLastError();
+  cudaError_t e = launch_overlapped(k_mlp_tc, nblk, 128, train_smem_bytes(L), s, step > 0, L, Bsz,
+                                    nullptr, nullptr, feat, beta, M, (uint32_t)seed,
+                                    (uint32_t)(seed >> 32), ctl, step, st, part,
+                                    (const uint8_t*)img, flags, polls);
+  if (e != cudaSuccess) return e;
+  return launch_overlapped(k_reduce_adam, (np + 1 + 31) / 32, 256, 0, s, true, part, nblk, np, grad,
+                           loss, params, adam_m, adam_v, ctl, Bsz, 1e-8f, flags, (uint8_t*)img, L,
+                           step == steps - 1 ? steps : 0);
 }
 
 }  // namespace fbs
