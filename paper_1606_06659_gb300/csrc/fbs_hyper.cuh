@@ -2,7 +2,7 @@
 // steps 3, 4, 6, 7 of Landau & Niemi, arXiv 1606.06659) as a block-level device
 // function, shared by the single-chain and the batched hyperparameter kernels.
 // tau and sigma_l^2 are drawn exactly, or (ModelConst::all_slice) by slice
-// updates of their conditionals: tau spread over warp 0, sigma_l on lane 32+l.
+// updates of their conditionals, each spread over a warp.
 #pragma once
 
 #include <math.h>
@@ -340,6 +340,7 @@ __device__ __forceinline__ void hyper_body(const ModelConst& mc, const double* p
   __shared__ double theta_z[kMaxL];      // from warp 3, for warp 1
   __shared__ double sig_g[kMaxL];        // from warp 2, for warp 1
   __shared__ int sig_gcap[kMaxL];
+  __shared__ double sig_S[kMaxL];        // all_slice: sum (beta - theta_new)^2
   __shared__ double inv_k;               // weight of the draw in the moments
   static_assert(sizeof(Hyper) % 8 == 0, "Hyper is copied as 8-byte words");
   const int L = mc.L, P = mc.P;
@@ -361,7 +362,7 @@ __device__ __forceinline__ void hyper_body(const ModelConst& mc, const double* p
     __syncthreads();
   }
   // barriers: 1 sig_g, 2 warp 3's numbers, 3 the sums and the logs at the nu points,
-  // 4 the proposals, 5 warps 4-7 among themselves
+  // 4 the proposals, 5 warps 4-7 among themselves, 6 (all_slice) sig_S
   constexpr int kSumsCount = kWide ? 96 : 64;
 
   if (warp == 0) {
@@ -453,34 +454,18 @@ __device__ __forceinline__ void hyper_body(const ModelConst& mc, const double* p
     if (on) {
       // step 7: sigma_l^2 ~ IG((G-1)/2, S/2) on (0, s_l^2), S = sum (beta - theta_new)^2
       Rng rs(mc.seed_lo, mc.seed_hi, mc.chain, kStreamSigma, (uint32_t)l, it32);
-      double s2n;
       if (mc.all_slice) {
-        // a slice update of sigma_l itself on (0, s_l); the state keeps sigma_l^2
-        const double x0 = sqrt(sig2);
-        SliceResult ss = slice_update(x0, sh.w_hyp[1 + l], SigDensity{G, 0.5 * S, mc.s[l]}, rs,
-                                      mc.K, mc.shrink_max);
-        s2n = ss.x * ss.x;
-        if (it <= sh.burnin) {
-          double w = sh.w_hyp[1 + l], waux = sh.waux_hyp[1 + l];
-          tune_width(w, waux, it, ss.x, x0, sh.burnin, sh.tune_start);
-          hy->w_hyp[1 + l] = w;
-          hy->waux_hyp[1 + l] = waux;
-        }
-        atomicAdd(&counters[FBS_CNT_EVALS_HYPER], (unsigned long long)ss.evals);
-        if (ss.capped) atomicAdd(&counters[FBS_CNT_SLICE_CAPS], 1ull);
-        if (ss.nonfinite) {
-          atomicAdd(&counters[FBS_CNT_NONFINITE], 1ull);
-          atomicOr(&hy->flags, kFlagNonfinite);
-        }
+        sig_S[l] = S;  // sigma_l by a slice update, on a warp of its own below
       } else {
+        double s2n;
         bool gcap = false, tcap = false;
         s2n = hyper_trunc_invgamma(0.5 * (G - 1.0), 0.5 * S, mc.s2[l], sig2, sig_g[l],
                                    sig_gcap[l] != 0, rs, &gcap, &tcap);
         if (gcap) atomicAdd(&counters[FBS_CNT_GAMMA_CAPS], 1ull);
         if (tcap) atomicAdd(&counters[FBS_CNT_TRUNC_CAPS], 1ull);
+        phi_new[2 + L + l] = s2n;
       }
       phi_new[2 + l] = th;
-      phi_new[2 + L + l] = s2n;
     }
   } else if (warp == 2) {
     // the first truncated-draw attempt of every sigma_l^2: a Gamma((G-1)/2) draw
@@ -549,6 +534,36 @@ __device__ __forceinline__ void hyper_body(const ModelConst& mc, const double* p
     }
   }
   if (tid == NT - 1) inv_k = 1.0 / (double)(sh.n_mom + 1);
+  if (kWide && mc.all_slice && warp != 0 && warp != 3) {
+    // all_slice (never in the 128-thread block of the FP32 form): slice updates of the
+    // sigma_l themselves on (0, s_l), each spread over a warp; the state keeps
+    // sigma_l^2.  One after the other on a lane each they were the kernel's longest
+    // part.
+    named_sync(6, 192);  // sig_S
+    const int slot = warp < 3 ? warp - 1 : warp - 2;
+    for (int l = slot; l < L; l += 6) {
+      Rng rs(mc.seed_lo, mc.seed_hi, mc.chain, kStreamSigma, (uint32_t)l, it32);
+      const double x0 = sqrt(sh.phi[2 + L + l]);
+      const SliceResult ss = slice_update_warp(x0, sh.w_hyp[1 + l],
+                                               SigDensity{G, 0.5 * sig_S[l], mc.s[l]}, rs, mc.K,
+                                               mc.shrink_max);
+      if (lane == 0) {
+        phi_new[2 + L + l] = ss.x * ss.x;
+        if (it <= sh.burnin) {
+          double w = sh.w_hyp[1 + l], waux = sh.waux_hyp[1 + l];
+          tune_width(w, waux, it, ss.x, x0, sh.burnin, sh.tune_start);
+          hy->w_hyp[1 + l] = w;
+          hy->waux_hyp[1 + l] = waux;
+        }
+        atomicAdd(&counters[FBS_CNT_EVALS_HYPER], (unsigned long long)ss.evals);
+        if (ss.capped) atomicAdd(&counters[FBS_CNT_SLICE_CAPS], 1ull);
+        if (ss.nonfinite) {
+          atomicAdd(&counters[FBS_CNT_NONFINITE], 1ull);
+          atomicOr(&hy->flags, kFlagNonfinite);
+        }
+      }
+    }
+  }
   __syncthreads();
 
   const bool mom = it > sh.burnin;

@@ -15,7 +15,7 @@
 // neither, and theirs involve no beta (Figure 3); the counter-based generator
 // gives every variable the same uniforms in either order.
 // With ModelConst::all_slice the gamma_g draw (gb kernel), tau (warp 0 of the
-// hyper kernel, after nu) and sigma_l (lane 32+l) are slice updates of the same
+// hyper kernel, after nu) and sigma_l (a warp each) are slice updates of the same
 // full conditionals instead, each variable with its own tuned width, as
 // Section 4.2 slice-samples every non-normal conditional.
 #include <cooperative_groups.h>
