@@ -39,8 +39,13 @@ int fail(int code, const std::string& msg) {
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Results of up to kPackMost bytes are read back in one copy if the staging area
-// holds them (see read_arrays); it has kPackBytes at least.
+// holds them (see read_arrays); it has kPackBytes at least, and room for the four
+// summaries of every beta and gamma.
 constexpr size_t kPackBytes = 256 << 10, kPackMost = 1 << 20;
+
+size_t stage_bytes(int N, int G, int L, size_t word) {
+  return std::max({(size_t)N * G * word, kPackBytes, 32 * (size_t)(L + 1) * G});
+}
 
 // Byte offsets of every device buffer inside one workspace.
 struct Layout {
@@ -65,7 +70,7 @@ Layout make_layout(int N, int G, int L, int nblk, long long trace_cap, int trace
   o.waux_eps = take(NG * 8);
   o.m_eps = take(NG * 8);
   o.q_eps = take(NG * 8);
-  o.mu = take(std::max(NG * 8, kPackBytes));  // also the staging area of read_arrays
+  o.mu = take(stage_bytes(N, G, L, 8));  // also the staging area of read_arrays
   o.beta = take(LG * 8);
   o.w_beta = take(LG * 8);
   o.waux_beta = take(LG * 8);
@@ -109,7 +114,7 @@ LayoutF32 make_layout_f32(int N, int G, int L, int nblk, long long trace_cap, in
   o.w_eps = take(NG * 4);
   o.waux_eps = take(NG * 4);
   o.mom_eps = take(4 * NG * 4);
-  o.mu = take(std::max(NG * 4, kPackBytes));  // also the staging area of read_arrays
+  o.mu = take(stage_bytes(N, G, L, 4));  // also the staging area of read_arrays
   o.beta = take(LG * 4);
   o.w_beta = take(LG * 4);
   o.waux_beta = take(LG * 4);
@@ -775,13 +780,13 @@ int fbs_init(fbs_handle** out, const int32_t* y, int N, int G, int gene_major, c
     y_raw = (int32_t*)f.mom_eps;
     d_pinv = (double*)(base + o32.pinv);
     h->stage = (char*)f.mu;
-    h->stage_cap = std::max((size_t)N * G * 4, kPackBytes);
+    h->stage_cap = stage_bytes(N, G, L, 4);
     if ((e = prepare_gene_kernel_f32(mc, h->block)) != cudaSuccess)
       return bail(FBS_E_CUDA, std::string("kernel attribute: ") + cudaGetErrorString(e));
   } else {
     h->p = carve(base, h->lay, mc.trace_beta);
     h->stage = (char*)h->p.mu;
-    h->stage_cap = std::max((size_t)N * G * 8, kPackBytes);
+    h->stage_cap = stage_bytes(N, G, L, 8);
     y_raw = (int32_t*)h->p.q_eps;
     d_pinv = (double*)(base + h->lay.pinv);
     if ((e = prepare_gene_kernel(N, h->block)) != cudaSuccess)
@@ -1649,6 +1654,7 @@ int pooled_read(int C, fbs_handle* const* chains, long long M, const std::vector
     }
     const size_t row = (size_t)q.R * k * 8;
     const size_t chunk = pack ? q.n : h0->stage_cap / row;
+    const bool small = !pack && q.n * row <= kPackBytes;  // one copy for this quantity
     for (size_t g0 = 0; g0 < q.n; g0 += chunk) {
       const size_t ng = std::min(chunk, q.n - g0), bytes = ng * q.R * 8;
       in.g0 = (long long)g0;
@@ -1657,13 +1663,18 @@ int pooled_read(int C, fbs_handle* const* chains, long long M, const std::vector
       for (size_t i = 0; i < k; ++i) {
         double* host = (*q.dst)[i];
         if (!host) continue;
-        if (pack)
+        if (pack || small)
           outs.push_back(StageOut{host, off + i * bytes, bytes});
         else
           FBS_CUDA(cudaMemcpyAsync(host + g0 * q.R, h0->stage + i * bytes, bytes,
                                    cudaMemcpyDeviceToHost, h0->s));
       }
       if (pack) off += bytes * k;
+    }
+    if (small) {
+      int rc = stage_fetch(h0, q.n * row, outs);
+      if (rc) return rc;
+      outs.clear();
     }
   }
   if (pack) return total ? stage_fetch(h0, total, outs) : FBS_OK;
@@ -2133,7 +2144,7 @@ int fbs_batch_init(fbs_batch** out, int C, const fbs_dataset* sets, const fbs_op
     carve_f32(base, lay[c], b->mcs[c].trace_beta, v->pf, v->p);
     b->pfs[c] = v->pf;
     v->stage = (char*)v->pf.mu;
-    v->stage_cap = std::max((size_t)ds.N * ds.G * 4, kPackBytes);
+    v->stage_cap = stage_bytes(ds.N, ds.G, ds.L, 4);
     if ((e = cudaEventCreateWithFlags(&v->ev_in, cudaEventDisableTiming)) != cudaSuccess ||
         (e = cudaEventCreateWithFlags(&v->ev_out, cudaEventDisableTiming)) != cudaSuccess)
       return bail(FBS_E_CUDA, cudaGetErrorString(e));
