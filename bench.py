@@ -90,21 +90,21 @@ def parse():
 # FP64 floating-point operations per slice log-density evaluation of the FP64
 # sweep kernels k_eps_f64 + k_gb_f64 (DFMA counted as 2, DADD and DMUL as 1),
 # from one ncu capture of each in a sampling sweep at config 1 (bench.py --form
-# f64 --profile-run 2): 1.339e8 (eps) + 1.000e8 (gb) flop per sweep over the
-# 6.141e6 log-density evaluations the device counted per sweep = 38.1.  The slice
-# comparisons are decided in FP32 (0.35% fall back to FP64), so this covers the
-# FP64 work that remains per evaluation on average (rates at accepted points,
-# log-rates, class sums and rate updates, gamma draws, interval arithmetic,
+# f64 --profile-run 2): 3.84e7 (eps) + 3.60e7 (gb) flop per sweep over the
+# 6.141e6 log-density evaluations the device counted per sweep = 12.1.  The slice
+# comparisons are decided in FP32 (about 2 in 1e5 fall back to FP64), so this
+# covers the FP64 work that remains per evaluation on average (rates at accepted
+# points, class sums and rate updates, gamma draws, interval arithmetic,
 # moments).  Re-measure when the kernels change.
-FP64_FLOP_PER_EVAL = 38.1
-FP64_TRAFFIC_BYTES = 44.1e6   # dram read+write of both kernels per sweep, same captures
+FP64_FLOP_PER_EVAL = 12.1
+FP64_TRAFFIC_BYTES = 44.6e6   # dram read+write of both kernels per sweep, same captures
 # FP32 forms: warp instructions issued per sweep (smsp__inst_executed.sum) by the
 # eps kernel and the gamma/beta kernel (k_gb_f32; with the learned proposal
 # k_gb_net_f32, which includes the network pass, in a sampling sweep after
 # calibration) and their dram read+write (writes stay in L2), from ncu captures
 # at config 1 (bench.py --profile-run)
-FP32_WARP_INST = {"f32": 21.01e6 + 9.12e6, "learned": 21.01e6 + 19.08e6}
-FP32_TRAFFIC_BYTES = {"f32": 19.7e6 + 13.24e6, "learned": 19.7e6 + 15.49e6}
+FP32_WARP_INST = {"f32": 20.78e6 + 10.23e6, "learned": 20.78e6 + 16.80e6}
+FP32_TRAFFIC_BYTES = {"f32": 19.7e6 + 13.22e6, "learned": 19.7e6 + 14.69e6}
 # issue peak: 152 SMs x 4 schedulers x 1 warp instruction per clock x 2.07 GHz
 ISSUE_PEAK_WARP_INST_S = 152 * 4 * 2.07e9
 # the proposal network's own flops per gene (2 x (F*64 + 64*64 + 64*K), F = 21,

@@ -8,8 +8,10 @@
 // number of 50 bits below the power of two above max |a| (the rounding is at
 // most 2^-51 of that power, against the 2^-53 |partial sum| which every FP64
 // addition of the sum makes), split into a signed high part and a 26-bit low
-// part, and the four partial products are accumulated exactly in 64 bits.  The
-// sums being exact, any split over threads gives the same result.
+// part, and the partial products are accumulated exactly in 64 bits: high x high,
+// low x low and (high + low) x (high + low) (Karatsuba: the third less
+// the first two is the sum of the cross products).  The sums being exact, any split
+// over threads gives the same result.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -72,16 +74,17 @@ __global__ void k_ess_mean(const double* __restrict__ tr, long long rows, long l
   const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= S) return;
   double m = 0.0;
-#pragma unroll 8
+#pragma unroll 16
   for (long long t = 0; t < rows; ++t) m += tr[t * S + s];
   mean[s] = m / (double)rows;
 }
 
-constexpr int kEssThreads = 512, kEssWarps = kEssThreads / 32;
-constexpr int kEssLags = 16;   // lags per round
-constexpr int kEssHalf = 8;    // lags per thread: 3 x 8 64-bit sums and a window of 8 values
-constexpr int kEssPad = 48;    // zero rows behind the series (a window reads up to 31 past the end)
-constexpr int kEssMaxRows = 5000;  // 2^50 rows < 2^63 needs rows < 8192; shared memory less
+constexpr int kEssThreads = 128, kEssWarps = kEssThreads / 32;
+constexpr int kEssBlocks = 4;  // per SM, where their shared memory fits
+constexpr int kEssLags = 16;   // lags per round while all series of a block go on
+constexpr int kEssPart = 8;    // lags per thread: 3 x 8 64-bit sums and a window of 8 values
+constexpr int kEssPad = 72;    // zero rows behind the series (a window reads up to 64 past the end)
+constexpr int kEssMaxRows = 8000;  // 2^50 rows < 2^63, and shared memory holds 9000
 
 struct Wide {  // a 128-bit integer sum
   long long hi;
@@ -91,60 +94,60 @@ struct Wide {  // a 128-bit integer sum
 __host__ __device__ constexpr size_t ess_smem_bytes(long long rows, int spb) {
   return (((size_t)(rows + kEssPad) * (spb + 1) * 8 + 15) & ~(size_t)15) +
          (size_t)(kEssWarps / 2) * kEssLags * spb * sizeof(Wide) + (size_t)kEssLags * spb * 8 +
-         (size_t)spb * 8 + (size_t)spb * 4 + 16;
+         2 * (size_t)spb * 8 + (size_t)spb * 4 + 16;
 }
 
-// SPB series per block.  The block keeps its series in shared memory (one read of
-// the trace; row stride SPB + 1, so that threads on different rows hit different
-// banks) and goes through the lags 16 at a time: a thread takes one series, 8 of
-// the lags and a range of rows, holds the 8 values ahead of its row in
-// registers, and per row reads two words and issues 32 multiply-adds.  Before
-// each round the block's threads are dealt out over the series that are not
-// finished yet (the lag at which a series ends varies from a few to hundreds),
-// so that the long ones get more threads and no lane waits.  Bound by the
-// 32 x 32 -> 64 multiply-add rate.  fbs_beta_ess of 30035 series of 1000 rows:
-// 145 ms with one thread per series in FP64, 8.0 ms with the threads fixed to
-// their series, 5.8 ms so.
+// SPB (4 or 2) series per block.  The block keeps its series in shared memory (one
+// read of the trace; row stride SPB + 1, so that threads on different rows hit
+// different banks) and goes through the lags in rounds: a thread takes one series,
+// 8 lags and a range of rows, holds the 8 values ahead of its row in registers, and
+// per row reads two words and issues 24 multiply-adds.  A round takes 16 lags of
+// SPB series; before each one the block's threads are dealt out over the series
+// that are not finished yet (the lag at which a series ends varies from a few to
+// hundreds): half the series, twice the lags, so that every round has the same
+// work and no lane waits.  Bound by the 32 x 32 -> 64 multiply-add rate and, at a
+// round's end, by barriers, which is why four small blocks share an SM (one works
+// while another waits).  fbs_beta_ess of 30035 series of 1000 rows: 145 ms with one
+// thread per series in FP64; with 16 series on 512 threads 8.0 ms with the threads
+// fixed to their series, 5.8 ms dealt out with 16 lags per round and four
+// multiply-adds per lag, 3.3 ms with three, up to 64 lags and the divisions off the
+// serial part; 2.7 ms with 8 series on 256 threads, 2.3 ms with 4 on 128,
+// 2.0 ms with the largest magnitude found in integers and one scale per series.
 template <int SPB>
-__global__ void __launch_bounds__(kEssThreads) k_ess_block(const double* __restrict__ tr, int rows,
-                                                           long long S, int L, int G,
-                                                           const double* __restrict__ mean,
-                                                           double* __restrict__ ess) {
+__global__ void __launch_bounds__(kEssThreads, kEssBlocks)
+    k_ess_block(const double* __restrict__ tr, int rows, long long S, int L, int G,
+                const double* __restrict__ mean, double* __restrict__ ess) {
   extern __shared__ __align__(16) unsigned char sm_ess[];
-  constexpr int ST = SPB + 1;
+  constexpr int ST = SPB + 1, LW = SPB == 4 ? 2 : 1;  // log2 SPB
   int2* A = reinterpret_cast<int2*>(sm_ess);  // [rows + kEssPad][ST]
   double* Ad = reinterpret_cast<double*>(sm_ess);
   Wide* red = reinterpret_cast<Wide*>(sm_ess + (((size_t)(rows + kEssPad) * ST * 8 + 15) & ~(size_t)15));
   double* ckd = reinterpret_cast<double*>(red + kEssWarps / 2 * kEssLags * SPB);  // [kEssLags][SPB]
-  double* mx = ckd + kEssLags * SPB;               // [SPB]
-  int* list = reinterpret_cast<int*>(mx + SPB);    // [SPB] unfinished series
+  double* scale = ckd + kEssLags * SPB;            // [SPB]
+  double* c0 = scale + SPB;                        // [SPB] variances
+  int* list = reinterpret_cast<int*>(c0 + SPB);    // [SPB] unfinished series
   int* n_list = list + SPB;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 
-  // centred values and their largest magnitude
+  // centred values and their largest magnitude (compared as integers: the order of
+  // the magnitudes, with infinity and NaN above all)
   {
     constexpr int NSEG = kEssThreads / SPB;
     const int sl = tid % SPB, seg = tid / SPB;
     const long long s = (long long)blockIdx.x * SPB + sl;
     const bool on = s < S;
     const double m = on ? mean[s] : 0.0;
-    double big = 0.0;
-    int bad = 0;
+    unsigned long long big = 0;
 #pragma unroll 4
     for (int t = seg; t < rows; t += NSEG) {
       const double a = on ? tr[(long long)t * S + s] - m : 0.0;
-      bad |= !isfinite(a);
-      big = fmax(big, fabs(a));
+      big = max(big, (unsigned long long)__double_as_longlong(a) & ~(1ull << 63));
       Ad[t * ST + sl] = a;
     }
     for (int t = rows + seg; t < rows + kEssPad; t += NSEG) A[t * ST + sl] = make_int2(0, 0);
 #pragma unroll
-    for (int o = SPB; o < 32; o <<= 1) {
-      big = fmax(big, __shfl_xor_sync(0xffffffffu, big, o));
-      bad |= __shfl_xor_sync(0xffffffffu, bad, o);
-    }
-    if (bad) big = INFINITY;
-    if (lane < SPB) reinterpret_cast<double*>(red)[warp * SPB + lane] = big;
+    for (int o = SPB; o < 32; o <<= 1) big = max(big, __shfl_xor_sync(0xffffffffu, big, o));
+    if (lane < SPB) reinterpret_cast<unsigned long long*>(red)[warp * SPB + lane] = big;
   }
   __syncthreads();
 
@@ -159,12 +162,14 @@ __global__ void __launch_bounds__(kEssThreads) k_ess_block(const double* __restr
   };
   if (warp == 0) {
     if (lane < SPB) {
-      double b = 0.0;
-      for (int w = 0; w < kEssWarps; ++w) b = fmax(b, reinterpret_cast<double*>(red)[w * SPB + lane]);
-      mx[lane] = b;
+      unsigned long long big = 0;
+      for (int w = 0; w < kEssWarps; ++w)
+        big = max(big, reinterpret_cast<unsigned long long*>(red)[w * SPB + lane]);
+      const double b = __longlong_as_double((long long)big);
       // a constant series (every residual zero) has ess = rows; a range of values
       // that fixed point or its squares do not hold is left to ess_series
       act = mine && b > 0x1p-400 && b < 0x1p400;
+      scale[lane] = act ? scalbn(1.0, 49 - ilogb(b)) : 0.0;
       if (mine && !act)
         ess[ess_slot(s_mine, L, G)] = b == 0.0 ? (double)rows : ess_series(tr, rows, S, s_mine);
     }
@@ -175,103 +180,126 @@ __global__ void __launch_bounds__(kEssThreads) k_ess_block(const double* __restr
   int n_act = *n_list;
 
   // fixed point: |a| 2^(49 - e) <= 2^50 with 2^e <= max |a|
-  for (int i = tid; i < rows * n_act; i += kEssThreads) {
-    const int sl = list[i % n_act], at = (i / n_act) * ST + sl;
-    const long long v = __double2ll_rn(Ad[at] * scalbn(1.0, 49 - ilogb(mx[sl])));
+  for (int i = tid; i < rows * SPB; i += kEssThreads) {
+    const int at = i / SPB * ST + i % SPB;
+    const long long v = __double2ll_rn(Ad[at] * scale[i % SPB]);
     const int hi = (int)((v + (1ll << 25)) >> 26);
     A[at] = make_int2(hi, (int)(v - ((long long)hi << 26)));
   }
   __syncthreads();
 
   const double n = (double)rows;
-  double c0 = 0.0, sum = 0.0, prev = INFINITY;  // of this lane's series (warp 0)
-  for (int k0 = 0; n_act > 0; k0 += kEssLags) {
-    // thread: entry q of the list, lags k0 + 8 half .. + 7, rows t0 .. t1 - 1
+  double sum = 0.0, prev = INFINITY;  // of this lane's series (warp 0)
+  for (int k0 = 0, lags; n_act > 0; k0 += lags) {
+    // thread: entry q of the list, lags k0 + 8 part .. + 7, rows t0 .. t1 - 1
     const int lw = 32 - __clz(n_act - 1);  // log2 of the list's length, rounded up
-    const int q = tid & ((1 << lw) - 1), half = (tid >> lw) & 1, seg = tid >> (lw + 1);
+    lags = kEssLags << (LW - lw);
+    const int q = tid & ((1 << lw) - 1), part = (tid & (2 * SPB - 1)) >> lw;
+    constexpr int nseg = kEssThreads / (2 * SPB);
+    const int seg = tid / (2 * SPB);
     const int m = rows - k0;  // terms of lag k0 (the rows past the end are zero)
-    const int nseg = kEssThreads >> (lw + 1);
     const int per = ((m + nseg - 1) / nseg) | 1;  // odd: threads on different banks
     const int t0 = seg * per, t1 = min(m, t0 + per);
-    long long hh[kEssHalf], md[kEssHalf], ll[kEssHalf];
+    long long hh[kEssPart], ss[kEssPart], ll[kEssPart];
 #pragma unroll
-    for (int j = 0; j < kEssHalf; ++j) hh[j] = md[j] = ll[j] = 0;
+    for (int j = 0; j < kEssPart; ++j) hh[j] = ss[j] = ll[j] = 0;
     if (q < n_act && t0 < t1) {
-      const int2* a = A + list[q];
-      const int k = k0 + half * kEssHalf;
-      int2 w[kEssHalf];
+      const int2* a = A + list[q] + t0 * ST;
+      const int2* b = a + (k0 + part * kEssPart) * ST;
+      int2 w[kEssPart];
+      int ws[kEssPart];
 #pragma unroll
-      for (int j = 0; j < kEssHalf; ++j) w[j] = a[(t0 + k + j) * ST];
-      for (int tb = t0; tb < t1; tb += kEssHalf) {
+      for (int j = 0; j < kEssPart; ++j) {
+        w[j] = b[j * ST];
+        ws[j] = w[j].x + w[j].y;
+      }
+      auto row = [&](int i) {  // row i of eight: the window starts at w[i]
+        const int2 x = a[i * ST];
+        const int xs = x.x + x.y;
 #pragma unroll
-        for (int i = 0; i < kEssHalf; ++i) {
-          int2 x = a[(tb + i) * ST];
-          if (tb + i >= t1) x = make_int2(0, 0);
-#pragma unroll
-          for (int j = 0; j < kEssHalf; ++j) {
-            const int2 v = w[(i + j) % kEssHalf];
-            hh[j] += (long long)x.x * v.x;
-            ll[j] += (long long)x.y * v.y;
-          }
-#pragma unroll
-          for (int j = 0; j < kEssHalf; ++j) md[j] += (long long)x.x * w[(i + j) % kEssHalf].y;
-#pragma unroll
-          for (int j = 0; j < kEssHalf; ++j) md[j] += (long long)x.y * w[(i + j) % kEssHalf].x;
-          w[i] = a[(tb + i + k + kEssHalf) * ST];
+        for (int j = 0; j < kEssPart; ++j) {
+          const int2 v = w[(i + j) % kEssPart];
+          hh[j] += (long long)x.x * v.x;
+          ll[j] += (long long)x.y * v.y;
+          ss[j] += (long long)xs * ws[(i + j) % kEssPart];
         }
+        w[i] = b[(i + kEssPart) * ST];
+        ws[i] = w[i].x + w[i].y;
+      };
+      int left = t1 - t0;
+      for (; left >= kEssPart; left -= kEssPart, a += kEssPart * ST, b += kEssPart * ST) {
+#pragma unroll
+        for (int i = 0; i < kEssPart; ++i) row(i);
+      }
+#pragma unroll
+      for (int i = 0; i < kEssPart - 1; ++i) {
+        if (i >= left) break;
+        row(i);
       }
     }
-    for (int o = 2 << lw; o < 32; o <<= 1) {
 #pragma unroll
-      for (int j = 0; j < kEssHalf; ++j) {
+    for (int o = 2 * SPB; o < 32; o <<= 1) {
+#pragma unroll
+      for (int j = 0; j < kEssPart; ++j) {
         hh[j] += __shfl_xor_sync(0xffffffffu, hh[j], o);
-        md[j] += __shfl_xor_sync(0xffffffffu, md[j], o);
+        ss[j] += __shfl_xor_sync(0xffffffffu, ss[j], o);
         ll[j] += __shfl_xor_sync(0xffffffffu, ll[j], o);
       }
     }
-    // the warps' sums: the upper half of the warps first, the lower half adds its own
-    Wide* slot = red + ((size_t)(warp % (kEssWarps / 2)) * kEssLags + half * kEssHalf) * SPB + q;
-    const bool writes = lane < (2 << lw) && q < n_act;
+    // the warps' sums, [lag][series of the list]: the upper half of the warps first,
+    // the lower half adds its own
+    Wide* slot = red + (size_t)(warp % (kEssWarps / 2)) * kEssLags * SPB + (part * kEssPart << lw) + q;
+    const bool writes = lane < 2 * SPB && q < n_act;
 #pragma unroll
     for (int step = 0; step < 2; ++step) {
       if (writes && (warp >= kEssWarps / 2) == (step == 0)) {
 #pragma unroll
-        for (int j = 0; j < kEssHalf; ++j) {
-          __int128 v = ((__int128)hh[j] << 52) + ((__int128)md[j] << 26) + ll[j];
-          if (step == 1) v += ((__int128)slot[j * SPB].hi << 64) + slot[j * SPB].lo;
-          slot[j * SPB] = Wide{(long long)(v >> 64), (unsigned long long)v};
+        for (int j = 0; j < kEssPart; ++j) {
+          __int128 v = ((__int128)hh[j] << 52) + ((__int128)(ss[j] - hh[j] - ll[j]) << 26) + ll[j];
+          if (step == 1) v += ((__int128)slot[j << lw].hi << 64) + slot[j << lw].lo;
+          slot[j << lw] = Wide{(long long)(v >> 64), (unsigned long long)v};
         }
       }
       __syncthreads();
     }
-    for (int i = tid; i < kEssLags * SPB; i += kEssThreads) {
-      if (i % SPB >= n_act) continue;
-      __int128 v = 0;
+    {
+      // a thread per lag and series: the autocorrelation (the divisions here, not in
+      // warp 0's loop below)
+      const bool on = tid < kEssLags * SPB && q < n_act;
+      const int sl = on ? list[q] : 0;
+      double ck = 0.0;
+      if (on) {
+        __int128 v = 0;
 #pragma unroll
-      for (int w = 0; w < kEssWarps / 2; ++w) {
-        const Wide x = red[w * kEssLags * SPB + i];
-        v += ((__int128)x.hi << 64) + x.lo;
+        for (int w = 0; w < kEssWarps / 2; ++w) {
+          const Wide x = red[w * kEssLags * SPB + tid];
+          v += ((__int128)x.hi << 64) + x.lo;
+        }
+        ck = ((double)(long long)(v >> 64) * 0x1p64 + (double)(unsigned long long)v) / n;
       }
-      ckd[i] = (double)(long long)(v >> 64) * 0x1p64 + (double)(unsigned long long)v;
+      if (k0 == 0) {
+        if (on && tid < 1 << lw) c0[sl] = ck;
+        __syncthreads();
+      }
+      if (on) ckd[tid] = ck / c0[sl];
     }
     __syncthreads();
     if (warp == 0) {
       const unsigned todo = __ballot_sync(0xffffffffu, act);
       if (act) {
         const double* ck = ckd + __popc(todo & ((1u << lane) - 1u));
-        if (k0 == 0) c0 = ck[0] / n;
         bool go = true;
-        for (int j = 0; j < kEssLags && go; j += 2) {
+        for (int j = 0; j < lags && go; j += 2) {
           go = false;
           if (k0 + j + 1 >= rows) break;
-          double pair = ck[j * SPB] / n / c0 + ck[(j + 1) * SPB] / n / c0;
+          double pair = ck[j << lw] + ck[(j + 1) << lw];
           if (!(pair > 0.0)) break;
           if (pair > prev) pair = prev;
           sum += pair;
           prev = pair;
           go = true;
         }
-        if (!go || k0 + kEssLags >= rows) {
+        if (!go || k0 + lags >= rows) {
           double tau = -1.0 + 2.0 * sum;
           if (tau < 1.0 / n) tau = 1.0 / n;
           ess[ess_slot(s_mine, L, G)] = n / tau;
@@ -300,13 +328,12 @@ cudaError_t launch_block(const double* tr, int rows, long long S, int L, int G,
 
 }  // namespace
 
-// mean: S doubles of scratch.  16 series per block where their rows fit its
-// shared memory (about 1400) and the blocks then fill the chip, else 8 (2900) or
-// 4 (5000); longer traces take one thread per series.
+// mean: S doubles of scratch.  4 series per block where four such blocks fit an SM
+// (1295 rows), else 2 (2000 rows of 15000 series: 2.9 ms against 3.6 ms
+// with 4; 4000 rows of 10000: 5.6 against 8.0); longer traces take one thread per
+// series.
 cudaError_t launch_ess(const double* tr, long long rows, int L, int G, double* mean, double* ess,
                        cudaStream_t s) {
-  constexpr size_t kSmem = 227 * 1024;
-  constexpr long long kBlocks = 152;
   const long long S = (long long)L * G;
   const int blk = 128;
   const unsigned grid = (unsigned)((S + blk - 1) / blk);
@@ -317,11 +344,10 @@ cudaError_t launch_ess(const double* tr, long long rows, int L, int G, double* m
   k_ess_mean<<<grid, blk, 0, s>>>(tr, rows, S, mean);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  if (ess_smem_bytes(rows, 16) <= kSmem && S >= 16 * kBlocks)
-    return launch_block<16>(tr, (int)rows, S, L, G, mean, ess, s);
-  if (ess_smem_bytes(rows, 8) <= kSmem && S >= 8 * kBlocks)
-    return launch_block<8>(tr, (int)rows, S, L, G, mean, ess, s);
-  return launch_block<4>(tr, (int)rows, S, L, G, mean, ess, s);
+  // an SM's shared memory, 1 KB per block its own
+  if (kEssBlocks * (ess_smem_bytes(rows, 4) + 1024) <= 228 * 1024)
+    return launch_block<4>(tr, (int)rows, S, L, G, mean, ess, s);
+  return launch_block<2>(tr, (int)rows, S, L, G, mean, ess, s);
 }
 
 }  // namespace fbs

@@ -48,3 +48,15 @@ def test_beta_ess_of_series_that_never_move():
     assert np.ptp(s.trace(beta=True)["beta"], axis=0).max() == 0.0
     _check(s, 77, 180)
     s.close()
+
+
+@pytest.mark.parametrize("rows,G", [(64, 31), (250, 503), (1000, 503), (1295, 487), (1296, 487),
+                                    (8000, 31), (8001, 31)])
+def test_beta_ess_of_series_that_mix_slowly(rows, G):
+    """Series that end after a few dozen to hundreds of lags: rounds with few of them left."""
+    d = synthetic.make_config(1, G=G)
+    s = fbs.Sampler(d["y"], d["X"], d["h"], d["priors"], seed=rows, precision=fbs.FBS_F32,
+                    trace_cap=rows, trace_beta=1)
+    s.run(rows + 200, burnin=200, thin=1)
+    _check(s, rows, 120)
+    s.close()
