@@ -408,20 +408,50 @@ __device__ __forceinline__ void grid_dep_launch() {
 constexpr uint32_t kTrainTmemCols = 512;
 constexpr int kTrainOutPad = (kMaxOut + 15) & ~15;
 
-// Writes 32 FP32 columns of this thread's tensor-memory lane and waits for the
+// Writes 16 FP32 columns of this thread's tensor-memory lane and waits for the
 // store.
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const float* v) {
-  asm volatile(
-      "tcgen05.st.sync.aligned.32x32b.x32.b32 [%0], "
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};" ::"r"(taddr),
-      "f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]),
-      "f"(v[8]), "f"(v[9]), "f"(v[10]), "f"(v[11]), "f"(v[12]), "f"(v[13]), "f"(v[14]),
-      "f"(v[15]), "f"(v[16]), "f"(v[17]), "f"(v[18]), "f"(v[19]), "f"(v[20]), "f"(v[21]),
-      "f"(v[22]), "f"(v[23]), "f"(v[24]), "f"(v[25]), "f"(v[26]), "f"(v[27]), "f"(v[28]),
-      "f"(v[29]), "f"(v[30]), "f"(v[31])
-      : "memory");
+__device__ __forceinline__ void tmem_st16f(uint32_t taddr, const float* v) {
+  uint32_t r[16];
+#pragma unroll
+  for (int i = 0; i < 16; ++i) r[i] = __float_as_uint(v[i]);
+  tmem_st16(taddr, r);
   asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+}
+
+// A hidden layer of a training step, forward: the activations into the operand rows
+// at dst, GELU's derivative in place of Z at z.  As in the network pass the columns
+// are a loop of 16: in line (64 columns per layer, forward and backward) a block of
+// four warps spent most of its time waiting for instructions it runs once (a call
+// of 123 steps of 8192 rows at L = 5: 4.17 ms, and 3.18 ms so).
+__device__ __forceinline__ void train_hidden(uint32_t z, const float* b, uint8_t* dst, uint32_t sbo,
+                                             int ch_hi, int ch_lo) {
+#pragma unroll 1
+  for (int c0 = 0; c0 < kMlpHidden; c0 += 16) {
+    float v[16], gd[16];
+    tmem_ld16(z + (uint32_t)c0, v);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) gelu_and_grad_f(v[i] + b[c0 + i], &v[i], &gd[i]);
+    tmem_st16f(z + (uint32_t)c0, gd);
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      store_split8_ch(dst, sbo, threadIdx.x, ch_hi + c0 / 8 + q, ch_lo + c0 / 8 + q, v + 8 * q);
+  }
+}
+
+// Backward: the gradient at d times GELU's derivative at z into the rows at dst.
+__device__ __forceinline__ void train_hidden_back(uint32_t d, uint32_t z, uint8_t* dst,
+                                                  uint32_t sbo, int ch_hi, int ch_lo) {
+#pragma unroll 1
+  for (int c0 = 0; c0 < kMlpHidden; c0 += 16) {
+    float v[16], gd[16];
+    tmem_ld16(d + (uint32_t)c0, v);
+    tmem_ld16(z + (uint32_t)c0, gd);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) v[i] *= gd[i];
+#pragma unroll
+    for (int q = 0; q < 2; ++q)
+      store_split8_ch(dst, sbo, threadIdx.x, ch_hi + c0 / 8 + q, ch_lo + c0 / 8 + q, v + 8 * q);
+  }
 }
 
 // Gaussian head, per row: loss = |u|^2 / 2 + sum log C_ll with C u = beta - mu;
@@ -670,34 +700,16 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
                 sbo_f, sW1, sW1 + cx * 128, 256, 128, t.sbo_w1);
   });
   if (ok) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float v[32];
-      float gd[32];
-      tmem_ld32(tm + la + 32 * h, v);
-#pragma unroll
-      for (int i = 0; i < 32; ++i) gelu_and_grad_f(v[i] + bsm[32 * h + i], &v[i], &gd[i]);
-      tmem_st32(tm + la + 32 * h, gd);  // Z1 becomes gelu'(Z1 + b1)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) store_split8_ch(bF, sbo_f, tid, 4 * h + q, 4 * h + q + half, v + 8 * q);
-    }
+    // Z1 becomes gelu'(Z1 + b1)
+    train_hidden(tm + la, bsm, bF, sbo_f, 0, half);
     ok = tc_run(c, &s_abort, [&] {  // Z2 = A1 W2^T
       issue_split(tm + 64, umma_idesc_bf16(128, H), 4, sF, sF + hb, 256, 128, sbo_f, sW2,
                   sW2 + 8 * 128, 256, 128, 2048);
     });
   }
   if (ok) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float v[32];
-      float gd[32];
-      tmem_ld32(tm + la + 64 + 32 * h, v);
-#pragma unroll
-      for (int i = 0; i < 32; ++i) gelu_and_grad_f(v[i] + bsm[H + 32 * h + i], &v[i], &gd[i]);
-      tmem_st32(tm + la + 64 + 32 * h, gd);  // Z2 becomes gelu'(Z2 + b2)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) store_split8_ch(bG, 4096, tid, 8 + 4 * h + q, 24 + 4 * h + q, v + 8 * q);
-    }
+    // Z2 becomes gelu'(Z2 + b2)
+    train_hidden(tm + la + 64, bsm + H, bG, 4096, 8, 24);
     ok = tc_run(c, &s_abort, [&] {  // O = A2 W3^T
       issue_split(tm + 128, umma_idesc_bf16(128, n3), 4, sG + 8 * 128, sG + 24 * 128, 256, 128,
                   4096, sW3, sW3 + 8 * 128, 256, 128, 2048);
@@ -728,32 +740,14 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
   }
   // ---- backward
   if (ok) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float d[32], z[32];
-      tmem_ld32(tm + la + 192 + 32 * h, d);
-      tmem_ld32(tm + la + 64 + 32 * h, z);  // gelu'(Z2 + b2)
-#pragma unroll
-      for (int i = 0; i < 32; ++i) d[i] *= z[i];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) store_split8_ch(bG, 4096, tid, 4 * h + q, 16 + 4 * h + q, d + 8 * q);
-    }
+    train_hidden_back(tm + la + 192, tm + la + 64, bG, 4096, 0, 16);
     ok = tc_run(c, &s_abort, [&] {  // G2 W2 (W2 read as an MN-major B)
       issue_split(tm + 256, umma_idesc_bf16_mn(128, H, 0, 1), 4, sG, sG + 16 * 128, 256, 128,
                   4096, sW2, sW2 + 8 * 128, 4096, 2048, 128);
     });
   }
   if (ok) {
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      float d[32], z[32];
-      tmem_ld32(tm + la + 256 + 32 * h, d);
-      tmem_ld32(tm + la + 32 * h, z);  // gelu'(Z1 + b1)
-#pragma unroll
-      for (int i = 0; i < 32; ++i) d[i] *= z[i];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) store_split8_ch(bG1, 2048, tid, 4 * h + q, 8 + 4 * h + q, d + 8 * q);
-    }
+    train_hidden_back(tm + la + 256, tm + la, bG1, 2048, 0, 8);
     // the weight gradients: K = the block's 128 rows, both operands MN-major
     ok = tc_run(c, &s_abort, [&] {
       issue_split(tm + 320, umma_idesc_bf16_mn(128, H + k1 + n3, 1, 1), 8, sG, sG + 16 * 128,
@@ -772,12 +766,12 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
               ob3 = oW3 + K * H;
     if (warp < 2) {
       // first product, rows 0..63 (unit of G2): dW2 in columns 0..63, db2 in column 64 + F
+#pragma unroll 1
+      for (int c0 = 0; c0 < H; c0 += 16) {
+        float v[16];
+        tmem_ld16(tm + la + 320 + (uint32_t)c0, v);
 #pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float v[32];
-        tmem_ld32(tm + la + 320 + 32 * h, v);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) out[oW2 + tid * H + 32 * h + i] = v[i];
+        for (int i = 0; i < 16; ++i) out[oW2 + tid * H + c0 + i] = v[i];
       }
       {
         float v[16];
@@ -789,16 +783,16 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
       }
       // second product, rows 0..63 (feature m of X, then the ones at m = F):
       // dW1^T and db1 in columns 0..63
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        float v[32];
-        tmem_ld32(tm + la + 128 + 32 * h, v);
+#pragma unroll 1
+      for (int c0 = 0; c0 < H; c0 += 16) {
+        float v[16];
+        tmem_ld16(tm + la + 128 + (uint32_t)c0, v);
         if (tid < F) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) out[oW1 + (32 * h + i) * F + tid] = v[i];
+          for (int i = 0; i < 16; ++i) out[oW1 + (c0 + i) * F + tid] = v[i];
         } else if (tid == F) {
 #pragma unroll
-          for (int i = 0; i < 32; ++i) out[ob1 + 32 * h + i] = v[i];
+          for (int i = 0; i < 16; ++i) out[ob1 + c0 + i] = v[i];
         }
       }
     } else {

@@ -247,26 +247,6 @@ __device__ __forceinline__ float gelu_fast(float x) {
   return __fdividef(x, 1.0f + __expf(-2.0f * u));
 }
 
-// 32 consecutive FP32 columns of this thread's TMEM lane (one load, one wait).
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
-  uint32_t r[32];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
-        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]),
-        "=r"(r[14]), "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]),
-        "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]),
-        "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-
-
 // Tensor-memory A operands: 16-bit elements packed two per 32-bit column (element
 // 2c in the low half of column c), row m in lane m.
 __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
@@ -318,24 +298,31 @@ __device__ __forceinline__ void issue_layer_ta(uint32_t d, uint32_t a, uint32_t 
       acc = 1u;
     }
 }
-// Bias, GELU and the split tensor-memory store of this thread's 32 columns c0.. of a
-// hidden layer (D at taddr_d, the next layer's A at a_hi / a_hi + 32).
+// Bias, GELU and the split tensor-memory store of a hidden layer's row (D at taddr_d,
+// the next layer's A at a_hi / a_hi + 32).  A warp walks this code once per sweep
+// and waits for its instructions more than for the tensor memory, so the loop over
+// the columns stays a loop, 16 of them at a time (N=16 G=40000 L=5: k_gb_net_f32
+// 34.5 us with 64 columns in line, 33.6 with 32, 33.4 with 16; k_proposal_tc 20.6,
+// 19.5, 17.9).
 __device__ __forceinline__ void hidden_epilogue_ta(uint32_t taddr_d, const float* bias,
-                                                   uint32_t a_hi, int c0) {
-  float v[32];
-  tmem_ld32(taddr_d, v);
+                                                   uint32_t a_hi) {
+#pragma unroll 1
+  for (int c0 = 0; c0 < kMlpHidden; c0 += 16) {
+    float v[16];
+    tmem_ld16(taddr_d + (uint32_t)c0, v);
 #pragma unroll
-  for (int i = 0; i < 32; i += 4) {
-    const float4 bb = *reinterpret_cast<const float4*>(bias + c0 + i);
-    v[i] = gelu_fast(v[i] + bb.x);
-    v[i + 1] = gelu_fast(v[i + 1] + bb.y);
-    v[i + 2] = gelu_fast(v[i + 2] + bb.z);
-    v[i + 3] = gelu_fast(v[i + 3] + bb.w);
+    for (int i = 0; i < 16; i += 4) {
+      const float4 bb = *reinterpret_cast<const float4*>(bias + c0 + i);
+      v[i] = gelu_fast(v[i] + bb.x);
+      v[i + 1] = gelu_fast(v[i + 1] + bb.y);
+      v[i + 2] = gelu_fast(v[i + 2] + bb.z);
+      v[i + 3] = gelu_fast(v[i + 3] + bb.w);
+    }
+    uint32_t hi[8], lo[8];
+    pack_split<8>(v, hi, lo);
+    tmem_st8(a_hi + (uint32_t)(c0 / 2), hi);
+    tmem_st8(a_hi + 32u + (uint32_t)(c0 / 2), lo);
   }
-  uint32_t hi[16], lo[16];
-  pack_split<16>(v, hi, lo);
-  tmem_st16(a_hi + (uint32_t)(c0 / 2), hi);
-  tmem_st16(a_hi + 32u + (uint32_t)(c0 / 2), lo);
 }
 
 constexpr uint32_t kTmemCols = 128;  // accumulators at columns 0..63, A operands at 64..127
@@ -468,6 +455,7 @@ __device__ __forceinline__ bool tc_tile(TcBlock& c, const ModelConst& mc, const 
   // three layers: D1 = A1 W1^T, D2 = A2 W2^T, D3 = A3 W3^T, each D at columns 0..;
   // A2, A3 overwrite the A columns once the product before them has completed
   const uint32_t ta = c.tmem + 64u;
+#pragma unroll 1
   for (int layer = 0; layer < 3; ++layer) {
     tc_fence_before();
     __syncthreads();
@@ -486,11 +474,10 @@ __device__ __forceinline__ bool tc_tile(TcBlock& c, const ModelConst& mc, const 
     c.ph ^= 1u;
     tc_fence_after();
     if (layer < 2) {
-      const float* bl = bias + layer * kMlpHidden;
-      hidden_epilogue_ta(c.tmem + lane_addr, bl, a_col, 0);
-      hidden_epilogue_ta(c.tmem + lane_addr + 32u, bl, a_col, 32);
+      hidden_epilogue_ta(c.tmem + lane_addr, bias + layer * kMlpHidden, a_col);
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     } else {
+#pragma unroll 1
       for (int c0 = 0; c0 < t.n3; c0 += 16) {
         float v[16];
         tmem_ld16(c.tmem + lane_addr + (uint32_t)c0, v);
