@@ -103,7 +103,7 @@ FP64_TRAFFIC_BYTES = 44.6e6   # dram read+write of both kernels per sweep, same 
 # k_gb_net_f32, which includes the network pass, in a sampling sweep after
 # calibration) and their dram read+write (writes stay in L2), from ncu captures
 # at config 1 (bench.py --profile-run)
-FP32_WARP_INST = {"f32": 20.78e6 + 10.23e6, "learned": 20.78e6 + 16.80e6}
+FP32_WARP_INST = {"f32": 20.78e6 + 10.23e6, "learned": 20.78e6 + 16.90e6}
 FP32_TRAFFIC_BYTES = {"f32": 19.7e6 + 13.22e6, "learned": 19.7e6 + 14.69e6}
 # issue peak: 152 SMs x 4 schedulers x 1 warp instruction per clock x 2.07 GHz
 ISSUE_PEAK_WARP_INST_S = 152 * 4 * 2.07e9

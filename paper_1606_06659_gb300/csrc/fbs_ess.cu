@@ -68,14 +68,32 @@ __global__ void k_ess(const double* __restrict__ tr, long long rows, long long S
 }
 
 // The mean of every series, rows added in order (a constant series then has the
-// same residuals, zero or not, as in ess_series).
-__global__ void k_ess_mean(const double* __restrict__ tr, long long rows, long long S,
-                           double* __restrict__ mean) {
+// same residuals, zero or not, as in ess_series).  A few warps per SM and one chain
+// of additions per series: bound by the latency of the reads, so the next 32 rows
+// are on their way while 32 are added (30035 series of 1000 rows: fbs_beta_ess 2.0 ms
+// with 16 rows unrolled in 32 registers, 1.85 ms so).
+__global__ void __launch_bounds__(64) k_ess_mean(const double* __restrict__ tr, long long rows,
+                                                 long long S, double* __restrict__ mean) {
   const long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= S) return;
-  double m = 0.0;
-#pragma unroll 16
-  for (long long t = 0; t < rows; ++t) m += tr[t * S + s];
+  constexpr int R = 32;
+  const double* x = tr + s;
+  const long long full = rows / R * R;
+  double m = 0.0, v[R];
+#pragma unroll
+  for (int i = 0; i < R; ++i) v[i] = i < rows ? x[i * S] : 0.0;
+  for (long long t = 0; t < full; t += R) {
+    double w[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) w[i] = t + R + i < rows ? x[(t + R + i) * S] : 0.0;
+#pragma unroll
+    for (int i = 0; i < R; ++i) m += v[i];
+#pragma unroll
+    for (int i = 0; i < R; ++i) v[i] = w[i];
+  }
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+    if (full + i < rows) m += v[i];
   mean[s] = m / (double)rows;
 }
 
@@ -112,7 +130,8 @@ __host__ __device__ constexpr size_t ess_smem_bytes(long long rows, int spb) {
 // fixed to their series, 5.8 ms dealt out with 16 lags per round and four
 // multiply-adds per lag, 3.3 ms with three, up to 64 lags and the divisions off the
 // serial part; 2.7 ms with 8 series on 256 threads, 2.3 ms with 4 on 128,
-// 2.0 ms with the largest magnitude found in integers and one scale per series.
+// 2.0 ms with the largest magnitude found in integers and one scale per series; 1.85
+// ms with the means read ahead.
 template <int SPB>
 __global__ void __launch_bounds__(kEssThreads, kEssBlocks)
     k_ess_block(const double* __restrict__ tr, int rows, long long S, int L, int G,
@@ -341,7 +360,7 @@ cudaError_t launch_ess(const double* tr, long long rows, int L, int G, double* m
     k_ess<<<grid, blk, 0, s>>>(tr, rows, S, L, G, ess);
     return cudaGetLastError();
   }
-  k_ess_mean<<<grid, blk, 0, s>>>(tr, rows, S, mean);
+  k_ess_mean<<<(unsigned)((S + 63) / 64), 64, 0, s>>>(tr, rows, S, mean);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   // an SM's shared memory, 1 KB per block its own
