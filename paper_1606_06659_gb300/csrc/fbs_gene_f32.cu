@@ -966,8 +966,9 @@ static size_t gb_net_smem_bytes(const ModelConst& mc) {
 // gamma/beta updates.  A kernel of its own, so that the plain gamma/beta kernel
 // keeps its own register allocation.  kBlocks: resident blocks per SM it is
 // compiled for: 3 (154 registers) while the genes fit them, else 4 (128, a few
-// spilled).  N=16 L=5: 34.6 against 35.7 us at G = 40000, 61.9 against 41.7 at 59500
-// (one block more than 3 per SM hold), 99 against 79 at 120000.
+// spilled).  N=16 L=5: 34.6 against 35.7 us at G = 40000 (33.4 since the network's
+// columns are loops), 61.9 against 41.7 at 59500 (one block more than 3 per SM hold),
+// 99 against 79 at 120000.
 template <int kBlocks>
 __global__ void __launch_bounds__(128, kBlocks) k_gb_net_f32(ModelConst mc, DevPtrsF32 p, int seg_i,
                                                     const uint8_t* __restrict__ img) {

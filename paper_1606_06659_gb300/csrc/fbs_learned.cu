@@ -998,7 +998,7 @@ cudaError_t launch_mlp_grad(const float* params, int L, int Bsz, const float* fb
 // A step's kernels overlap at their edges: the reduction's blocks are launched
 // while the gradient kernel writes its sums, and the next step's blocks draw,
 // gather and split their rows beside the reduction.  33.8 -> 29.5 us per step
-// of 8192 rows at L = 5.
+// of 8192 rows at L = 5 (21 us since a layer's columns are loops).
 cudaError_t launch_train_step(float* params, int L, int Bsz, const float* feat, const float* beta,
                               long long M, uint64_t seed, TrainCtl* ctl, int step, int steps,
                               const float* st, float* part, float* grad, float* loss,
