@@ -669,7 +669,9 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
   // Up to here nothing depends on the previous step, and the launch may have begun
   // beside its update; from here on everything does.  The weight image (written by
   // that update, or packed before the first step): one bulk copy, waited for before
-  // the first product.
+  // the first product.  The block barrier in front: no thread may poll a barrier word
+  // (or set s_abort) that thread 0 has not initialised yet.
+  __syncthreads();
   grid_dep_wait();
   if (tid == 0) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(c.bar_w),

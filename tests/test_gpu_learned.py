@@ -316,3 +316,26 @@ def test_learned_move_raises_beta_ess_per_sweep(mode):
     med = np.median(ess_l) / np.median(ess_p)
     p05 = np.percentile(ess_l, 5) / np.percentile(ess_p, 5)
     assert med >= 1.5 and p05 >= 5.0, (med, p05, np.median(ess_l), np.median(ess_p))
+
+
+@pytest.mark.parametrize("L,B", [(5, 1), (1, 2), (8, 129)])
+def test_gradient_of_nearly_empty_blocks(L, B):
+    """Blocks whose warps have no row but the first: they reach the wait for the
+    weight image at once, while thread 0 still sets the block's barriers up.  The
+    gradient is a fixed sequence of operations, so every call gives the same bits;
+    against the oracle with the bounds of the test above."""
+    F = P.n_features(L)
+    flat = _flat(_random_params(L, seed=L))
+    rng = np.random.default_rng(B)
+    feat = rng.normal(0, 1, (B, F)).astype(np.float32)
+    beta = rng.normal(0, 0.5, (B, L)).astype(np.float32)
+    loss, grad = fbs.proposal_loss_grad(flat, L, feat, beta)
+    want_loss, want = P.loss_and_grads(_unflat(flat, F, P.n_outputs(L)), feat.astype(np.float64),
+                                       beta.astype(np.float64), L)
+    assert loss == pytest.approx(want_loss, rel=1e-4, abs=1e-4)
+    got = _unflat(grad, F, P.n_outputs(L))
+    for k in ORDER:
+        assert np.abs(got[k] - want[k]).max() <= 2e-4 * np.abs(want[k]).max() + 1e-7, k
+    for _ in range(30):
+        again = fbs.proposal_loss_grad(flat, L, feat, beta)
+        assert again[0] == loss and np.array_equal(again[1], grad)
