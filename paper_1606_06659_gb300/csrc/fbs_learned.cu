@@ -567,8 +567,7 @@ template <class Issue>
 __device__ __forceinline__ bool tc_run(TcBlock& c, volatile int* s_abort, Issue issue) {
   fence_async_smem();
   tc_fence_before();
-  __syncthreads();
-  if (*s_abort) return false;
+  if (block_aborted(s_abort)) return false;
   if (threadIdx.x == 0) {
     tc_fence_after();
     issue();

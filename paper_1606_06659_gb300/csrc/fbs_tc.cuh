@@ -379,6 +379,14 @@ __device__ __forceinline__ void tc_begin(TcBlock& c, uint64_t* bars, uint32_t* t
   c.w_ok = mbar_wait(c.bar_w, 0, c.polls);
 }
 
+// Block barrier that tells every thread the same thing: whether a wait before it
+// gave up.  *s_abort is read in front of the barrier, where a thread that has set it
+// reads its own 1; read behind it, a thread that is late could see what a faster one
+// sets after its next wait, and the block's threads would part at the barriers.
+__device__ __forceinline__ bool block_aborted(volatile int* s_abort) {
+  return __syncthreads_or(*s_abort) != 0;
+}
+
 // Frees the block's c.cols tensor-memory columns.  After a wait that gave up (aborted) it first sets
 // kFlagTimeout in *flags and waits again, up to kTcWaitLimit polls, for the copy
 // and the MMAs still in flight, so that none of them outlives the block.
@@ -458,8 +466,7 @@ __device__ __forceinline__ bool tc_tile(TcBlock& c, const ModelConst& mc, const 
 #pragma unroll 1
   for (int layer = 0; layer < 3; ++layer) {
     tc_fence_before();
-    __syncthreads();
-    if (*s_abort) return false;
+    if (block_aborted(s_abort)) return false;
     const uint32_t d = c.tmem;
     if (tid == 0) {
       tc_fence_after();

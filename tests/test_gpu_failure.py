@@ -217,3 +217,48 @@ def test_training_wait_that_gives_up_is_reported():
     after = s.proposal_params()
     assert np.all(np.isfinite(after)) and not np.allclose(after, before)
     s.close()
+
+
+@pytest.mark.parametrize("polls", [1, 2, 8, 64])
+def test_waits_that_give_up_midway_end_the_pass_for_the_whole_block(polls):
+    """A poll bound at which some waits of a pass succeed and others give up: every
+    thread of a block must then leave the pass at the same place.  Whatever the
+    waits did, the genes of a block either all make their network moves or none,
+    a training step either counts or leaves the parameters, and both are reported."""
+    d = synthetic.make_config(1, G=1000)
+    s = fbs.Sampler(d["y"], d["X"], d["h"], d["priors"], seed=14, precision=fbs.FBS_F32)
+    t = d["truth"]
+    s.set_state(it=0, eps=t["eps"], beta=t["beta"], gam=t["gam"], phi=t["phi"])
+    s.proposal_collect(20, burnin=20, thin=1)
+    s.proposal_train(epochs=2, batch=2048, lr=2e-3, seed=14)
+    s.proposal_calibrate(20, burnin=100, min_accept=0.0)
+    before = s.proposal_stats()
+    params = s.proposal_params()
+    kinds = s.proposal_kinds()
+    net = [int((kinds[g:g + 128] == 1).sum()) for g in range(0, 1000, 128)]
+    s.proposal_wait_limit(polls)
+    tried = []
+    for _ in range(20):
+        s.run(1, burnin=1000)
+        after = s.proposal_stats()
+        tried.append(after["tried"] - before["tried"] - (before["mh_genes"] - sum(net)))
+        before = after
+    sums = {0}
+    for n in net:
+        sums |= {a + n for a in sums}
+    assert set(tried) <= sums, (tried, net)
+    try:
+        s.sync()
+        assert all(n == sum(net) for n in tried)
+    except fbs.FbsError as e:
+        assert e.code == fbs.FBS_E_CUDA and "tensor-core wait" in str(e)
+    try:
+        assert np.isfinite(s.proposal_train(epochs=1, batch=2048, lr=2e-3, seed=15))
+    except fbs.FbsError as e:
+        assert e.code == fbs.FBS_E_CUDA and "tensor-core wait" in str(e)
+    assert np.isfinite(s.proposal_params()).all() and s.proposal_params().shape == params.shape
+    s.proposal_wait_limit(1 << 24)
+    assert np.isfinite(s.proposal_train(epochs=1, batch=2048, lr=2e-3, seed=15))
+    st = s.get_state()
+    assert all(np.isfinite(st[k]).all() for k in ("eps", "beta", "gam", "phi"))
+    s.close()
