@@ -781,7 +781,7 @@ int fbs_init(fbs_handle** out, const int32_t* y, int N, int G, int gene_major, c
     d_pinv = (double*)(base + o32.pinv);
     h->stage = (char*)f.mu;
     h->stage_cap = stage_bytes(N, G, L, 4);
-    if ((e = prepare_gene_kernel_f32(mc, h->block)) != cudaSuccess)
+    if ((e = prepare_gene_kernel_f32()) != cudaSuccess)
       return bail(FBS_E_CUDA, std::string("kernel attribute: ") + cudaGetErrorString(e));
   } else {
     h->p = carve(base, h->lay, mc.trace_beta);
@@ -789,7 +789,7 @@ int fbs_init(fbs_handle** out, const int32_t* y, int N, int G, int gene_major, c
     h->stage_cap = stage_bytes(N, G, L, 8);
     y_raw = (int32_t*)h->p.q_eps;
     d_pinv = (double*)(base + h->lay.pinv);
-    if ((e = prepare_gene_kernel(N, h->block)) != cudaSuccess)
+    if ((e = prepare_gene_kernel()) != cudaSuccess)
       return bail(FBS_E_CUDA, std::string("kernel attribute: ") + cudaGetErrorString(e));
   }
 
@@ -2001,7 +2001,7 @@ int batch_tables(fbs_batch* b, int eps_block, int gb_block) {
   FBS_CUDA(cudaStreamSynchronize(b->s));
   b->gb_smem = 0;
   for (const ModelConst& mc : b->mcs) b->gb_smem = std::max(b->gb_smem, gb_smem_f32(mc, gb_block, false));
-  FBS_CUDA(prepare_batch_kernels(b->gb_smem));
+  FBS_CUDA(prepare_batch_kernels());
   b->n_eps = (int)et.size();
   b->n_gb = (int)gt.size();
   b->eps_block = eps_block;

@@ -651,8 +651,8 @@ struct GbLayout {
   int bs, ws, mom, es, mu, rows;
 };
 
-__host__ __device__ inline GbLayout gb_layout_f32(int N, int L, bool pat, bool move) {
-  GbLayout o;
+__host__ __device__ constexpr GbLayout gb_layout_f32(int N, int L, bool pat, bool move) {
+  GbLayout o{};
   o.bs = kNumPart;
   o.ws = o.bs + kMaxL;
   o.mom = o.ws + kMaxL;
@@ -662,10 +662,15 @@ __host__ __device__ inline GbLayout gb_layout_f32(int N, int L, bool pat, bool m
   return o;
 }
 
-__host__ __device__ inline size_t gb_smem_bytes_f32(int N, int L, int B, bool pat, bool move) {
+__host__ __device__ constexpr size_t gb_smem_bytes_f32(int N, int L, int B, bool pat, bool move) {
   return ((size_t)gb_layout_f32(N, L, pat, move).rows * B + 2) * sizeof(float) +
          (size_t)(B / 32) * kNumPart * sizeof(double);
 }
+
+// What the largest dataset in the largest block needs (the kernels' limits).
+constexpr size_t kGbMostSmem = gb_smem_bytes_f32(kMaxN, kMaxL, 128, false, false);
+constexpr size_t kGbMoveMostSmem = gb_smem_bytes_f32(kMaxN, kMaxL, 128, false, true);
+static_assert(kGbMoveMostSmem <= 227 * 1024, "a block's shared memory");
 
 // A thread's own copy of one word into its shared memory, without a register and
 // without waiting (cp_wait).
@@ -946,18 +951,21 @@ __global__ void __launch_bounds__(128) k_gb_move_f32(ModelConst mc, DevPtrsF32 p
 // arrays from offset 0, and
 // the network's outputs of the block's genes ([K][128] floats) at
 // gb_net_stash_offset, past both the weight image and those arrays.
-__host__ __device__ inline size_t gb_net_stash_offset(const ModelConst& mc) {
+__host__ __device__ inline size_t gb_net_stash_offset(int N, int L, bool pat) {
   size_t off_a;
-  tc_smem_layout(mc.L, &off_a);
-  const size_t gb = gb_smem_bytes_f32(mc.N, mc.L, 128, mc.npat <= kMaxPat, true);
+  tc_smem_layout(L, &off_a);
+  const size_t gb = gb_smem_bytes_f32(N, L, 128, pat, true);
   return ((off_a > gb ? off_a : gb) + 15) & ~(size_t)15;
 }
 
-static size_t gb_net_smem_bytes(const ModelConst& mc) {
-  const size_t tc = tc_smem_layout(mc.L, nullptr);
-  const size_t st = gb_net_stash_offset(mc) + (size_t)tc_shape(mc.L).K * 128 * sizeof(float);
+static size_t gb_net_smem_bytes(int N, int L, bool pat) {
+  const size_t tc = tc_smem_layout(L, nullptr);
+  const size_t st = gb_net_stash_offset(N, L, pat) + (size_t)tc_shape(L).K * 128 * sizeof(float);
   return tc > st ? tc : st;
 }
+
+// Every part grows with N and L, and without row patterns.
+static size_t gb_net_most_smem() { return gb_net_smem_bytes(kMaxN, kMaxL, false); }
 
 // With the learned proposal (128 threads): the block first evaluates the network
 // for its 128 genes on the tensor cores (outputs to shared memory, read by the
@@ -989,7 +997,7 @@ __global__ void __launch_bounds__(128, kBlocks) k_gb_net_f32(ModelConst mc, DevP
     if (!c.w_ok) s_abort = 1;
     __syncthreads();
     const int g = blockIdx.x * 128 + (int)threadIdx.x;
-    prop_s = reinterpret_cast<float*>(sm_tc + gb_net_stash_offset(mc));
+    prop_s = reinterpret_cast<float*>(sm_tc + gb_net_stash_offset(mc.N, mc.L, mc.npat <= kMaxPat));
     if (!s_abort)
       tc_tile(c, mc, p, nh, t, sm_tc, g, net_gene(p, g, mc.G), prop_s, 128, (int)threadIdx.x,
               &s_abort);
@@ -1131,8 +1139,7 @@ cudaError_t launch_sweeps_f32(const ModelConst& mc, const DevPtrsF32& p, const D
   const int block = 128;
   const int nblk = (mc.G + block - 1) / block;
   const size_t smem = gb_smem_f32(mc, block, false);
-  cudaError_t e = cudaFuncSetAttribute(k_sweeps_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)gb_smem_bytes_f32(FBS_MAX_N, FBS_MAX_L, block, false, false));
+  cudaError_t e = set_smem_limit(k_sweeps_f32, kGbMostSmem);
   if (e != cudaSuccess) return e;
   int dev = 0, sms = 0, per_sm = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1266,12 +1273,7 @@ __global__ void k_set_run_batch(const DevPtrsF32* __restrict__ ps, int C, long l
   }
 }
 
-cudaError_t prepare_batch_kernels(size_t smem) {
-  if (smem > 48 * 1024)
-    return cudaFuncSetAttribute(k_gb_f32_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem);
-  return cudaSuccess;
-}
+cudaError_t prepare_batch_kernels() { return set_smem_limit(k_gb_f32_batch, kGbMostSmem); }
 
 cudaError_t launch_eps_f32_batch(const ModelConst* mcs, const DevPtrsF32* ps, const int4* tab,
                                  int n_blocks, int block, int seg_i, cudaStream_t s) {
@@ -1364,14 +1366,9 @@ size_t gb_smem_f32(const ModelConst& mc, int block, bool move) {
   return gb_smem_bytes_f32(mc.N, mc.L, block, mc.npat <= kMaxPat, move);
 }
 
-cudaError_t prepare_gene_kernel_f32(const ModelConst& mc, int block) {
-  const size_t smem = gb_smem_f32(mc, block, true);  // with the learned move or without
-  if (smem <= 48 * 1024) return cudaSuccess;
-  cudaError_t e = cudaFuncSetAttribute(k_gb_f32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(k_gb_move_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  return e;
+cudaError_t prepare_gene_kernel_f32() {
+  cudaError_t e = set_smem_limit(k_gb_f32, kGbMostSmem);
+  return e == cudaSuccess ? set_smem_limit(k_gb_move_f32, kGbMoveMostSmem) : e;
 }
 
 cudaError_t launch_eps_f32(const ModelConst& mc, const DevPtrsF32& p, int seg_i,
@@ -1391,9 +1388,9 @@ cudaError_t launch_gb_f32(const ModelConst& mc, const DevPtrsF32& p, int block, 
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    const size_t smem = gb_net_smem_bytes(mc);
+    const size_t smem = gb_net_smem_bytes(mc.N, mc.L, mc.npat <= kMaxPat);
     const auto kernel = nblk <= 3 * sms ? k_gb_net_f32<3> : k_gb_net_f32<4>;
-    e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = set_smem_limit(kernel, gb_net_most_smem());
     if (e != cudaSuccess) return e;
     kernel<<<nblk, block, smem, s>>>(mc, p, seg_i, (const uint8_t*)img);
     return cudaGetLastError();

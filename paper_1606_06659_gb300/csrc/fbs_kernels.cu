@@ -1093,17 +1093,13 @@ cudaError_t launch_hyper(const ModelConst& mc, const DevPtrs& p, int nblk, cudaS
   return cudaGetLastError();
 }
 
-size_t gb_smem_bytes_f64(int N, int block) {
+constexpr size_t gb_smem_bytes_f64(int N, int block) {
   return ((size_t)N + kMaxL + kNumPart) * block * sizeof(double) +
          (size_t)(block / 32) * kNumPart * sizeof(double);
 }
 
-cudaError_t prepare_gene_kernel(int N, int block) {
-  const size_t smem_gb = gb_smem_bytes_f64(N, block);
-  if (smem_gb > 48 * 1024)
-    return cudaFuncSetAttribute(k_gb_f64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)smem_gb);
-  return cudaSuccess;
+cudaError_t prepare_gene_kernel() {
+  return set_smem_limit(k_gb_f64, gb_smem_bytes_f64(kMaxN, 128));
 }
 
 cudaError_t launch_eps_f64(const ModelConst& mc, const DevPtrs& p, int seg_i, cudaStream_t s) {

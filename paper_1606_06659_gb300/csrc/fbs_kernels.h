@@ -12,6 +12,14 @@ namespace fbs {
 
 constexpr int kDefaultBlock = 128;
 
+// The limit of a kernel's dynamic shared memory belongs to the function, for every
+// handle and host thread: `most` is what the largest call that is accepted needs,
+// never a call's own size, so that no call can lower it under another.
+template <class Kernel>
+cudaError_t set_smem_limit(Kernel* kernel, size_t most) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
+}
+
 // Puts the samples 0..N-1 whose run(n) is 0..runs-1 in the order of their runs:
 // their numbers, and the marks kRunFirst, kRunLast and run << kRunShift.  Returns
 // how many there are.
@@ -33,7 +41,7 @@ inline int order_runs(int N, int runs, Run run, uint8_t* order, uint8_t* info) {
   return k;
 }
 
-cudaError_t prepare_gene_kernel(int N, int block);
+cudaError_t prepare_gene_kernel();
 // Steps 1, 2 and 5 in one launch, the rates kept on chip; partial sums per 128 genes.
 cudaError_t launch_sweep_f64(const ModelConst& mc, const DevPtrs& p, cudaStream_t s);
 cudaError_t launch_hyper(const ModelConst& mc, const DevPtrs& p, int nblk, cudaStream_t s);
@@ -53,7 +61,7 @@ cudaError_t launch_init_run(Hyper* hy, long long trace_cap, cudaStream_t s);
 // FP32 form (fbs_gene_f32.cu)
 // Shared memory of the gamma/beta kernel for one dataset's layout.
 size_t gb_smem_f32(const ModelConst& mc, int block, bool move);
-cudaError_t prepare_gene_kernel_f32(const ModelConst& mc, int block);
+cudaError_t prepare_gene_kernel_f32();
 cudaError_t launch_eps_f32(const ModelConst& mc, const DevPtrsF32& p, int seg_i, cudaStream_t s);
 // img: null, or the learned proposal's weight image, whose network the kernel
 // then evaluates for its own genes first (block must be 128)
@@ -155,7 +163,7 @@ size_t tc_image_bytes(int L);
 cudaError_t launch_pack_image(const float* params, void* img, int L, cudaStream_t s);
 
 // batched FP32 kernels (fbs_gene_f32.cu)
-cudaError_t prepare_batch_kernels(size_t gb_smem);
+cudaError_t prepare_batch_kernels();
 cudaError_t launch_eps_f32_batch(const ModelConst* mcs, const DevPtrsF32* ps, const int4* tab,
                                  int n_blocks, int block, int seg_i, cudaStream_t s);
 cudaError_t launch_gb_f32_batch(const ModelConst* mcs, const DevPtrsF32* ps, const int2* tab,
