@@ -1313,7 +1313,7 @@ int train_bufs_alloc(TrainBufs& t, int L, int B) {
   const int F = 4 * L + 1, np = mlp_param_count(L);
   memset(&t, 0, sizeof(t));
   const size_t n = (size_t)B * (F + L) + (size_t)train_blocks(B) * (np + 1) + np + 2;
-  FBS_CUDA(prepare_train_kernel(L));
+  FBS_CUDA(prepare_train_kernel());
   float* base = nullptr;
   FBS_CUDA(cudaMalloc((void**)&base, n * sizeof(float)));
   float* q = base;

@@ -155,7 +155,7 @@ cudaError_t launch_fold(float* params, const float* st, int L, int to_raw, cudaS
 // [train_blocks(Bsz)][np + 1]); flags and polls as for launch_train_step
 size_t train_smem_bytes(int L);
 int train_blocks(int Bsz);
-cudaError_t prepare_train_kernel(int L);
+cudaError_t prepare_train_kernel();
 cudaError_t launch_mlp_grad(const float* params, int L, int Bsz, const float* fb, const float* yb,
                             float* part, float* grad, float* loss, void* img, unsigned* flags,
                             unsigned polls, cudaStream_t s);

@@ -913,8 +913,7 @@ cudaError_t launch_proposal_f32(const ModelConst& mc, const DevPtrsF32& p, const
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   const size_t smem = tc_smem_layout(mc.L, nullptr);
-  e = cudaFuncSetAttribute(k_proposal_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)tc_smem_layout(FBS_MAX_L, nullptr));
+  e = set_smem_limit(k_proposal_tc, tc_smem_layout(kMaxL, nullptr));
   if (e != cudaSuccess) return e;
   // Up to four blocks per SM: 128 of the SM's 512 TMEM columns each.
   const int ntiles = (mc.G + 127) / 128;
@@ -951,10 +950,7 @@ size_t train_smem_bytes(int L) { return (size_t)train_tc_shape(L).bytes; }
 
 int train_blocks(int Bsz) { return (Bsz + 127) / 128; }
 
-cudaError_t prepare_train_kernel(int L) {
-  return cudaFuncSetAttribute(k_mlp_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)train_smem_bytes(L));
-}
+cudaError_t prepare_train_kernel() { return set_smem_limit(k_mlp_tc, train_smem_bytes(kMaxL)); }
 
 size_t train_image_bytes(int L) { return (size_t)train_tc_shape(L).img_bytes; }
 

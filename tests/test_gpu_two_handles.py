@@ -122,3 +122,41 @@ def test_network_kernels_of_two_threads():
     _two_threads([(lambda: work(a), 100), (lambda: work(b), 100)])
     a.close()
     b.close()
+
+
+def _collected(X, seed):
+    L = X.shape[1]
+    d = synthetic.simulate(X, (3.0,) + (0.0,) * (L - 1), (1.5,) + (0.3,) * (L - 1), 0.1, 3.0, 300,
+                           seed=L)
+    s = fbs.Sampler(d["y"], X, d["h"], synthetic.default_priors(L), seed=seed,
+                    precision=fbs.FBS_F32)
+    s.run(20, burnin=1000)
+    s.proposal_collect(10, burnin=1000)
+    return s
+
+
+@pytest.mark.parametrize("other", ["train", "gradient"])
+def test_training_of_fewer_columns_between_two_training_calls(other):
+    """A handle keeps its training buffers; the kernel's limit for its L = 5 must
+    outlast another handle's training, or a gradient call, at L = 2."""
+    def train(s):
+        return s.proposal_train(epochs=2, batch=512, lr=1e-3, seed=3)
+
+    X = synthetic.paper_design(4)
+    s = _collected(X, 7)
+    want = train(s), train(s), s.proposal_params()
+    s.close()
+    s = _collected(X, 7)
+    first = train(s)
+    if other == "train":
+        t = _collected(synthetic.two_group_design(8), 8)
+        train(t)
+        t.close()
+    else:
+        rng = np.random.default_rng(2)
+        fbs.proposal_loss_grad((0.1 * rng.normal(size=fbs.proposal_param_count(2)))
+                               .astype(np.float32), 2, rng.normal(size=(40, 9)),
+                               rng.normal(size=(40, 2)))
+    assert (first, train(s)) == want[:2]
+    assert np.array_equal(s.proposal_params(), want[2])
+    s.close()
