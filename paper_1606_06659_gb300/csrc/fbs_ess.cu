@@ -104,6 +104,8 @@ constexpr int kEssPart = 8;    // lags per thread: 3 x 8 64-bit sums and a windo
 constexpr int kEssPad = 72;    // zero rows behind the series (a window reads up to 64 past the end)
 constexpr int kEssMaxRows = 8000;  // 2^50 rows < 2^63, and shared memory holds 9000
 
+constexpr int kEssFourRows = 1295;  // most rows at which four blocks of 4 series fit an SM
+
 struct Wide {  // a 128-bit integer sum
   long long hi;
   unsigned long long lo;
@@ -114,6 +116,12 @@ __host__ __device__ constexpr size_t ess_smem_bytes(long long rows, int spb) {
          (size_t)(kEssWarps / 2) * kEssLags * spb * sizeof(Wide) + (size_t)kEssLags * spb * 8 +
          2 * (size_t)spb * 8 + (size_t)spb * 4 + 16;
 }
+
+// an SM's shared memory, 1 KB per block its own
+static_assert(kEssBlocks * (ess_smem_bytes(kEssFourRows, 4) + 1024) <= 228 * 1024 &&
+                  kEssBlocks * (ess_smem_bytes(kEssFourRows + 1, 4) + 1024) > 228 * 1024,
+              "four blocks of 4 series");
+static_assert(ess_smem_bytes(kEssMaxRows, 2) <= 227 * 1024, "a block of 2 series");
 
 // SPB (4 or 2) series per block.  The block keeps its series in shared memory (one
 // read of the trace; row stride SPB + 1, so that threads on different rows hit
@@ -333,15 +341,14 @@ __global__ void __launch_bounds__(kEssThreads, kEssBlocks)
   }
 }
 
+// most: the most rows that come here with SPB series per block
 template <int SPB>
-cudaError_t launch_block(const double* tr, int rows, long long S, int L, int G,
+cudaError_t launch_block(const double* tr, int rows, int most, long long S, int L, int G,
                          const double* mean, double* ess, cudaStream_t s) {
-  const size_t smem = ess_smem_bytes(rows, SPB);
-  cudaError_t e = cudaFuncSetAttribute(k_ess_block<SPB>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = set_smem_limit(k_ess_block<SPB>, ess_smem_bytes(most, SPB));
   if (e != cudaSuccess) return e;
-  k_ess_block<SPB><<<(unsigned)((S + SPB - 1) / SPB), kEssThreads, smem, s>>>(tr, rows, S, L, G,
-                                                                             mean, ess);
+  k_ess_block<SPB><<<(unsigned)((S + SPB - 1) / SPB), kEssThreads, ess_smem_bytes(rows, SPB), s>>>(
+      tr, rows, S, L, G, mean, ess);
   return cudaGetLastError();
 }
 
@@ -363,10 +370,9 @@ cudaError_t launch_ess(const double* tr, long long rows, int L, int G, double* m
   k_ess_mean<<<(unsigned)((S + 63) / 64), 64, 0, s>>>(tr, rows, S, mean);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  // an SM's shared memory, 1 KB per block its own
-  if (kEssBlocks * (ess_smem_bytes(rows, 4) + 1024) <= 228 * 1024)
-    return launch_block<4>(tr, (int)rows, S, L, G, mean, ess, s);
-  return launch_block<2>(tr, (int)rows, S, L, G, mean, ess, s);
+  if (rows <= kEssFourRows)
+    return launch_block<4>(tr, (int)rows, kEssFourRows, S, L, G, mean, ess, s);
+  return launch_block<2>(tr, (int)rows, kEssMaxRows, S, L, G, mean, ess, s);
 }
 
 }  // namespace fbs

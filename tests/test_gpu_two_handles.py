@@ -90,8 +90,8 @@ def test_a_smaller_batch_leaves_a_larger_one_running():
             assert np.array_equal(x[k], y[k]), k
 
 
-def _two_threads(work):
-    """work[i] run over and over by a thread each; the first error of either."""
+def _threads(work):
+    """work[i] run over and over by a thread each; the first error of any."""
     errors = []
 
     def loop(f, n):
@@ -110,7 +110,7 @@ def _two_threads(work):
         raise errors[0]
 
 
-def test_network_kernels_of_two_threads():
+def test_network_kernels_of_threads():
     a, b = (_sampler(_data(N), "net") for N in (40, 22))
     for s in (a, b):
         s.proposal_calibrate(4, burnin=10 ** 6, min_accept=0.0)
@@ -119,7 +119,7 @@ def test_network_kernels_of_two_threads():
         s.run(20, burnin=10 ** 6)
         s.sync()
 
-    _two_threads([(lambda: work(a), 100), (lambda: work(b), 100)])
+    _threads([(lambda: work(a), 100), (lambda: work(b), 100)])
     a.close()
     b.close()
 
@@ -160,3 +160,23 @@ def test_training_of_fewer_columns_between_two_training_calls(other):
     assert (first, train(s)) == want[:2]
     assert np.array_equal(s.proposal_params(), want[2])
     s.close()
+
+
+@pytest.mark.parametrize("rows", [(1290, 8), (4000, 1300)])  # four and two series per block
+def test_ess_of_traces_of_different_lengths_in_several_threads(rows):
+    """One long trace beside six short ones, whose calls come between its own."""
+    chains = []
+    for i, n in enumerate((rows[0],) + 6 * (rows[1],)):
+        d = synthetic.make_config(0, G=2, seed=i)
+        s = fbs.Sampler(d["y"], d["X"], d["h"], d["priors"], seed=n, precision=fbs.FBS_F32,
+                        trace_cap=n, trace_beta=1)
+        s.run(n + 20, burnin=20, thin=1)
+        s.sync()
+        chains.append((s, s.beta_ess()))
+
+    def work(s, want):
+        assert np.array_equal(s.beta_ess(), want)
+
+    _threads([(lambda c=c: work(*c), 3000) for c in chains])
+    for s, _ in chains:
+        s.close()
