@@ -5,13 +5,13 @@
 // the lags k = 0, 1, .. up to the first pair of lags whose sum is not positive.
 // In FP64 that is one fused multiply-add per (t, k) at best, 1/64 of the FP32
 // rate here, so the sums are made in integers: a is rounded to a fixed-point
-// number of 50 bits below the power of two above max |a| (the rounding is at
-// most 2^-51 of that power, against the 2^-53 |partial sum| which every FP64
-// addition of the sum makes), split into a signed high part and a 26-bit low
-// part, and the partial products are accumulated exactly in 64 bits: high x high,
-// low x low and (high + low) x (high + low) (Karatsuba: the third less
-// the first two is the sum of the cross products).  The sums being exact, any split
-// over threads gives the same result.
+// number of 55 bits below the power of two above max |a| (two bits more than the
+// largest values have; the rounding, at most 2^-55 max |a|, is what a series with
+// outliers loses in its small values), split into a signed high part and a 28-bit
+// low part, and the partial products are accumulated exactly in 64 bits: high x high,
+// low x low and (high + low) x (high + low) modulo 2^64 (Karatsuba: the third
+// less the first two is the sum of the cross products).  The sums being exact, any
+// split over threads gives the same result.
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
@@ -102,7 +102,8 @@ constexpr int kEssBlocks = 4;  // per SM, where their shared memory fits
 constexpr int kEssLags = 16;   // lags per round while all series of a block go on
 constexpr int kEssPart = 8;    // lags per thread: 3 x 8 64-bit sums and a window of 8 values
 constexpr int kEssPad = 72;    // zero rows behind the series (a window reads up to 64 past the end)
-constexpr int kEssMaxRows = 8000;  // 2^50 rows < 2^63, and shared memory holds 9000
+constexpr int kEssMaxRows = 8000;  // shared memory holds 9000
+constexpr int kEssBits = 55, kEssLow = 28;  // of a fixed-point value, of its low part
 
 constexpr int kEssFourRows = 1295;  // most rows at which four blocks of 4 series fit an SM
 
@@ -122,6 +123,18 @@ static_assert(kEssBlocks * (ess_smem_bytes(kEssFourRows, 4) + 1024) <= 228 * 102
                   kEssBlocks * (ess_smem_bytes(kEssFourRows + 1, 4) + 1024) > 228 * 1024,
               "four blocks of 4 series");
 static_assert(ess_smem_bytes(kEssMaxRows, 2) <= 227 * 1024, "a block of 2 series");
+
+// Rows that one thread sums at most, of m rows with SPB series per block (odd, so
+// that threads on different rows hit different banks).
+__host__ __device__ constexpr int ess_thread_rows(int m, int spb) {
+  return ((m + kEssThreads / (2 * spb) - 1) / (kEssThreads / (2 * spb))) | 1;
+}
+
+// A thread's sums must fit 63 bits (its warp and block add them in 128): with high and
+// low parts up to 2^27, of products up to 2^54, and of 2^55 for the cross products.
+static_assert(kEssBits - kEssLow == 27 && kEssLow - 1 == 27, "parts up to 2^27");
+static_assert(2ll * ess_thread_rows(kEssMaxRows, 2) < 1ll << (63 - 54), "sums of 63 bits");
+static_assert(2ll * ess_thread_rows(kEssFourRows, 4) < 1ll << (63 - 54), "sums of 63 bits");
 
 // SPB (4 or 2) series per block.  The block keeps its series in shared memory (one
 // read of the trace; row stride SPB + 1, so that threads on different rows hit
@@ -196,7 +209,7 @@ __global__ void __launch_bounds__(kEssThreads, kEssBlocks)
       // a constant series (every residual zero) has ess = rows; a range of values
       // that fixed point or its squares do not hold is left to ess_series
       act = mine && b > 0x1p-400 && b < 0x1p400;
-      scale[lane] = act ? scalbn(1.0, 49 - ilogb(b)) : 0.0;
+      scale[lane] = act ? scalbn(1.0, kEssBits - 1 - ilogb(b)) : 0.0;
       if (mine && !act)
         ess[ess_slot(s_mine, L, G)] = b == 0.0 ? (double)rows : ess_series(tr, rows, S, s_mine);
     }
@@ -206,12 +219,12 @@ __global__ void __launch_bounds__(kEssThreads, kEssBlocks)
   __syncthreads();
   int n_act = *n_list;
 
-  // fixed point: |a| 2^(49 - e) <= 2^50 with 2^e <= max |a|
+  // fixed point: |a| 2^(kEssBits - 1 - e) <= 2^kEssBits with 2^e <= max |a|
   for (int i = tid; i < rows * SPB; i += kEssThreads) {
     const int at = i / SPB * ST + i % SPB;
     const long long v = __double2ll_rn(Ad[at] * scale[i % SPB]);
-    const int hi = (int)((v + (1ll << 25)) >> 26);
-    A[at] = make_int2(hi, (int)(v - ((long long)hi << 26)));
+    const int hi = (int)((v + (1ll << (kEssLow - 1))) >> kEssLow);
+    A[at] = make_int2(hi, (int)(v - ((long long)hi << kEssLow)));
   }
   __syncthreads();
 
@@ -222,14 +235,17 @@ __global__ void __launch_bounds__(kEssThreads, kEssBlocks)
     const int lw = 32 - __clz(n_act - 1);  // log2 of the list's length, rounded up
     lags = kEssLags << (LW - lw);
     const int q = tid & ((1 << lw) - 1), part = (tid & (2 * SPB - 1)) >> lw;
-    constexpr int nseg = kEssThreads / (2 * SPB);
     const int seg = tid / (2 * SPB);
     const int m = rows - k0;  // terms of lag k0 (the rows past the end are zero)
-    const int per = ((m + nseg - 1) / nseg) | 1;  // odd: threads on different banks
+    const int per = ess_thread_rows(m, SPB);
     const int t0 = seg * per, t1 = min(m, t0 + per);
-    long long hh[kEssPart], ss[kEssPart], ll[kEssPart];
+    long long hh[kEssPart], ll[kEssPart];
+    unsigned long long ss[kEssPart];
 #pragma unroll
-    for (int j = 0; j < kEssPart; ++j) hh[j] = ss[j] = ll[j] = 0;
+    for (int j = 0; j < kEssPart; ++j) {
+      hh[j] = ll[j] = 0;
+      ss[j] = 0;
+    }
     if (q < n_act && t0 < t1) {
       const int2* a = A + list[q] + t0 * ST;
       const int2* b = a + (k0 + part * kEssPart) * ST;
@@ -248,7 +264,7 @@ __global__ void __launch_bounds__(kEssThreads, kEssBlocks)
           const int2 v = w[(i + j) % kEssPart];
           hh[j] += (long long)x.x * v.x;
           ll[j] += (long long)x.y * v.y;
-          ss[j] += (long long)xs * ws[(i + j) % kEssPart];
+          ss[j] += (unsigned long long)((long long)xs * ws[(i + j) % kEssPart]);
         }
         w[i] = b[(i + kEssPart) * ST];
         ws[i] = w[i].x + w[i].y;
@@ -264,14 +280,18 @@ __global__ void __launch_bounds__(kEssThreads, kEssBlocks)
         row(i);
       }
     }
+    __int128 sums[kEssPart];
 #pragma unroll
-    for (int o = 2 * SPB; o < 32; o <<= 1) {
+    for (int j = 0; j < kEssPart; ++j) {
+      const long long cross = (long long)(ss[j] - (unsigned long long)hh[j] - (unsigned long long)ll[j]);
+      __int128 v = ((__int128)hh[j] << (2 * kEssLow)) + ((__int128)cross << kEssLow) + ll[j];
 #pragma unroll
-      for (int j = 0; j < kEssPart; ++j) {
-        hh[j] += __shfl_xor_sync(0xffffffffu, hh[j], o);
-        ss[j] += __shfl_xor_sync(0xffffffffu, ss[j], o);
-        ll[j] += __shfl_xor_sync(0xffffffffu, ll[j], o);
+      for (int o = 2 * SPB; o < 32; o <<= 1) {
+        const unsigned long long lo = __shfl_xor_sync(0xffffffffu, (unsigned long long)v, o);
+        const long long hi = __shfl_xor_sync(0xffffffffu, (long long)(v >> 64), o);
+        v += (__int128)(((unsigned __int128)(unsigned long long)hi << 64) | lo);
       }
+      sums[j] = v;
     }
     // the warps' sums, [lag][series of the list]: the upper half of the warps first,
     // the lower half adds its own
@@ -282,7 +302,7 @@ __global__ void __launch_bounds__(kEssThreads, kEssBlocks)
       if (writes && (warp >= kEssWarps / 2) == (step == 0)) {
 #pragma unroll
         for (int j = 0; j < kEssPart; ++j) {
-          __int128 v = ((__int128)hh[j] << 52) + ((__int128)(ss[j] - hh[j] - ll[j]) << 26) + ll[j];
+          __int128 v = sums[j];
           if (step == 1) v += ((__int128)slot[j << lw].hi << 64) + slot[j << lw].lo;
           slot[j << lw] = Wide{(long long)(v >> 64), (unsigned long long)v};
         }
