@@ -267,9 +267,19 @@ __device__ __forceinline__ double eps_moment_weight(const Hyper* hy, long long i
   return 1.0 / (double)(hy->seg_nmom + before + 1);
 }
 
+// s + x^2 with one rounding, or (kRounded) with that of x^2 too.  The sweep on
+// caller-owned arrays rounds the squares of the eps and the other forms do not, each
+// as it always has: which of them the compiler fuses must not change with the code
+// around them.
+template <bool kRounded>
+__device__ __forceinline__ double add_square(double s, double x) {
+  return kRounded ? __dadd_rn(__dmul_rn(x, x), s) : __fma_rn(x, x, s);
+}
+
 // Step 1 for one eps_gn: the update, the width, the moments and the rate at the
 // new value (returned in aux).  hg = 1/(2 gamma_g) and inv_k (the weight of the
 // draw in the moments) are the same for many elements and come from the caller.
+template <bool kRounded = false>
 __device__ __forceinline__ SliceResult eps_update_f64(const ModelConst& mc, const DevPtrs& p, int n,
                                                       int g, double hg, float hgf, long long it,
                                                       double inv_k) {
@@ -306,7 +316,7 @@ __device__ __forceinline__ SliceResult eps_update_f64(const ModelConst& mc, cons
   } else if (mc.moments_eps) {
     const double m = p.m_eps[e], q = p.q_eps[e];
     p.m_eps[e] = m + (s.x - m) * inv_k;
-    p.q_eps[e] = q + (s.x * s.x - q) * inv_k;
+    p.q_eps[e] = q + add_square<kRounded>(-q, s.x) * inv_k;
   }
   return s;
 }
@@ -504,6 +514,7 @@ __device__ __forceinline__ GbF64 gb_begin_f64(const ModelConst& mc, const DevPtr
 // the sums for steps 3, 4, 6, 7): the gamma_g draw and its moments.  It and the beta
 // updates need the sweep's eps and the hyperparameters but not each other, so they
 // may run on different warps.
+template <bool kRounded = false>
 __device__ __forceinline__ void gb_gamma_f64(const ModelConst& mc, const DevPtrs& p, int g, int B,
                                              int tid, double* ps, GbF64& c) {
   const int G = mc.G, N = mc.N;
@@ -512,8 +523,7 @@ __device__ __forceinline__ void gb_gamma_f64(const ModelConst& mc, const DevPtrs
   double ss = 0.0;
 #pragma unroll 8
   for (int n = 0; n < N; ++n) {
-    const double x = p.eps[(size_t)n * G + g];
-    ss += x * x;
+    ss = add_square<kRounded>(ss, p.eps[(size_t)n * G + g]);
   }
   // ---- step 2: gamma_g ~ IG((N + nu)/2, (sum eps^2 + nu tau)/2), exactly or
   // (all_slice) by a slice update of that density with the gene's own width
@@ -732,7 +742,8 @@ __global__ void __cluster_dims__(kSweepCluster, 1, 1) __launch_bounds__(32 * kSw
   unsigned evals_e = 0;
   if (g < G) {
     for (int n = warp; n < N; n += kSweepWarps) {
-      const SliceResult s = eps_update_f64(mc, p, n, g, s_hg[lane], s_hgf[lane], c.it, s_inv_k);
+      const SliceResult s =
+          eps_update_f64<true>(mc, p, n, g, s_hg[lane], s_hgf[lane], c.it, s_inv_k);
       evals_e += s.evals;
       c.caps += s.capped;
       c.nonfin += s.nonfinite;
@@ -743,7 +754,7 @@ __global__ void __cluster_dims__(kSweepCluster, 1, 1) __launch_bounds__(32 * kSw
   c.inv_k = u.inv_k;
   if (g < G) {
     if (warp == 0) gb_beta_f64(mc, p, g, 32, lane, mu, bs, ps, u, c);
-    else if (warp == 1) gb_gamma_f64(mc, p, g, 32, lane, ps, c);
+    else if (warp == 1) gb_gamma_f64<true>(mc, p, g, 32, lane, ps, c);
   }
   __syncthreads();
   if (warp == 0) warp_sums(ps, lane, [&](int i, double x) { s_sum[i] = x; });

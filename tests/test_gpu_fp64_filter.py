@@ -107,3 +107,34 @@ def test_noalloc_equals_run(kind, N, G):
         assert close(arr["q_" + k].cpu().numpy().T, m["msq_" + k], RTOL, ATOL).all(), k
     assert close(arr["hyp"].cpu().numpy()[: 2 * L + 2], got["phi"], RTOL, ATOL).all()
     s.close()
+
+
+def test_noalloc_rounds_the_squares_of_eps():
+    """The second moments of eps fold in the square rounded to FP64: with one draw
+    before it the weight of the next is 1/2, so that everything else is exact but
+    the subtraction and the final sum."""
+    import torch
+    d = _data("two", 9, 1501)
+    L, (G, N) = 2, d["y"].shape
+    s = fbs.Sampler(d["y"], d["X"], d["h"], d["priors"], seed=8)
+    st = s.get_state()
+    s.close()
+
+    def dev(a):
+        return torch.from_numpy(np.ascontiguousarray(np.asarray(a).T)).cuda()
+
+    arr = {k: dev(st[k]) for k in ("eps", "w_eps", "waux_eps", "beta", "w_beta", "waux_beta", "gam")}
+    arr["y"] = dev(d["y"].astype(np.int32))
+    arr["T"] = dev(d["y"].astype(np.float64) @ d["X"])
+    arr["hyp"] = dev(np.concatenate([st["phi"], st["w_nu"], st["waux_nu"]]))
+    for k, shape in (("eps", (N, G)), ("beta", (L, G)), ("gam", (G,)), ("phi", (2 * L + 2,))):
+        arr["m_" + k] = torch.zeros(shape, dtype=torch.float64, device="cuda")
+        arr["q_" + k] = torch.zeros(shape, dtype=torch.float64, device="cuda")
+    q = np.zeros((N, G))
+    for it in range(1, 3):
+        fbs.sweep_noalloc(d["X"], d["h"], d["priors"], seed=8, it=it, burnin=0, n_mom=it - 1,
+                          stream=torch.cuda.current_stream().cuda_stream, G=G,
+                          **{k: v.data_ptr() for k, v in arr.items()})
+        x = arr["eps"].cpu().numpy()
+        q = q + (x * x - q) / it
+        assert np.array_equal(arr["q_eps"].cpu().numpy(), q), it
