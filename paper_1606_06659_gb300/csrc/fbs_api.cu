@@ -146,7 +146,7 @@ void fbs::set_last_error(const std::string& msg) { g_err = msg; }
 
 // Scratch of one training step for batch size B; flags: the tensor-core wait
 // flag word of the step's kernels; img: the training kernel's weight image; stat:
-// scratch of the column statistics.
+// scratch of the column statistics (training calls only).
 struct TrainBufs {
   float *fb, *yb, *part, *grad, *loss;
   unsigned* flags;
@@ -1309,7 +1309,7 @@ int mlp_step(const float* params, int L, int B, TrainBufs& t, cudaStream_t s) {
   return FBS_OK;
 }
 
-int train_bufs_alloc(TrainBufs& t, int L, int B) {
+int train_bufs_alloc(TrainBufs& t, int L, int B, bool stats) {
   const int F = 4 * L + 1, np = mlp_param_count(L);
   memset(&t, 0, sizeof(t));
   const size_t n = (size_t)B * (F + L) + (size_t)train_blocks(B) * (np + 1) + np + 2;
@@ -1327,7 +1327,7 @@ int train_bufs_alloc(TrainBufs& t, int L, int B) {
   cudaError_t e = cudaMemset(t.flags, 0, sizeof(unsigned));
   if (e == cudaSuccess) e = cudaMalloc(&t.img, train_image_bytes(L));
   if (e == cudaSuccess) e = cudaMemset(t.img, 0, train_image_bytes(L));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&t.stat, col_stats_bytes(L));
+  if (e == cudaSuccess && stats) e = cudaMalloc((void**)&t.stat, col_stats_bytes(L));
   if (e != cudaSuccess) train_bufs_free(t);
   FBS_CUDA(e);
   return FBS_OK;
@@ -1396,7 +1396,7 @@ int fbs_proposal_train(fbs_handle* h, int epochs, int batch, double lr, uint64_t
   }
   if (!ls->bufs) {
     TrainBufs fresh;
-    rc = train_bufs_alloc(fresh, ls->L, batch);
+    rc = train_bufs_alloc(fresh, ls->L, batch, true);
     if (rc) return rc;
     ls->bufs = new TrainBufs(fresh);
     ls->bufs_batch = batch;
@@ -1899,7 +1899,7 @@ int fbs_proposal_loss_grad(const float* params, int L, int B, const float* feat,
     return fail(FBS_E_ARG, "bad arguments");
   const int F = 4 * L + 1, np = mlp_param_count(L);
   TrainBufs t;
-  int rc = train_bufs_alloc(t, L, B);
+  int rc = train_bufs_alloc(t, L, B, false);
   if (rc) return rc;
   float* dp = nullptr;
   cudaError_t e = cudaMalloc((void**)&dp, sizeof(float) * np);
