@@ -138,3 +138,23 @@ def test_noalloc_rounds_the_squares_of_eps():
         x = arr["eps"].cpu().numpy()
         q = q + (x * x - q) / it
         assert np.array_equal(arr["q_eps"].cpu().numpy(), q), it
+
+
+@pytest.mark.parametrize("kind", ["three", "eight"])
+def test_lockstep_above_the_genes_of_split_blocks(kind):
+    """More genes than the blocks with gamma on a second warp hold at once: the
+    one-warp blocks, with columns of three and eight value classes."""
+    import torch
+    G = 32 * 6 * torch.cuda.get_device_properties(0).multi_processor_count + 33
+    g, o = make_pair(_data(kind, 9, G), seed=7)
+    o.init_default()
+    o.set_opts(burnin=1, tune_start=0)
+    for it in range(1, 3):
+        sync_gpu_to_oracle(g, o, it - 1)
+        c0, o0 = g.counters(), o.counters_dict()
+        g.run(1, burnin=1, thin=1)
+        o.sweep()
+        assert_state_close(g.get_state(), o.get_state(), where=f"sweep {it}")
+        c1, o1 = g.counters(), o.counters_dict()
+        for k in COUNTS:
+            assert c1[k] - c0[k] == o1[k] - o0[k], (it, k)

@@ -339,3 +339,59 @@ def test_gradient_of_nearly_empty_blocks(L, B):
     for _ in range(30):
         again = fbs.proposal_loss_grad(flat, L, feat, beta)
         assert again[0] == loss and np.array_equal(again[1], grad)
+
+
+def _random_learned(d, seed, fused, **kw):
+    """A sampler whose proposal network has random weights, calibrated."""
+    L = d["X"].shape[1]
+    s = fbs.Sampler(d["y"], d["X"], d["h"], d["priors"], seed=seed, precision=fbs.FBS_F32, **kw)
+    s.set_state(it=0, **_truth(d))
+    s.proposal_params(set_to=_flat(_random_params(L, seed=3)))
+    s.proposal_fused(fused)
+    s.proposal_calibrate(6, burnin=100, min_accept=0.0)
+    return s
+
+
+@pytest.mark.parametrize("extra", [0, 1])
+def test_fused_network_pass_equals_separate_kernel_at_many_genes(extra):
+    """As above at the number of genes up to which three blocks per SM hold them
+    all, and one gene more, where the kernel compiled for four blocks runs."""
+    import torch
+    G = 3 * 128 * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    d = synthetic.make_config(1, G=G)
+    runs = []
+    for fused in (True, False):
+        s = _random_learned(d, 73, fused, graph_segment=4)
+        s.run(7, burnin=100)
+        s.sync()
+        runs.append((s.get_state(), s.proposal_stats(), s.counters()))
+        s.close()
+    (sa, pa, ca), (sb, pb, cb) = runs
+    for k in ("eps", "beta", "gam", "phi", "w_eps", "w_beta"):
+        assert np.array_equal(sa[k], sb[k]), k
+    assert pa == pb and ca == cb and pa["tried"] > 0 and pa["accepted"] > 0
+
+
+@pytest.mark.parametrize("batch,other", [(300, 1000), (1000, 129), (129, 4000)])
+def test_training_buffers_kept_or_made_anew_give_the_same_steps(batch, other):
+    """Two training calls of one batch size on the buffers of the first, and with
+    the buffers given back and made anew in between by a call of another size,
+    whose steps all give up (a poll bound of 0): the same losses and parameters.
+    3000 pairs: 10, 3 and 24 steps per epoch, groups of eight and less."""
+    d = synthetic.make_config(1, G=300)
+
+    def calls(middle):
+        s = fbs.Sampler(d["y"], d["X"], d["h"], d["priors"], seed=6, precision=fbs.FBS_F32)
+        s.set_state(it=0, **_truth(d))
+        s.proposal_collect(10, burnin=100)
+        out = [s.proposal_train(epochs=1, batch=batch, lr=1e-3, seed=1), s.proposal_params()]
+        s.proposal_wait_limit(0)
+        with pytest.raises(fbs.FbsError):
+            s.proposal_train(epochs=1, batch=middle, lr=1e-3, seed=2)
+        s.proposal_wait_limit(1 << 24)
+        out += [s.proposal_train(epochs=2, batch=batch, lr=1e-3, seed=3), s.proposal_params()]
+        s.close()
+        return out
+
+    for a, b in zip(calls(batch), calls(other)):
+        assert np.array_equal(a, b)
