@@ -108,8 +108,6 @@ __host__ __device__ inline TcShape tc_shape(int L) {
   return t;
 }
 
-constexpr int kMaxK1 = (kMaxFeat + 15) & ~15;
-
 // Shared memory of the network pass: the weight image alone (the A operands are
 // in tensor memory); *off_a = its size rounded to 1 KB, where a caller's own
 // shared data may start.
