@@ -63,3 +63,47 @@ def test_state_moments_and_summaries_round_trip(prec, N, G, L):
         assert np.array_equal(a[k], b[k]), k
     s.close()
     t.close()
+
+
+def test_summaries_into_new_arrays_cost_what_their_pages_cost():
+    """Arrays whose pages were never touched: the call may take as long as into used
+    ones and what the host takes to touch such pages, here with a factor of two,
+    but not the several times that of pages faulted in by the copies."""
+    import ctypes
+    import mmap
+    import time
+    N, G = 32, 60000
+    d = _data(N, G, 2)
+    s = fbs.Sampler(d["y"], d["X"], d["h"], d["priors"], seed=1, precision=fbs.FBS_F32)
+    s.run(4, burnin=2)
+
+    def arrays():
+        return [np.frombuffer(mmap.mmap(-1, G * N * 8), np.float64).reshape(G, N) for _ in range(4)]
+
+    def call(out):
+        o = fbs.EstimatesOut()
+        o.z = 2.0
+        for q, a in zip(("mean", "sd", "lo", "hi"), out):
+            setattr(o, q + "_eps", a.ctypes.data_as(ctypes.POINTER(ctypes.c_double)))
+        h = (ctypes.c_void_p * 1)(s.h)
+        t = time.perf_counter()
+        assert s.lib.fbs_estimates_pooled(1, h, ctypes.byref(o)) == 0
+        return time.perf_counter() - t
+
+    def fill(out):
+        t = time.perf_counter()
+        for a in out:
+            a[:] = 1.0
+        return time.perf_counter() - t
+
+    used = arrays()
+    call(used)
+    host = min(fill(arrays()) for _ in range(5))
+    again = min(call(used) for _ in range(5))
+    times = []
+    for _ in range(5):
+        out = arrays()
+        times.append(call(out))
+        assert all(np.array_equal(a, b) for a, b in zip(out, used))
+    assert min(times) < again + 2.0 * host, (min(times), again, host)
+    s.close()
