@@ -42,11 +42,11 @@ size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 // Results of up to kPackMost bytes are read back in one copy if the staging area
 // holds them (see read_arrays); it has kPackBytes at least, and room for the four
-// summaries of every beta and gamma.
+// summaries of every beta, gamma and phi.
 constexpr size_t kPackBytes = 256 << 10, kPackMost = 1 << 20;
 
 size_t stage_bytes(int N, int G, int L, size_t word) {
-  return std::max({(size_t)N * G * word, kPackBytes, 32 * (size_t)(L + 1) * G});
+  return std::max({(size_t)N * G * word, kPackBytes, 32 * ((size_t)(L + 1) * G + 2 * L + 2)});
 }
 
 // Byte offsets of every device buffer inside one workspace.
