@@ -8,9 +8,10 @@
 //                 FP64 partial sums that feed steps 3, 4, 6, 7;
 //                 both with width tuning (Algorithm 2 step 7) and Welford moments
 //                 (Section 3.1);
-//   hyper kernel  one block: fixed-order reduction of the partials, then nu (slice,
-//                 step 3) and tau (step 4) on lane 0 while lanes 1..L draw
-//                 theta_l (step 6) and sigma_l^2 (step 7).
+//   hyper kernel  one block: fixed-order reduction of the partials beside all that
+//                 needs no sums, then nu (slice, step 3) and tau (step 4) on warp 0
+//                 while warp 1 draws theta_l (step 6) and sigma_l^2 (step 7) on
+//                 lane l (fbs_hyper.cuh).
 // Drawing beta before nu and tau is exact: the beta_gl conditional involves
 // neither, and theirs involve no beta (Figure 3); the counter-based generator
 // gives every variable the same uniforms in either order.
@@ -324,7 +325,7 @@ __device__ __forceinline__ SliceResult eps_update_f64(const ModelConst& mc, cons
 // Step 1: one thread per eps_gn, a block 32 genes and blockDim.x / 32 samples (one
 // warp each), so that 1/(2 gamma_g) and the moments' weight, an FP64 division of a
 // dozen instructions each, are taken once per block instead of by every warp.
-// Bound by the FP64 pipe (16 cycles per warp instruction; 84% busy).  N=16 G=40000
+// Bound by the FP64 pipe (16 cycles per warp instruction; 78% busy).  N=16 G=40000
 // L=5: 88 us; 258 us with the offsets taken in FP64 per evaluation, bounds that
 // grow with the counts, the divisions per thread and the level's density and log
 // in every update.
