@@ -562,12 +562,14 @@ __device__ __forceinline__ void issue_split(uint32_t d, uint32_t idesc, int kste
 
 // Block barrier, then (thread 0) the products `issue` describes and a commit;
 // every thread waits for their completion, and a second block barrier makes
-// the outcome the same for every thread: false once any wait gave up.
+// the outcome the same for every thread: false once any wait gave up.  The block
+// calls it while none has: s_abort is only written between the two barriers, and
+// only read behind the second.
 template <class Issue>
 __device__ __forceinline__ bool tc_run(TcBlock& c, volatile int* s_abort, Issue issue) {
   fence_async_smem();
   tc_fence_before();
-  if (block_aborted(s_abort)) return false;
+  __syncthreads();
   if (threadIdx.x == 0) {
     tc_fence_after();
     issue();
@@ -693,13 +695,14 @@ __global__ void __launch_bounds__(128) k_mlp_tc(
   const uint32_t sW1 = smem_u32(w1s), sW2 = smem_u32(w2s), sW3 = smem_u32(w3s);
   const uint32_t sbo_f = t.sbo_f, hb = (uint32_t)half * 128;
   const int cx = t.cx, k1 = t.k1, n3 = t.n3;
-  bool ok = true;
+  bool ok = s_abort == 0;  // the wait for the weight image
 
   // ---- forward
-  ok = tc_run(c, &s_abort, [&] {  // Z1 = X W1^T
-    issue_split(tm, umma_idesc_bf16(128, H), k1 / 16, sF + 8 * 128, sF + 8 * 128 + hb, 256, 128,
-                sbo_f, sW1, sW1 + cx * 128, 256, 128, t.sbo_w1);
-  });
+  if (ok)
+    ok = tc_run(c, &s_abort, [&] {  // Z1 = X W1^T
+      issue_split(tm, umma_idesc_bf16(128, H), k1 / 16, sF + 8 * 128, sF + 8 * 128 + hb, 256, 128,
+                  sbo_f, sW1, sW1 + cx * 128, 256, 128, t.sbo_w1);
+    });
   if (ok) {
     // Z1 becomes gelu'(Z1 + b1)
     train_hidden(tm + la, bsm, bF, sbo_f, 0, half);
